@@ -498,16 +498,19 @@ SAMPLE_KERNEL_TRAFFIC = {"source_sha256": "7861a6430fbac9e0c146a8aa2dfbd32476343
 # MINRES update (10 arrays per node) on mesh 1/1024, 16 samples of the six-level workload's finest
 # level (summarised under profiles/), scaled to a launch by its algorithmic bytes; valid only for
 # the kernel source it was measured on
-KMINRES_TRAFFIC = {"source_sha256": "22f59b77c3bc4dc0a0e79efd7d578bdcdaa1e7ff1ab891b96076f838197586da",
+KMINRES_TRAFFIC = {"source_sha256": "544ec7444614d4ab700b9665f19c3a860cc656f51459c999e0266c26273cc0c7",
                    "dram_per_algorithmic": (471.794432e6 + 170.729984e6) / (16 * 1023 * 1023 * 40)}
 
 
 def _stream_source_hash():
+    """sha256 of the operator sweep's source: the kernel and the tile sum it ends with."""
     import hashlib
 
+    src = open(os.path.join(ROOT, "paper_2103_03407_gb300", "csrc", "mq_stream.cu")).read()
     h = hashlib.sha256()
-    for f in ("mq_stream.cu", "mq_device.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2103_03407_gb300", "csrc", f), "rb").read())
+    for sig in ("__global__ void k_minres_q4(", "__device__ __forceinline__ void tile_partials("):
+        i = src.index(sig)
+        h.update(src[i:src.index("\n}\n", i)].encode())
     return h.hexdigest()
 
 

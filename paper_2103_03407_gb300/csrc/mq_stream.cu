@@ -24,9 +24,11 @@
 #include <cmath>
 #include <cstdint>
 #include <initializer_list>
+#include <type_traits>
 #include <vector>
 
 #include "mq_device.cuh"
+#include "mq_df.cuh"
 #include "mq_internal.h"
 
 namespace mq {
@@ -101,6 +103,7 @@ struct SS {  // per-sample solver scalars
   double xsum;      // sum of the nodal values of x64 in that pass (h^2 xsum = integral of x)
   float amax;     // largest centroid coefficient (for the bound ||A - sigma M|| <= 8 amax + sigma h^2)
   float bmax;     // largest reaction coefficient (the bound gains bmax h^2)
+  df cs, c12;     // lambda_H h^2 / 12 and lambda_H h^2 as double-floats (FP32 path: the residual's mass factors)
   int act_outer;  // refinement still running
   int act;        // inner MINRES running
   int pend;       // a w/x update is pending
@@ -133,32 +136,19 @@ __device__ __forceinline__ double half_pos(double v) {
   return __longlong_as_double(__double_as_longlong(v) - (1LL << 52));
 }
 
-// weights and inverse diagonal of mesh n from per-triangle coefficients (lower plane, upper plane)
-// (with hx: BF16 copies of the weights and of om D^-1 for the V(1,1) sweeps of the FP32 path)
-// (with rcells: the reaction term of the second test problem of Sec. 5 -- om D^-1 includes the
-// lumped reaction h^2/6 sum_{T at p} b_T, written in BF16 to hr for the V(1,1) sweeps; with rxo also
-// the reaction's FP32 edge weights for the operator sweep (b averaged over the two triangles of
-// the edges to E, N and NE) and the largest b into ss)
+// weights and inverse diagonal (om D^-1) of mesh n from per-triangle coefficients (lower plane, upper
+// plane): the FP64 path (the FP32 path: k_weights4)
 template <typename T, typename S>
 __global__ void k_weights(int n, int B, const S* __restrict__ cells, size_t cstride, T* __restrict__ wx,
-                          T* __restrict__ wy, T* __restrict__ dinv, T om, double* __restrict__ wx64,
-                          double* __restrict__ wy64, const int* __restrict__ act, SS<T>* ss,
-                          __nv_bfloat16* __restrict__ hx = nullptr, __nv_bfloat16* __restrict__ hy = nullptr,
-                          __nv_bfloat16* __restrict__ hd = nullptr, const S* __restrict__ rcells = nullptr,
-                          __nv_bfloat16* __restrict__ hr = nullptr, T* __restrict__ rxo = nullptr,
-                          T* __restrict__ ryo = nullptr, T* __restrict__ rdo = nullptr) {
+                          T* __restrict__ wy, T* __restrict__ dinv, T om, SS<T>* ss) {
   const int nt = tiles_padded(n);
   const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
-  if (b >= B || (act && !act[b])) return;
+  if (b >= B) return;
   const S* lo = cells + (size_t)b * cstride;
   const S* up = lo + (size_t)n * n;
   const size_t V = ssz(n);
   const int ld = sld(n);
   int bad = 0;
-  const S* rlo = rcells ? rcells + (size_t)b * cstride : nullptr;
-  const S* rup = rcells ? rlo + (size_t)n * n : nullptr;
-  const double hr6 = 1.0 / (6.0 * (double)n * (double)n);
-  long long rbits = 0;  // largest reaction coefficient (bit pattern)
   // largest coefficient as the bit pattern of a double: positive doubles order as their bit patterns
   // (the coefficient checks run on the integer units; GB300 has few FP64 units)
   long long mbits = 0;
@@ -179,52 +169,20 @@ __global__ void k_weights(int n, int B, const S* __restrict__ cells, size_t cstr
       bad |= !(bl > 0 && bl <= kInfBits) | !(bu > 0 && bu <= kInfBits);
       mbits = max(mbits, max(bl, bu));
     }
-    T dr = T(0);
-    if (rlo) {
-      auto RL = [&](int ii, int jj) { return (double)rlo[jj * n + ii]; };
-      auto RU = [&](int ii, int jj) { return (double)rup[jj * n + ii]; };
-      if (i <= n - 1 && j <= n - 1) {  // b >= 0 and not NaN
-        const long long bl = __double_as_longlong(RL(i, j)), bu = __double_as_longlong(RU(i, j));
-        bad |= !(bl >= 0 && bl <= kInfBits) | !(bu >= 0 && bu <= kInfBits);
-        rbits = max(rbits, max(bl, bu));
-      }
-      if (i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1)
-        dr = T(hr6 * (RL(i, j) + RU(i, j) + RL(i - 1, j) + RU(i, j - 1) + RL(i - 1, j - 1) + RU(i - 1, j - 1)));
-      if (rxo) {
-        rxo[(size_t)b * V + q] = (i <= n - 1 && j >= 1 && j <= n - 1) ? T(0.5 * (RL(i, j) + RU(i, j - 1))) : T(0);
-        ryo[(size_t)b * V + q] = (i >= 1 && i <= n - 1 && j <= n - 1) ? T(0.5 * (RU(i, j) + RL(i - 1, j))) : T(0);
-        rdo[(size_t)b * V + q] = (i <= n - 1 && j <= n - 1) ? T(0.5 * (RL(i, j) + RU(i, j))) : T(0);
-      }
-      if (hr) hr[(size_t)b * V + q] = __float2bfloat16_rn((float)dr);
-    }
     if (i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1) {
       // the east and north edges are this node's own (a, c); west and south are the neighbours'
       const T ww = T(half_pos(LO(i - 1, j) + UP(i - 1, j - 1))), ws = T(half_pos(UP(i, j - 1) + LO(i - 1, j - 1)));
-      d = om / (a + ww + c + ws + dr);  // the damped Jacobi factor omega D^-1 (with the lumped reaction)
+      d = om / (a + ww + c + ws);  // the damped Jacobi factor omega D^-1
     }
     wx[(size_t)b * V + q] = a;
     wy[(size_t)b * V + q] = c;
     dinv[(size_t)b * V + q] = d;
-    if (hx) {
-      hx[(size_t)b * V + q] = __float2bfloat16_rn((float)a);
-      hy[(size_t)b * V + q] = __float2bfloat16_rn((float)c);
-      hd[(size_t)b * V + q] = __float2bfloat16_rn((float)d);
-    }
-    if (wx64) {
-      wx64[(size_t)b * V + q] = a64;
-      wy64[(size_t)b * V + q] = c64;
-    }
   }
   if (ss) {
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&ss[b].flags, kFlagBadCoef);
     float amax = (mbits > 0 && mbits <= kInfBits) ? (float)__longlong_as_double(mbits) * 1.0001f : 0.0f;
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if ((threadIdx.x & 31) == 0 && amax > 0.0f) atomicMax((int*)&ss[b].amax, __float_as_int(amax));  // positive floats order as ints
-    if (rlo) {
-      float bmx = (rbits > 0 && rbits <= kInfBits) ? (float)__longlong_as_double(rbits) * 1.0001f : 0.0f;
-      for (int o = 16; o > 0; o >>= 1) bmx = fmaxf(bmx, __shfl_xor_sync(0xffffffffu, bmx, o));
-      if ((threadIdx.x & 31) == 0 && bmx > 0.0f) atomicMax((int*)&ss[b].bmax, __float_as_int(bmx));
-    }
   }
 }
 
@@ -239,16 +197,25 @@ __global__ void k_coarsen(int n, int B, const S* __restrict__ in, size_t istride
   const S* lo = in + (size_t)b * istride;
   const S* up = lo + (size_t)n * n;
   T* o = out + (size_t)b * 2 * mm;
+  // the FP32 path rounds the four values first (the coarse operators only precondition; FP64
+  // additions and conversions bound this kernel otherwise)
+  auto val = [](S v) {
+    if constexpr (sizeof(S) == sizeof(double) && sizeof(T) == sizeof(float)) {
+      const df d = df_split(v);
+      return d.h + d.l;
+    } else {
+      return T(v);
+    }
+  };
   for (int k = 0; k < kPer; ++k) {
     const size_t q = (size_t)ch * kTile + threadIdx.x + k * kThreads;
     if (q >= mm) break;
     const int I = (int)(q % m), J = (int)(q / m), i = 2 * I, j = 2 * J;
-    const double l = (double)lo[j * n + i] + (double)lo[j * n + i + 1] + (double)lo[(j + 1) * n + i + 1] +
-                     (double)up[j * n + i + 1];
-    const double u = (double)up[j * n + i] + (double)up[(j + 1) * n + i + 1] + (double)up[(j + 1) * n + i] +
-                     (double)lo[(j + 1) * n + i];
-    o[q] = T(0.25 * l);
-    o[mm + q] = T(0.25 * u);
+    const T l = (val(lo[j * n + i]) + val(lo[j * n + i + 1])) + (val(lo[(j + 1) * n + i + 1]) + val(up[j * n + i + 1]));
+    const T u = (val(up[j * n + i]) + val(up[(j + 1) * n + i + 1])) +
+                (val(up[(j + 1) * n + i]) + val(lo[(j + 1) * n + i]));
+    o[q] = T(0.25) * l;
+    o[mm + q] = T(0.25) * u;
   }
 }
 
@@ -346,6 +313,8 @@ __global__ void k_sc_start(int B, int n, const double* sigma, int sig_stride, in
   const double s = t[0];
   ss[b].sigm = T(sigma[(size_t)b * sig_stride] / (12.0 * n * n));
   SS<T>& S = ss[b];
+  S.cs = df_split(sigma[(size_t)b * sig_stride] / (12.0 * n * n));
+  S.c12 = df_split(sigma[(size_t)b * sig_stride] / ((double)n * n));
   S.bnorm = S.rnorm = sqrt(s);
   S.rs = T(1.0 / S.rnorm);
   S.act_outer = S.rnorm > 0.0;
@@ -353,6 +322,19 @@ __global__ void k_sc_start(int B, int n, const double* sigma, int sig_stride, in
   S.pend = 0;
   S.iters = 0;
   S.outer = 0;
+}
+
+// a refinement step of sample S ends with residual norm rnew and ||x|| = xn
+template <typename T>
+__device__ __forceinline__ void outer_step_done(SS<T>& S, double rnew, double xn) {
+  S.xnorm = xn;
+  // No progress: stop refining.  Not on the first step: on fine meshes the FP32 rounding of the
+  // first inner solution alone leaves an FP64 residual above ||b|| (the operator amplifies its
+  // high-frequency part by O(h^-2)); the next step removes it.
+  if (S.outer >= 1 && !(rnew < 0.5 * S.rnorm)) S.act_outer = 0;
+  S.rnorm = rnew;
+  S.rs = T(1.0 / rnew);
+  S.outer += 1;
 }
 
 // start of a refinement step: samples above tolerance run an inner solve
@@ -917,6 +899,464 @@ __global__ void k_minres_v4(int n, int B, const int* __restrict__ act, const SS<
                           a.w - c1 * bv.w - c2 * o.w));
 }
 
+// ---------------------------------------------------------------------------------------------
+// Setup and residual of the FP32 path in double-float arithmetic (mq_df.cuh).  What is kept to FP64
+// accuracy -- the edge weights of the finest mesh, the right-hand side b, the solution x -- is held
+// as pairs of FP32 arrays (the same bytes as FP64 arrays; the high parts of the weights are the
+// FP32 operator's own), and the stencils run on the FP32 units: the FP64 forms of these kernels were
+// bound by GB300's FP64 issue rate at a fifth to a tenth of the memory bandwidth.
+
+// tiles of the setup kernels: (n + 1) padded rows of n / 4 + 1 groups of four nodes
+__host__ __device__ inline int tiles_setup(int n) {
+  return (int)(((long)(n + 1) * (n / kVec + 1) + kThreads - 1) / kThreads);
+}
+
+__device__ __forceinline__ df cell_value(double v) { return df_split(v); }
+__device__ __forceinline__ df cell_value(float v) { return {v, 0.0f}; }
+
+// four coefficients of a cell row at columns c0 .. c0+3 into v[1..4], the one at c0 - 1 into v[0]
+// (zeros when the row or the column is outside); returns nothing beyond the values
+__device__ __forceinline__ void cell_row(const double* __restrict__ row, int c0, bool ok, double (&v)[5]) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) v[k] = 0.0;
+  if (!ok) return;
+  if (c0) v[0] = row[c0 - 1];
+  const double2 a = *reinterpret_cast<const double2*>(row + c0), c = *reinterpret_cast<const double2*>(row + c0 + 2);
+  v[1] = a.x, v[2] = a.y, v[3] = c.x, v[4] = c.y;
+}
+__device__ __forceinline__ void cell_row(const float* __restrict__ row, int c0, bool ok, float (&v)[5]) {
+#pragma unroll
+  for (int k = 0; k < 5; ++k) v[k] = 0.0f;
+  if (!ok) return;
+  if (c0) v[0] = row[c0 - 1];
+  const float4 a = ld4(row + c0);
+  v[1] = a.x, v[2] = a.y, v[3] = a.z, v[4] = a.w;
+}
+
+// half the sum of two coefficients: an edge weight
+__device__ __forceinline__ df half_sum(df a, df b) {
+  const df s = df_add(a, b);
+  return {0.5f * s.h, 0.5f * s.l};
+}
+
+__device__ __forceinline__ void st4h(__nv_bfloat16* p, const float (&v)[kVec]) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+  uint2 u;
+  u.x = *reinterpret_cast<const unsigned*>(&a);
+  u.y = *reinterpret_cast<const unsigned*>(&b);
+  *reinterpret_cast<uint2*>(p) = u;
+}
+__device__ __forceinline__ void st4v(float* p, const float (&v)[kVec]) { st4(p, make_float4(v[0], v[1], v[2], v[3])); }
+
+// the bit test of a coefficient: positive (nonnegative with ZERO) and not NaN; positive doubles (and
+// floats) order as their bit patterns
+template <bool ZERO>
+__device__ __forceinline__ int cell_bad(double v, unsigned long long& top) {
+  const long long b = __double_as_longlong(v);
+  const bool ok = (ZERO ? b >= 0 : b > 0) && b <= 0x7ff0000000000000LL;
+  if (ok) top = max(top, (unsigned long long)b);
+  return !ok;
+}
+template <bool ZERO>
+__device__ __forceinline__ int cell_bad(float, unsigned long long&) {
+  return 0;  // coarsened values: checked on the finest mesh
+}
+
+// Edge weights and damped inverse diagonal of mesh n from per-triangle coefficients (lower plane,
+// upper plane), as k_weights<float>: four nodes of one row per thread.  S = double: the finest mesh,
+// with the low parts of the weights in wxl, wyl (and, with the reaction, rxl, ryl, rdl), the
+// coefficient checks and the largest coefficient into ss.  S = float: a coarsened mesh.  wx, wy or
+// dinv may be NULL when nothing reads them (the V(1,1) sweeps read the BF16 copies hx, hy, hd).
+// Bound by memory: 16 B in and 30 B out per node of the finest mesh; the FP64 form executed about 14
+// FP64 instructions per node.
+struct WeightOut {
+  float *wx, *wy, *dinv, *wxl, *wyl;
+  __nv_bfloat16 *hx, *hy, *hd, *hr;
+  float *rx, *ry, *rd, *rxl, *ryl, *rdl;
+};
+template <typename S, bool RX>
+__global__ void __launch_bounds__(kThreads) k_weights4(int n, int B, const S* __restrict__ cells, size_t cstride,
+                                                       const S* __restrict__ rcells, float om, WeightOut W,
+                                                       SS<float>* ss) {
+  constexpr bool FINE = sizeof(S) == sizeof(double);
+  const int nt = tiles_setup(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  if (b >= B) return;
+  const int groups = n / kVec + 1;
+  const int g = ch * kThreads + threadIdx.x;
+  const int j = g / groups, c0 = (g % groups) * kVec;
+  unsigned long long top = 0, rtop = 0;
+  int bad = 0;
+  if (j <= n) {
+    const size_t nn = (size_t)n * n;
+    const bool in = c0 < n, up_row = in && j < n, dn_row = in && j >= 1;
+    // edge weights: E edge of node (i, j) from LO(i, j), UP(i, j-1); N edge from UP(i, j), LO(i-1, j)
+    auto edges = [&](const S* __restrict__ lo, df (&e)[5], df (&no)[kVec], float (&so)[kVec], df* dg, float* lump,
+                     unsigned long long& mx, auto zero_ok) {
+      const S* up = lo + nn;
+      S l0[5], u0[5], l1[5], u1[5];
+      cell_row(lo + (size_t)j * n, c0, up_row, l0);
+      cell_row(up + (size_t)j * n, c0, up_row, u0);
+      cell_row(lo + (size_t)max(j - 1, 0) * n, c0, dn_row, l1);
+      cell_row(up + (size_t)max(j - 1, 0) * n, c0, dn_row, u1);
+      if (FINE && up_row) {
+#pragma unroll
+        for (int k = 1; k < 5; ++k) {
+          bad |= cell_bad<decltype(zero_ok)::value>(l0[k], mx);
+          bad |= cell_bad<decltype(zero_ok)::value>(u0[k], mx);
+        }
+      }
+      df L0[5], U0[5], L1[5], U1[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        L0[k] = cell_value(l0[k]);
+        U0[k] = cell_value(u0[k]);
+        L1[k] = cell_value(l1[k]);
+        U1[k] = cell_value(u1[k]);
+      }
+      const bool mid = j >= 1 && j < n;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) e[k] = mid ? half_sum(L0[k], U1[k]) : df{0.0f, 0.0f};
+#pragma unroll
+      for (int k = 0; k < kVec; ++k) {
+        const bool col = c0 + k >= 1;
+        no[k] = col && up_row ? half_sum(U0[k + 1], L0[k]) : df{0.0f, 0.0f};
+        // the S edge only enters the diagonal: its high part
+        so[k] = col && dn_row ? 0.5f * (U1[k + 1].h + L1[k].h) : 0.0f;
+        if (dg) dg[k] = up_row ? half_sum(L0[k + 1], U0[k + 1]) : df{0.0f, 0.0f};
+        if (lump)
+          lump[k] = ((L0[k + 1].h + U0[k + 1].h) + (L0[k].h + U1[k + 1].h)) + (L1[k].h + U1[k].h);
+      }
+    };
+    df e[5], no[kVec];
+    float so[kVec], dr[kVec] = {0.0f, 0.0f, 0.0f, 0.0f};
+    edges(cells + (size_t)b * cstride, e, no, so, nullptr, nullptr, top, std::false_type());
+    const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
+    auto put = [&](float* hi, float* lo, auto val) {
+      float h[kVec], l[kVec];
+#pragma unroll
+      for (int k = 0; k < kVec; ++k) {
+        const df v = val(k);
+        h[k] = v.h, l[k] = v.l;
+      }
+      if (hi) st4v(hi + p, h);
+      if (lo) st4v(lo + p, l);
+    };
+    if (RX) {
+      df re[5], rn[kVec], rdg[kVec];
+      float rs[kVec];
+      edges(rcells + (size_t)b * cstride, re, rn, rs, rdg, dr, rtop, std::true_type());
+      const float hr6 = 1.0f / (6.0f * (float)n * (float)n);
+#pragma unroll
+      for (int k = 0; k < kVec; ++k) {
+        const int i = c0 + k;
+        dr[k] = (i >= 1 && i < n && j >= 1 && j < n) ? hr6 * dr[k] : 0.0f;
+      }
+      if (W.rx) {
+        put(W.rx, W.rxl, [&](int k) { return re[k + 1]; });
+        put(W.ry, W.ryl, [&](int k) { return rn[k]; });
+        put(W.rd, W.rdl, [&](int k) { return rdg[k]; });
+      }
+      if (W.hr) st4h(W.hr + p, dr);
+    }
+    put(W.wx, W.wxl, [&](int k) { return e[k + 1]; });
+    put(W.wy, W.wyl, [&](int k) { return no[k]; });
+    float d[kVec], a[kVec], c[kVec];
+#pragma unroll
+    for (int k = 0; k < kVec; ++k) {
+      const int i = c0 + k;
+      a[k] = e[k + 1].h, c[k] = no[k].h;
+      d[k] = (i >= 1 && i < n && j >= 1 && j < n) ? om / (a[k] + e[k].h + c[k] + so[k] + dr[k]) : 0.0f;
+    }
+    if (W.dinv) st4v(W.dinv + p, d);
+    if (W.hx) {
+      st4h(W.hx + p, a);
+      st4h(W.hy + p, c);
+      st4h(W.hd + p, d);
+    }
+  }
+  if (FINE) {
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&ss[b].flags, kFlagBadCoef);
+    auto largest = [&](unsigned long long bits, float* to) {
+      float v = df_split(__longlong_as_double((long long)bits)).h * 1.0001f;
+      if (!(v < INFINITY)) v = 0.0f;
+      for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+      if ((threadIdx.x & 31) == 0 && v > 0.0f) atomicMax((int*)to, __float_as_int(v));  // positive floats order as ints
+    };
+    largest(top, &ss[b].amax);
+    if (RX) largest(rtop, &ss[b].bmax);
+  }
+}
+
+// P u_H at the fine nodes as double-floats: two differences and two products with exact dyadic
+// barycentric coordinates per node (see k_interp); xh, xl: rings zero
+__global__ void __launch_bounds__(kThreads) k_interp4(int n, int nc, int B, const double* __restrict__ uH,
+                                                      float* __restrict__ xh, float* __restrict__ xl) {
+  const int nt = tiles_vec(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  int j, c0;
+  if (b >= B || !vec_walk(n, ch, j, c0)) return;
+  const int lr = ilog2(n / nc), rm = (1 << lr) - 1, ldc = nc + 1;
+  const float inv = 1.0f / (float)(1 << lr);
+  const double* __restrict__ u = uH + (size_t)b * gsz(nc);
+  float h[kVec], l[kVec];
+  const int kj = j & rm;
+#pragma unroll
+  for (int k = 0; k < kVec; ++k) {
+    const int i = c0 + k, ki = i & rm;
+    const int q = (j >> lr) * ldc + (i >> lr);
+    const bool lower = ki >= kj;
+    const df u00 = df_split(u[q]), u11 = df_split(u[q + ldc + 1]), uc = df_split(lower ? u[q + 1] : u[q + ldc]);
+    const float s1 = (float)(lower ? ki : kj) * inv, s2 = (float)(lower ? kj : ki) * inv;
+    const df v = df_add(df_add(u00, df_mul(df_sub(uc, u00), s1)), df_mul(df_sub(u11, uc), s2));
+    h[k] = i ? v.h : 0.0f;
+    l[k] = i ? v.l : 0.0f;
+  }
+  const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
+  st4v(xh + p, h);
+  st4v(xl + p, l);
+}
+
+// block sum of the warp totals of NV double-floats into part[slot][NV] (fixed order)
+template <int NV>
+__device__ __forceinline__ void tile_partials_df(df (&v)[NV], double* part, size_t slot) {
+  __shared__ double red[32 * NV];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int base = 0, c = NV;
+  DfButterfly<NV, 16>::run(v, lane, base, c);
+  if (c >= 1) red[wid * NV + base] = df_double(v[0]);
+  __syncthreads();
+  if (wid == 0 && lane < NV) {
+    double s = red[lane];
+    for (int w = 1; w < nw; ++w) s += red[w * NV + lane];
+    part[slot * NV + lane] = s;
+  }
+}
+
+// the four nodes of a thread and their row neighbours: v[0] = column c0 - 1, v[5] = column c0 + 4
+struct Row6 {
+  float h[kVec + 2], l[kVec + 2];
+};
+template <bool W, bool E>
+__device__ __forceinline__ Row6 load_row6(const float* __restrict__ ph, const float* __restrict__ pl, bool first) {
+  Row6 r;
+  const float4 a = ld4(ph), c = ld4(pl);
+  r.h[1] = a.x, r.h[2] = a.y, r.h[3] = a.z, r.h[4] = a.w;
+  r.l[1] = c.x, r.l[2] = c.y, r.l[3] = c.z, r.l[4] = c.w;
+  r.h[0] = (W && !first) ? ph[-1] : 0.0f;
+  r.l[0] = (W && !first) ? pl[-1] : 0.0f;
+  r.h[5] = E ? ph[kVec] : 0.0f;
+  r.l[5] = E ? pl[kVec] : 0.0f;
+  return r;
+}
+
+// b = M (P u_H) with P u_H in (xh, xl); (bh, bl) = b, v = its FP32 rounding; partial ||b||^2 (it only
+// scales the residual targets: FP32 sums per thread)
+__global__ void __launch_bounds__(kThreads) k_rhs4(int n, int B, const float* __restrict__ xh,
+                                                   const float* __restrict__ xl, float* __restrict__ bh,
+                                                   float* __restrict__ bl, float* __restrict__ v, df hm,
+                                                   double* part) {
+  const int nt = tiles_vec(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  if (b >= B) return;
+  const int ld = sld(n);
+  df acc[1] = {{0.0f, 0.0f}};
+  int j, c0;
+  if (vec_walk(n, ch, j, c0)) {
+    const size_t p = (size_t)b * ssz(n) + (size_t)j * ld + c0;
+    const bool first = c0 == 0;
+    const Row6 C = load_row6<true, true>(xh + p, xl + p, first);
+    const Row6 N = load_row6<false, true>(xh + p + ld, xl + p + ld, first);
+    const Row6 S = load_row6<true, false>(xh + p - ld, xl + p - ld, first);
+    float h[kVec], l[kVec];
+#pragma unroll
+    for (int k = 0; k < kVec; ++k) {
+      const int q = k + 1;
+      df m = df_mul(df{C.h[q], C.l[q]}, 6.0f);
+      df_acc(m, df{C.h[q + 1], C.l[q + 1]});
+      df_acc(m, df{C.h[q - 1], C.l[q - 1]});
+      df_acc(m, df{N.h[q], N.l[q]});
+      df_acc(m, df{S.h[q], S.l[q]});
+      df_acc(m, df{N.h[q + 1], N.l[q + 1]});
+      df_acc(m, df{S.h[q - 1], S.l[q - 1]});
+      df r = df_mul(m, hm);
+      r = fast_two_sum(r.h, r.l);
+      if (first && k == 0) r = {0.0f, 0.0f};
+      h[k] = r.h, l[k] = r.l;
+      acc[0].h = fmaf(r.h, r.h, acc[0].h);
+    }
+    st4v(bh + p, h);
+    st4v(bl + p, l);
+    st4v(v + p, h);
+  }
+  tile_partials_df<1>(acc, part, (size_t)b * nt + ch);
+}
+
+// x += ||r|| xi (double-float x) for samples that ran an inner solve this step
+__global__ void __launch_bounds__(kThreads) k_outer_update4(int n, int B, const SS<float>* __restrict__ ss,
+                                                            const int* __restrict__ ran, const float* __restrict__ xi,
+                                                            float* __restrict__ xh, float* __restrict__ xl) {
+  const int nt = tiles_vec(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  int j, c0;
+  if (b >= B || !ran[b] || !vec_walk(n, ch, j, c0)) return;
+  const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
+  const df rn = df_split(ss[b].rnorm);
+  const float4 d = ld4(xi + p), a = ld4(xh + p), c = ld4(xl + p);
+  float h[kVec], l[kVec];
+#pragma unroll
+  for (int k = 0; k < kVec; ++k) {
+    const df v = df_add(df{at(a, k), at(c, k)}, df_mul(rn, at(d, k)));
+    h[k] = v.h, l[k] = v.l;
+  }
+  st4v(xh + p, h);
+  st4v(xl + p, l);
+}
+
+// Residual r = b - K x, K = A (+ B) - sigma M, in double-float arithmetic; v = r rounded to FP32.
+// With the differences d_q = x_p - x_q to the six neighbours (exact in double-float up to its last
+// bit, and the same on both sides of an edge)
+//     A x = sum_{E,W,N,S} w_q d_q,   M x = h^2 (x_p - S6 / 12),   S6 = sum_q d_q,
+//     B x = h^2/12 (2 x_p sum_q r_q - sum_q r_q d_q),
+// so that the large terms of the operator never cancel against x itself.  Partials: r.r, x.x, x.Kx =
+// x.(b - r), x.S6 and sum x; the scalar kernel forms x.Mx = h^2 (x.x - x.S6 / 12) and x.(A + B)x =
+// x.Kx + sigma x.Mx: the Rayleigh quotient is sigma + x.Kx / x.Mx, whose second term is small (the
+// distance of the fine from the coarse eigenvalue), so the rounding of these sums enters it scaled
+// by that distance.  r.r only steers the refinement: plain FP32.  About 200 FP32 instructions and
+// 36 B (60 B with a reaction) per node; the FP64 form executed 22 FP64 instructions per node.
+struct ResidualIn {
+  const float *wx, *wy, *wxl, *wyl;
+  const float *rx, *ry, *rd, *rxl, *ryl, *rdl;
+};
+template <bool RX>
+__global__ void __launch_bounds__(kThreads) k_residual4(int n, int B, const int* __restrict__ ran, ResidualIn W,
+                                                        const SS<float>* __restrict__ ss, df hm,
+                                                        const float* __restrict__ xh, const float* __restrict__ xl,
+                                                        const float* __restrict__ bh, const float* __restrict__ bl,
+                                                        float* __restrict__ v, double* part, int with_sum) {
+  const int nt = tiles_vec(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  if (b >= B || !ran[b]) return;
+  const int ld = sld(n);
+  // acc: r.r, x.x, x.Kx, x.S6, sum x
+  df acc[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) acc[k] = {0.0f, 0.0f};
+  int j, c0;
+  if (vec_walk(n, ch, j, c0)) {
+    const df cs = ss[b].cs, c12 = ss[b].c12;
+    const size_t p = (size_t)b * ssz(n) + (size_t)j * ld + c0;
+    const bool first = c0 == 0;
+    const Row6 C = load_row6<true, true>(xh + p, xl + p, first);
+    const Row6 N = load_row6<false, true>(xh + p + ld, xl + p + ld, first);
+    const Row6 S = load_row6<true, false>(xh + p - ld, xl + p - ld, first);
+    const float4 wch = ld4(W.wx + p), wcl = ld4(W.wxl + p), ych = ld4(W.wy + p), ycl = ld4(W.wyl + p);
+    const float4 ysh = ld4(W.wy + p - ld), ysl = ld4(W.wyl + p - ld);
+    const float4 b4h = ld4(bh + p), b4l = ld4(bl + p);
+    auto X = [](const Row6& r, int q) { return df{r.h[q], r.l[q]}; };
+    // E-W edges c0 - 1 .. c0 + 3: differences x_i - x_{i+1} and fluxes
+    df dE[kVec + 1], fE[kVec + 1];
+#pragma unroll
+    for (int k = 0; k <= kVec; ++k) {
+      dE[k] = df_sub(X(C, k), X(C, k + 1));
+      const df w = k ? df{at(wch, k - 1), at(wcl, k - 1)}
+                     : (first ? df{0.0f, 0.0f} : df{W.wx[p - 1], W.wxl[p - 1]});
+      fE[k] = df_mul(w, dE[k]);
+    }
+    df rE[kVec + 1], fR[kVec + 1];
+    if (RX) {
+      const float4 h4 = ld4(W.rx + p), l4 = ld4(W.rxl + p);
+#pragma unroll
+      for (int k = 0; k <= kVec; ++k) {
+        rE[k] = k ? df{at(h4, k - 1), at(l4, k - 1)} : (first ? df{0.0f, 0.0f} : df{W.rx[p - 1], W.rxl[p - 1]});
+        fR[k] = df_mul(rE[k], dE[k]);
+      }
+    }
+    float4 rnh, rnl, rsh, rsl, rdh, rdl, reh, rel;
+    df rdw = {0.0f, 0.0f};
+    if (RX) {
+      rnh = ld4(W.ry + p), rnl = ld4(W.ryl + p);
+      rsh = ld4(W.ry + p - ld), rsl = ld4(W.ryl + p - ld);
+      rdh = ld4(W.rd + p), rdl = ld4(W.rdl + p);
+      reh = ld4(W.rd + p - ld), rel = ld4(W.rdl + p - ld);
+      if (!first) rdw = {W.rd[p - ld - 1], W.rdl[p - ld - 1]};
+    }
+    float out[kVec];
+#pragma unroll
+    for (int k = 0; k < kVec; ++k) {
+      const int q = k + 1;
+      const df x = X(C, q);
+      const df dN = df_sub(x, X(N, q)), dS = df_sub(x, X(S, q));
+      const df dNE = df_sub(x, X(N, q + 1)), dSW = df_sub(x, X(S, q - 1));
+      df ax = fE[k + 1];
+      df_acc(ax, df_neg(fE[k]));
+      df_acc(ax, df_mul(df{at(ych, k), at(ycl, k)}, dN));
+      df_acc(ax, df_mul(df{at(ysh, k), at(ysl, k)}, dS));
+      df s6 = dE[k + 1];
+      df_acc(s6, df_neg(dE[k]));
+      df_acc(s6, dN);
+      df_acc(s6, dS);
+      df_acc(s6, dNE);
+      df_acc(s6, dSW);
+      s6 = fast_two_sum(s6.h, s6.l);
+      // r = b + sigma h^2 x - (A x + sigma h^2/12 S6)
+      df r = {at(b4h, k), at(b4l, k)};
+      df_acc(r, df_mul(c12, x));
+      df_acc(r, df_neg(ax));
+      df_acc(r, df_neg(df_mul(cs, s6)));
+      if (RX) {
+        const df rN = {at(rnh, k), at(rnl, k)}, rS = {at(rsh, k), at(rsl, k)}, rNE = {at(rdh, k), at(rdl, k)};
+        const df rSW = k ? df{at(reh, k - 1), at(rel, k - 1)} : rdw;
+        // 2 x sum r_q - sum r_q d_q
+        df rs = rE[k + 1];
+        df_acc(rs, rE[k]);
+        df_acc(rs, rN);
+        df_acc(rs, rS);
+        df_acc(rs, rNE);
+        df_acc(rs, rSW);
+        rs = fast_two_sum(rs.h, rs.l);
+        df bx = df_mul(rs, df{2.0f * x.h, 2.0f * x.l});
+        df_acc(bx, df_neg(fR[k + 1]));
+        df_acc(bx, fR[k]);
+        df_acc(bx, df_neg(df_mul(rN, dN)));
+        df_acc(bx, df_neg(df_mul(rS, dS)));
+        df_acc(bx, df_neg(df_mul(rNE, dNE)));
+        df_acc(bx, df_neg(df_mul(rSW, dSW)));
+        bx = fast_two_sum(bx.h, bx.l);
+        df_acc(r, df_neg(df_mul(hm, bx)));
+      }
+      const bool in = !(first && k == 0);
+      const float rf = in ? __fadd_rn(r.h, r.l) : 0.0f;
+      out[k] = rf;
+      if (in) {  // (x is zero on the ring)
+        acc[0].h = fmaf(rf, rf, acc[0].h);
+        df_acc(acc[1], df_mul(x, x));
+        df_acc(acc[2], df_mul(x, df{at(b4h, k), at(b4l, k)}));
+        df_acc(acc[2], df_mul(x, -rf));
+        df_acc(acc[3], df_mul(x, s6));
+        if (with_sum) df_acc(acc[4], x);
+      }
+    }
+    st4v(v + p, out);
+  }
+  tile_partials_df<5>(acc, part, (size_t)b * nt + ch);
+}
+
+// the scalars of a refinement step from the partial sums of k_residual4
+__global__ void k_sc_outer_end4(int B, int n, int nch, const double* part, const double* sigma, int sig_stride,
+                                const int* ran, SS<float>* ss) {
+  const int b = warp_sample();
+  if (b >= B || !ran[b]) return;
+  double t[5];
+  warp_sum_slots<5>(part, b, nch, t);
+  if ((threadIdx.x & 31) != 0) return;
+  SS<float>& S = ss[b];
+  S.xmx = (t[1] - t[3] / 12.0) / ((double)n * n);
+  S.xax = t[2] + sigma[(size_t)b * sig_stride] * S.xmx;
+  S.xsum = t[4];
+  outer_step_done(S, sqrt(t[0]), sqrt(t[1]));
+}
+
 // V(1,1) up-sweep, vectorised: t = om D^-1 b + P xc at the four nodes and their stencil
 // neighbours, then out = t + om D^-1 (b - A t); with DOT also the partial <dotv, out>.  The coarse
 // correction P xc (mean of the two coarse values on the coarse edge through each fine node) reads
@@ -1246,19 +1686,16 @@ __global__ void k_outer_update(int n, int B, const SS<T>* __restrict__ ss, const
   for_tile(n, ch, [&](int p, int, int) { x64[off + p] += rn * (double)xi[off + p]; });
 }
 
-// FP64 residual r = b - (A - sigma M) x64 (FP64 edge weights); v = T(r).
+// FP64 residual r = b - (A - sigma M) x64 of the FP64 path (the FP32 path: k_residual4); v = T(r).
 // Partials r.r, x.x, x.Ax, x.Mx, sum x: the last pass of a sample gives its Rayleigh quotient and
 // its functional.  The two norms only steer the refinement (stopping tests, the scale of the next
 // correction, which the following pass measures again), so each thread sums them in FP32: GB300
 // issues FP64 at 1/64 of the FP32 rate.  The nodal sum is formed only for the functional (with_sum).
-// (rcb: the reaction coefficient's centroid values [B][2 n^2], or NULL; its seven-point form is added
-// to the operator, formed on the fly in FP64)
 template <typename T>
 __global__ void k_residual(int n, int B, const int* __restrict__ ran, const double* __restrict__ wx64,
                            const double* __restrict__ wy64,
                            const double* __restrict__ sigma, int sig_stride, const double* __restrict__ x64,
-                           const double* __restrict__ b64, T* __restrict__ v, double* part,
-                           const double* __restrict__ rcb, int with_sum) {
+                           const double* __restrict__ b64, T* __restrict__ v, double* part, int with_sum) {
   const int nt = tiles_interior(n);
   const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
   if (b >= B || !ran[b]) return;
@@ -1271,11 +1708,9 @@ __global__ void k_residual(int n, int B, const int* __restrict__ ran, const doub
   const double* __restrict__ X = x64 + off;
   double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   float rr = 0.0f, xx = 0.0f;
-  const double* RB = rcb ? rcb + (size_t)b * 2 * n * n : nullptr;
-  for_tile(n, ch, [&](int p, int i, int j) {
+  for_tile(n, ch, [&](int p, int, int) {
     const double xv = X[p];
-    double ax = stiff<double, double>(WX, WY, X, p, ld);
-    if (RB) ax += hm * react_cells(RB, n, X, p, ld, i, j);
+    const double ax = stiff<double, double>(WX, WY, X, p, ld);
     const double mx = hm * mass7(X, p, ld);
     const double r = b64[off + p] - (ax - sg * mx);
     const float rf = (float)r, xf = (float)xv;
@@ -1298,20 +1733,11 @@ __global__ void k_sc_outer_end(int B, int nch, const double* part, const int* ra
   double t[5];
   warp_sum_slots<5>(part, b, nch, t);
   if ((threadIdx.x & 31) != 0) return;
-  const double s = t[0], sx = t[1], sa = t[2], sm = t[3], su = t[4];
   SS<T>& S = ss[b];
-  S.xnorm = sqrt(sx);
-  S.xax = sa;
-  S.xmx = sm;
-  S.xsum = su;
-  const double rnew = sqrt(s);
-  // No progress: stop refining.  Not on the first step: on fine meshes the FP32 rounding of the
-  // first inner solution alone leaves an FP64 residual above ||b|| (the operator amplifies its
-  // high-frequency part by O(h^-2)); the next step removes it.
-  if (S.outer >= 1 && !(rnew < 0.5 * S.rnorm)) S.act_outer = 0;
-  S.rnorm = rnew;
-  S.rs = T(1.0 / rnew);
-  S.outer += 1;
+  S.xax = t[2];
+  S.xmx = t[3];
+  S.xsum = t[4];
+  outer_step_done(S, sqrt(t[0]), sqrt(t[1]));
 }
 
 // the Rayleigh quotient x.Ax / x.Mx, or with qoi the functional G(x) = h^2 |sum x| / sqrt(x.Mx)
@@ -1408,8 +1834,9 @@ struct Arena {
   int nu;        // Jacobi sweeps per side of the V-cycle (1 or 2)
   size_t V0;
   T *v, *vo, *z, *zn, *w, *wo, *q, *xi;
-  double *x64, *b64;
-  double *wx64, *wy64;  // FP64 edge weights of the finest mesh (the residual operator)
+  double *x64, *b64;  // FP64 path: solution and right-hand side
+  // FP32 path: the same as double-floats, and the low parts of the finest mesh's edge weights
+  float *xh, *xl, *bh, *bl, *wxl, *wyl;
   T *wx[kMaxMG], *wy[kMaxMG], *dinv[kMaxMG], *x[kMaxMG], *t[kMaxMG], *b[kMaxMG];
   // FP32 path: BF16 copies of wx, wy, om D^-1 per streaming level, read by the V(1,1) sweeps
   __nv_bfloat16 *hx[kMaxMG], *hy[kMaxMG], *hd[kMaxMG];
@@ -1418,6 +1845,7 @@ struct Arena {
   // reaction per streaming level (BF16, V(1,1) sweeps) and the coarsened reaction coefficients
   int rxn;
   T *rx, *ry, *rd;
+  float *rxl, *ryl, *rdl;  // their low parts
   __nv_bfloat16* hr[kMaxMG];
   T* rcells[kMaxMG];
   T *bsub, *xsub;
@@ -1444,10 +1872,11 @@ size_t carve_arena(void* base, int n, int B, Arena<T>& A, bool rxn = false) {
   A.wo = c.take<T>(Bz * A.V0);
   A.q = c.take<T>(Bz * A.V0);
   A.xi = c.take<T>(Bz * A.V0);
-  A.x64 = c.take<double>(Bz * A.V0);
-  A.b64 = c.take<double>(Bz * A.V0);
-  A.wx64 = c.take<double>(Bz * A.V0);
-  A.wy64 = c.take<double>(Bz * A.V0);
+  const bool f32 = sizeof(T) == sizeof(float);
+  A.x64 = f32 ? nullptr : c.take<double>(Bz * A.V0);
+  A.b64 = f32 ? nullptr : c.take<double>(Bz * A.V0);
+  float** const pairs[6] = {&A.xh, &A.xl, &A.bh, &A.bl, &A.wxl, &A.wyl};
+  for (float** a : pairs) *a = f32 ? c.take<float>(Bz * A.V0) : nullptr;
   A.Ls = 0;
   for (int nl = n; nl > kSub; nl >>= 1) ++A.Ls;
   for (int l = 0; l < (A.Ls > 1 ? A.Ls : 1); ++l) {  // level 0 always: the MINRES operator
@@ -1467,6 +1896,8 @@ size_t carve_arena(void* base, int n, int B, Arena<T>& A, bool rxn = false) {
   A.rx = rxn ? c.take<T>(Bz * A.V0) : nullptr;
   A.ry = rxn ? c.take<T>(Bz * A.V0) : nullptr;
   A.rd = rxn ? c.take<T>(Bz * A.V0) : nullptr;
+  float** const rlow[3] = {&A.rxl, &A.ryl, &A.rdl};
+  for (float** a : rlow) *a = rxn ? c.take<float>(Bz * A.V0) : nullptr;
   for (int l = 0; l < kMaxMG; ++l) A.rcells[l] = nullptr;
   for (int l = 1; l <= A.Ls; ++l) {
     const size_t nl = (size_t)(n >> l);
@@ -1655,9 +2086,40 @@ cudaError_t close_while(cudaStream_t body) {
   return cudaStreamEndCapture(body, &g);
 }
 
+// the end of a refinement step: x += ||r|| xi, the residual of the new x with the sums of the Rayleigh
+// quotient, the step's scalars
+template <typename T>
+cudaError_t outer_pass(const StreamSolve& s, Arena<T>& A, df hm, cudaStream_t st) {
+  const int n = s.n, B = s.B, gw = (B + 7) / 8;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    const int nt = tiles_vec(n);
+    const ResidualIn W{A.wx[0], A.wy[0], A.wxl, A.wyl, A.rx, A.ry, A.rd, A.rxl, A.ryl, A.rdl};
+    ++tl_launches, k_outer_update4<<<B * nt, kThreads, 0, st>>>(n, B, A.ss, A.ran, A.xi, A.xh, A.xl);
+    LAUNCH_CHECK();
+    ++tl_launches;
+    if (A.rxn)
+      k_residual4<true><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, W, A.ss, hm, A.xh, A.xl, A.bh, A.bl, A.v, A.part, s.qoi);
+    else
+      k_residual4<false><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, W, A.ss, hm, A.xh, A.xl, A.bh, A.bl, A.v, A.part, s.qoi);
+    LAUNCH_CHECK();
+    ++tl_launches, k_sc_outer_end4<<<gw, 256, 0, st>>>(B, n, nt, A.part, s.lamH, s.lam_stride, A.ran, A.ss);
+  } else {
+    const int nt = tiles_interior(n);
+    ++tl_launches, k_outer_update<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ss, A.ran, A.xi, A.x64);
+    LAUNCH_CHECK();
+    ++tl_launches, k_residual<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, A.wx[0], A.wy[0], s.lamH, s.lam_stride, A.x64,
+                                                              A.b64, A.v, A.part, s.qoi);
+    LAUNCH_CHECK();
+    ++tl_launches, k_sc_outer_end<T><<<gw, 256, 0, st>>>(B, nt, A.part, A.ran, A.ss);
+  }
+  LAUNCH_CHECK();
+  return cudaSuccess;
+}
+
 template <typename T>
 cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, const StreamGraph* sg) {
   Arena<T> A;
+  constexpr bool kF32 = sizeof(T) == sizeof(float);
   // the reaction term runs on the FP32 path with V(1,1) smoothing
   if (s.b && (sizeof(T) != sizeof(float) || s.nu != 1)) return cudaErrorNotSupported;
   carve_arena<T>(arena, s.n, s.B, A, s.b != nullptr);
@@ -1666,6 +2128,8 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   const int nt = tiles_interior(n);
   const size_t Bz = (size_t)B;
   const T om = T(s.omega);
+  const double hm64 = 1.0 / (12.0 * n * n);
+  const df hm{(float)hm64, (float)(hm64 - (double)(float)hm64)};
   const int ns = n >> A.Ls;
   const size_t sub_smem = sub_vectors_bytes<T>(ns, A.rxn != 0);
   cudaError_t e = raise_smem_limit((const void*)k_subcycle<T>, (int)sub_smem);
@@ -1681,8 +2145,13 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     ++tl_launches, k_zero<T><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, vecs[k]);
     LAUNCH_CHECK();
   }
-  ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.x64);
-  ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.b64);
+  if constexpr (kF32) {
+    float* const pairs[4] = {A.xh, A.xl, A.bh, A.bl};
+    for (float* a : pairs) ++tl_launches, k_zero<float><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, a);
+  } else {
+    ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.x64);
+    ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.b64);
+  }
   for (int l = 0; l < A.Ls; ++l) {
     const size_t V = ssz(n >> l);
     T* const lv[3] = {A.t[l], A.x[l], A.b[l]};
@@ -1698,15 +2167,36 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   const size_t astride = (size_t)2 * n * n;
   for (int l = 0; l < (A.Ls > 1 ? A.Ls : 1); ++l) {
     const int nl = n >> l;
-    if (l == 0)
+    if constexpr (kF32) {
+      // the V(1,1) sweeps read only the BF16 copies; the operator reads wx, wy of the finest mesh
+      const bool half = A.nu == 1 && A.hx[l];
+      WeightOut W{};
+      W.wx = l && half ? nullptr : A.wx[l];
+      W.wy = l && half ? nullptr : A.wy[l];
+      W.dinv = half ? nullptr : A.dinv[l];
+      W.hx = A.hx[l], W.hy = A.hy[l], W.hd = A.hd[l], W.hr = A.hr[l];
+      ++tl_launches;
+      if (l == 0) {
+        W.wxl = A.wxl, W.wyl = A.wyl;
+        W.rx = A.rx, W.ry = A.ry, W.rd = A.rd, W.rxl = A.rxl, W.ryl = A.ryl, W.rdl = A.rdl;
+        if (A.rxn)
+          k_weights4<double, true><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, s.a, astride, s.b, om, W, A.ss);
+        else
+          k_weights4<double, false><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, s.a, astride, nullptr, om, W, A.ss);
+      } else if (A.rxn) {
+        k_weights4<float, true><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl,
+                                                                          A.rcells[l], om, W, A.ss);
+      } else {
+        k_weights4<float, false><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl,
+                                                                           nullptr, om, W, A.ss);
+      }
+    } else if (l == 0) {
       ++tl_launches, k_weights<T, double><<<B * tiles_padded(nl), kThreads, 0, st>>>(nl, B, s.a, astride, A.wx[0], A.wy[0],
-                                                                     A.dinv[0], om, A.wx64, A.wy64, nullptr, A.ss,
-                                                                     A.hx[0], A.hy[0], A.hd[0], s.b, A.hr[0], A.rx,
-                                                                     A.ry, A.rd);
-    else
+                                                                     A.dinv[0], om, A.ss);
+    } else {
       ++tl_launches, k_weights<T, T><<<B * tiles_padded(nl), kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl, A.wx[l],
-                                                                A.wy[l], A.dinv[l], om, nullptr, nullptr, nullptr, nullptr,
-                                                                A.hx[l], A.hy[l], A.hd[l], A.rcells[l], A.hr[l]);
+                                                                A.wy[l], A.dinv[l], om, nullptr);
+    }
     LAUNCH_CHECK();
     if (l >= A.Ls) continue;
     const int m = nl / 2;
@@ -1731,12 +2221,22 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
                                                                 A.rcells[A.Ls]);
   LAUNCH_CHECK();
   // ---- right-hand side b = M P u_H
-  ++tl_launches, k_interp<T><<<B * nt, kThreads, 0, st>>>(n, s.nc, B, s.uH, A.x64);
+  int nts = nt;  // partial slots per sample of ||b||^2 and of the residual's sums
+  if constexpr (kF32) {
+    // q and xi hold P u_H for a moment (their rings are zero; the first sweep overwrites them)
+    nts = tiles_vec(n);
+    ++tl_launches, k_interp4<<<B * nts, kThreads, 0, st>>>(n, s.nc, B, s.uH, A.q, A.xi);
+    LAUNCH_CHECK();
+    ++tl_launches, k_rhs4<<<B * nts, kThreads, 0, st>>>(n, B, A.q, A.xi, A.bh, A.bl, A.v, hm, A.part);
+  } else {
+    ++tl_launches, k_interp<T><<<B * nt, kThreads, 0, st>>>(n, s.nc, B, s.uH, A.x64);
+    LAUNCH_CHECK();
+    ++tl_launches, k_rhs<T><<<B * nt, kThreads, 0, st>>>(n, B, A.x64, A.b64, A.v, A.part);
+    LAUNCH_CHECK();
+    ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.x64);
+  }
   LAUNCH_CHECK();
-  ++tl_launches, k_rhs<T><<<B * nt, kThreads, 0, st>>>(n, B, A.x64, A.b64, A.v, A.part);
-  LAUNCH_CHECK();
-  ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.x64);
-  ++tl_launches, k_sc_start<T><<<gw, 256, 0, st>>>(B, n, s.lamH, s.lam_stride, nt, A.part, A.ss);
+  ++tl_launches, k_sc_start<T><<<gw, 256, 0, st>>>(B, n, s.lamH, s.lam_stride, nts, A.part, A.ss);
   LAUNCH_CHECK();
   if (sg) {
     // ---- refinement loop as nested WHILE nodes: no host reads.  The inner loop runs iterations in
@@ -1795,10 +2295,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     if ((e = close_while(b1)) != cudaSuccess) return e;
     // an even number of iterations: the rotating vectors are back where they started
     ++tl_launches, k_minres_finish<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.ran, A.ss, zn, wo, w, A.xi);
-    ++tl_launches, k_outer_update<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.ss, A.ran, A.xi, A.x64);
-    ++tl_launches, k_residual<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.ran, A.wx64, A.wy64, s.lamH, s.lam_stride, A.x64,
-                                                             A.b64, A.v, A.part, s.b, s.qoi);
-    ++tl_launches, k_sc_outer_end<T><<<gw, 256, 0, b0>>>(B, nt, A.part, A.ran, A.ss);
+    if ((e = outer_pass<T>(s, A, hm, b0)) != cudaSuccess) return e;
     ++tl_launches, k_cond_outer<<<1, 1, 0, b0>>>(ho, oc, cnt_o, s.max_outer);
     LAUNCH_CHECK();
     if ((e = close_while(b0)) != cudaSuccess) return e;
@@ -1855,11 +2352,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     // apply the pending updates of every sample that ran this step (converged or capped)
     ++tl_launches, k_minres_finish<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, A.ss, zn, wo, w, A.xi);
     LAUNCH_CHECK();
-    ++tl_launches, k_outer_update<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ss, A.ran, A.xi, A.x64);
-    ++tl_launches, k_residual<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, A.wx64, A.wy64, s.lamH, s.lam_stride, A.x64, A.b64, A.v,
-                                               A.part, s.b, s.qoi);
-    ++tl_launches, k_sc_outer_end<T><<<gw, 256, 0, st>>>(B, nt, A.part, A.ran, A.ss);
-    LAUNCH_CHECK();
+    if ((e = outer_pass<T>(s, A, hm, st)) != cudaSuccess) return e;
   }
   }
   // ---- Rayleigh quotient (from each sample's last residual pass)
