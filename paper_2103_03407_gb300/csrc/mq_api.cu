@@ -54,10 +54,11 @@ struct mq_ctx {
   // the sum of |c_t| of the first K terms
   bool sep_ok = false;
   int* d_k1start = nullptr;
-  int* d_tlist = nullptr;
+  int2* d_tlist = nullptr;
   int k1max = 0, k2max = 0;
   std::vector<int> k1prefix;
   std::vector<double> csum;
+  double cabs[2] = {0.0, 0.0};  // sum of |term factors| of a (and, family 2, of b)
   std::map<int, std::pair<void*, mq::SepTables>> sep_tab;  // mesh n -> tables
   int qoi = MQ_QOI_EIGENVALUE;
 
@@ -351,7 +352,7 @@ mq_status coefficients_separable(mq_ctx* c, int n, int K, const double* d_Y, int
       cudaFree(mem);
       return fail(c, MQ_ECUDA, "separable tables: %s", cudaGetErrorString(e));
     }
-    c->n_launches += 6;
+    c->n_launches += 5;
     it = c->sep_tab.emplace(n, std::make_pair(mem, t)).first;
   }
   const int k1pad = mq::tc_pad_k(c->k1prefix[K - 1]);
@@ -360,12 +361,12 @@ mq_status coefficients_separable(mq_ctx* c, int n, int K, const double* d_Y, int
   const double cs = c->csum[K - 1];
   while (std::ldexp(cs, ey) > 1.0) --ey;
   while (std::ldexp(cs, ey + 1) <= 1.0) ++ey;
-  if ((st = grow(c, c->tsl, mq::sep_scratch_bytes(B, n, K, k1pad))) != MQ_OK) return st;
+  if ((st = grow(c, c->tsl, mq::sep_scratch_bytes(B, n, std::max(c->s_max, 1), k1pad))) != MQ_OK) return st;
   if ((st = grow(c, c->tc_err, sizeof(int))) != MQ_OK) return st;
-  const mq::SepTerms terms{c->d_k1start, c->d_tlist, c->d_k2, c->d_cj[0]};
+  const mq::SepTerms terms{c->d_k1start, c->d_tlist, std::max(c->s_max, 1), c->d_cj[0]};
   MQ_CUDA(c, mq::launch_coef_sep(d_Y, ldy, B, K, k1pad, terms, it->second.second, n, c->a0, ey, c->tsl.p, d_a,
-                                 (int*)c->tc_err.p, c->stream));
-  c->n_launches += 5;  // the products Y c, two stage-1 kernels and two tensor-core launches
+                                 (int*)c->tc_err.p, c->stream, std::fabs(c->a0) + 2.0 * cs));
+  c->n_launches += 4;  // the products Y c, stage 1 and two tensor-core launches
   return MQ_OK;
 }
 
@@ -376,6 +377,9 @@ mq_status coefficients(mq_ctx* c, int n, int K, const double* d_Y, int B, int ld
   if (c->family == 2 && (st = ensure_base(c, n, which, &base)) != MQ_OK) return st;
   if (!base && which == 0 && use_separable(c, n, K)) return coefficients_separable(c, n, K, d_Y, B, ldy, d_a);
   const double a0 = base ? 0.0 : c->a0;
+  // |a| for |y| <= 2 (the zeroth terms of family 2 are at most pi / sqrt(2) times their values off and on D_f)
+  const double z0 = base ? 2.3 * std::max(which ? kSigB[0] : kSigA[0], which ? kSigB[1] : kSigA[1]) : c->a0;
+  const double amax = z0 + 2.0 * c->cabs[which];
   if (c->prec == MQ_PREC_MIXED && K > 0) {
     const void* ps = nullptr;
     int kps = 0;
@@ -385,7 +389,7 @@ mq_status coefficients(mq_ctx* c, int n, int K, const double* d_Y, int B, int ld
     if ((st = grow(c, c->tc_err, sizeof(int))) != MQ_OK) return st;
     MQ_LAUNCH(c, mq::launch_y_slices(d_Y, B, ldy, K, kpad, c->ysl.p, c->stream));
     MQ_LAUNCH(c, mq::launch_coef_tc(c->ysl.p, B, kpad, ps, nT, kps, a0, d_a, (int*)c->tc_err.p, c->stream, base,
-                                    c->psi_exp[which]));
+                                    c->psi_exp[which], amax));
     return MQ_OK;
   }
   const double* psi = nullptr;
@@ -1062,11 +1066,13 @@ mq_status set_terms(mq_ctx* c, double a0, int32_t s_max, int32_t family, double 
       while (std::ldexp(mx, e + 1) <= 1.0) ++e;
     }
     c->psi_exp[w] = e;
+    c->cabs[w] = std::accumulate(cj[w].begin(), cj[w].end(), 0.0, [](double s, double v) { return s + std::fabs(v); });
   }
-  // separable evaluation (family 0): the terms grouped by k1 in increasing t
+  // separable evaluation (family 0): the terms grouped by k1 and the parity of k2, in increasing t
   if (c->d_k1start) cudaFree(c->d_k1start);
   if (c->d_tlist) cudaFree(c->d_tlist);
-  c->d_k1start = c->d_tlist = nullptr;
+  c->d_k1start = nullptr;
+  c->d_tlist = nullptr;
   c->sep_ok = false;
   if (family == 0) {
     int k1m = 0, k2m = 0;
@@ -1081,20 +1087,20 @@ mq_status set_terms(mq_ctx* c, double a0, int32_t s_max, int32_t family, double 
       c->csum[t] = cs;
     }
     const int kp = mq::tc_pad_k(k1m);
-    // start[v] .. start[v + 1] lists the terms of k1 = v (start[kp + 1] = m closes the last list)
-    std::vector<int> start(kp + 2, 0), list;
+    // start[v] .. start[v + 1] lists the terms of k1 = v / 2 + 1 with even (v even) or odd k2
+    std::vector<int> start(2 * kp + 1, 0);
+    std::vector<int2> list;
     list.reserve(m);
-    for (int v = 1; v <= kp; ++v) {
+    for (int v = 0; v < 2 * kp; ++v) {
       start[v] = (int)list.size();
       for (int t = 0; t < m; ++t)
-        if (k1[t] == v) list.push_back(t);
+        if (k1[t] == v / 2 + 1 && (k2[t] & 1) == (v & 1)) list.push_back(make_int2(t, k2[t]));
     }
-    start[kp + 1] = (int)list.size();
-    start[0] = 0;
+    start[2 * kp] = (int)list.size();
     MQ_CUDA(c, cudaMalloc(&c->d_k1start, start.size() * sizeof(int)));
-    MQ_CUDA(c, cudaMalloc(&c->d_tlist, std::max<size_t>(list.size(), 1) * sizeof(int)));
+    MQ_CUDA(c, cudaMalloc(&c->d_tlist, std::max<size_t>(list.size(), 1) * sizeof(int2)));
     MQ_CUDA(c, cudaMemcpy(c->d_k1start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice));
-    MQ_CUDA(c, cudaMemcpy(c->d_tlist, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice));
+    MQ_CUDA(c, cudaMemcpy(c->d_tlist, list.data(), list.size() * sizeof(int2), cudaMemcpyHostToDevice));
     c->k1max = k1m;
     c->k2max = k2m;
     c->sep_ok = true;

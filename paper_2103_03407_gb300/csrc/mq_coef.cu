@@ -67,9 +67,10 @@ __global__ void psi_kernel(int n, int s, const int* __restrict__ k1, const int* 
     const size_t t = q % nT;
     long nx, ny;
     centroid_num(n, t, nx, ny);
-    const double x = (double)nx / (double)(3 * n);
-    const double y = (double)ny / (double)(3 * n);
-    double v = cj[j] * sinpi((double)k1[j] * x) * sinpi((double)k2[j] * y);
+    // k x modulo 2 in integers (x = nx / 3n): the argument keeps FP64 accuracy however large k is
+    const double x = (double)((k1[j] * nx) % (6L * n)) / (double)(3 * n);
+    const double y = (double)((k2[j] * ny) % (6L * n)) / (double)(3 * n);
+    double v = cj[j] * sinpi(x) * sinpi(y);
     if (region && region[j]) {
       const bool in = island_band(nx, n) && island_band(ny, n);
       if (in != (region[j] == 1)) v = 0.0;

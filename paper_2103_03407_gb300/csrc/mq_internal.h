@@ -110,24 +110,25 @@ int tc_pad_k(int k);
 // slices of 2^pexp psi (|2^pexp psi| <= 1 required)
 cudaError_t launch_psi_slices(const double* d_psi, int s_rows, int nT, void* d_out, cudaStream_t st, int pexp = 0);
 cudaError_t launch_y_slices(const double* d_Y, int B, int ldy, int k, int kpad, void* d_out, cudaStream_t st);
-// pexp: the scale exponent the psi slices were built with
+// pexp: the scale exponent the psi slices were built with; amax: a bound of |a| (with room for |y| up to
+// 2, four times the lattice points' range), which sets the kernel's fixed-point unit
 cudaError_t launch_coef_tc(const void* d_yslices, int B, int kpad, const void* d_pslices, int nT, int kpad_psi,
-                           double a0, double* d_a, int* d_err, cudaStream_t st, const double* d_base = nullptr,
-                           int pexp = 0);
+                           double a0, double* d_a, int* d_err, cudaStream_t st, const double* d_base,
+                           int pexp, double amax);
 
 // Separable coefficient evaluation for the workload family (mq_tc.cu): the terms grouped by k1
-// (device arrays: tlist[k1start[k1] .. k1start[k1+1]) the terms t of wave number k1 in increasing
-// t; tk2[t] = k2_t; cj[t] = c_t), and per mesh the tables of both triangle planes (sx: BF16 slices
-// of sin(pi k1 x_i), [n][k1pad]; syt: sin(pi k2 y_j), [k2max + 1][n]).
+// (device arrays: list[start[v] .. start[v+1]) the terms (t, k2_t) of wave number k1 = v / 2 + 1 with even (v
+// even) or odd k2, in increasing t; nlist entries in all; cj[t] = c_t), and per mesh the tables (sx: BF16 slices of sin(pi k1 x_i) of both triangle planes,
+// [n][k1pad]; sy: sin(pi k2 y_j) of the lower plane in fixed point, [k2max + 1][n]).
 struct SepTerms {
-  const int* k1start;
-  const int* tlist;
-  const int* tk2;
+  const int* start;
+  const int2* list;
+  int nlist;
   const double* cj;
 };
 struct SepTables {
   const void* sx[2];
-  const double* syt[2];
+  const int2* sy;
   int k1pad;
 };
 size_t sep_tables_bytes(int n, int k1pad, int k2max);
@@ -136,11 +137,11 @@ cudaError_t launch_sep_tables(int n, int k1max, int k1pad, int k2max, double* d_
                               cudaStream_t st);
 // a[b][t] for B rows of Y with the first K terms: k1pad >= the padded largest k1 of those terms,
 // ey the exponent with |2^ey T| <= 1/2 for every stage-1 value T; d_tslices: sep_scratch_bytes(B,
-// n, K, k1pad) bytes of scratch (the stage-1 slices, then the products Y c)
-size_t sep_scratch_bytes(int B, int n, int K, int k1pad);
+// n, nlist, k1pad) bytes of scratch (the stage-1 slices of both planes, then the products Y c)
+size_t sep_scratch_bytes(int B, int n, int nlist, int k1pad);
 cudaError_t launch_coef_sep(const double* d_Y, int ldy, int B, int K, int k1pad, const SepTerms& terms,
                             const SepTables& tab, int n, double a0, int ey, void* d_tslices, double* d_a, int* d_err,
-                            cudaStream_t st);
+                            cudaStream_t st, double amax);
 
 // Sample flags (stat[b][3])
 enum : int {
