@@ -26,6 +26,7 @@
 #include <cstddef>
 #include <cstdint>
 
+#include "mq_df.cuh"
 #include "mq_internal.h"
 
 namespace mq {
@@ -76,7 +77,7 @@ struct MGDesc {
 };
 
 template <typename T>
-__host__ __device__ void carve_mg(Carver& c, int n, MGDesc<T>& d, bool reaction = false) {
+__host__ __device__ void carve_mg(Carver& c, int n, MGDesc<T>& d, bool reaction = false, bool cells_too = true) {
   d.L = ilog2(n);
   for (int l = 0; l < d.L; ++l) {
     const int nl = n >> l;
@@ -90,11 +91,13 @@ __host__ __device__ void carve_mg(Carver& c, int n, MGDesc<T>& d, bool reaction 
     d.b[l] = l ? c.take<T>(V) : nullptr;
     d.dr[l] = reaction ? c.take<T>(V) : nullptr;
   }
-  const size_t cells = n >= 4 ? (size_t)2 * (n / 2) * (n / 2) : 1;
-  d.cell[0] = c.take<T>(cells);
-  d.cell[1] = c.take<T>(cells);
-  d.rcell[0] = reaction ? c.take<T>(cells) : nullptr;
-  d.rcell[1] = reaction ? c.take<T>(cells) : nullptr;
+  if (cells_too) {  // else the caller places the building buffers
+    const size_t cells = n >= 4 ? (size_t)2 * (n / 2) * (n / 2) : 1;
+    d.cell[0] = c.take<T>(cells);
+    d.cell[1] = c.take<T>(cells);
+    d.rcell[0] = reaction ? c.take<T>(cells) : nullptr;
+    d.rcell[1] = reaction ? c.take<T>(cells) : nullptr;
+  }
   d.cinv = c.take<T>(81);
   d.Lc = d.L >= 2 ? d.L - 2 : d.L - 1;
 }
@@ -283,29 +286,68 @@ __device__ __forceinline__ double react_cells(const double* __restrict__ b, int 
 }
 
 // ---------------------------------------------------------------------------------------------
-// operator setup
+// operator setup.  FP32 arrays are formed on the FP32 units, from FP64 coefficients by double-floats (an
+// FP64 addition or conversion takes sixteen clocks of an SM); FP64 arrays in FP64.
 template <typename T, typename S>
-__device__ void weights_from_cells(int n, const S* low, const S* up, T* wx, T* wy) {
+struct CellSum {  // (a + b) / 2 and sums of coefficients in T
+  static __device__ __forceinline__ T half(S a, S b) { return T(0.5) * (T(a) + T(b)); }
+  static __device__ __forceinline__ T val(S a) { return T(a); }
+};
+template <>
+struct CellSum<float, double> {
+  static __device__ __forceinline__ float half(double a, double b) { return 0.5f * df_add(df_split(a), df_split(b)).h; }
+  static __device__ __forceinline__ float val(double a) {
+    const df d = df_split(a);
+    return d.h + d.l;
+  }
+};
+// a coefficient that is not positive (not nonnegative with zero_ok), or NaN; on the integer units
+__device__ __forceinline__ int cell_invalid(double v, bool zero_ok) {
+  const long long b = __double_as_longlong(v);
+  return !((zero_ok ? b >= 0 : b > 0) && b <= 0x7ff0000000000000LL);
+}
+__device__ __forceinline__ int cell_invalid(float v, bool zero_ok) { return !(zero_ok ? v >= 0.0f : v > 0.0f); }
+
+// (lx, ly: NULL, or the low parts of the weights -- FP32 weights of FP64 coefficients as double-floats)
+template <typename T, typename S>
+__device__ void weights_from_cells(int n, const S* low, const S* up, T* wx, T* wy, T* lx = nullptr, T* ly = nullptr) {
   const int ld = n + 1;
   for_all(gsz(n), [&](size_t q) {
     const int i = (int)(q % ld), j = (int)(q / ld);
-    T a = T(0), b = T(0);
-    if (i <= n - 1 && j >= 1 && j <= n - 1) a = T(0.5 * ((double)low[j * n + i] + (double)up[(j - 1) * n + i]));
-    if (i >= 1 && i <= n - 1 && j <= n - 1) b = T(0.5 * ((double)up[j * n + i] + (double)low[j * n + i - 1]));
-    wx[q] = a;
-    wy[q] = b;
+    const bool e = i <= n - 1 && j >= 1 && j <= n - 1, v = i >= 1 && i <= n - 1 && j <= n - 1;
+    if constexpr (sizeof(T) == sizeof(float) && sizeof(S) == sizeof(double)) {
+      if (lx) {
+        df a = {0.0f, 0.0f}, b = {0.0f, 0.0f};
+        if (e) a = df_add(df_split(low[j * n + i]), df_split(up[(j - 1) * n + i]));
+        if (v) b = df_add(df_split(up[j * n + i]), df_split(low[j * n + i - 1]));
+        wx[q] = 0.5f * a.h, lx[q] = 0.5f * a.l;
+        wy[q] = 0.5f * b.h, ly[q] = 0.5f * b.l;
+        return;
+      }
+    }
+    wx[q] = e ? CellSum<T, S>::half(low[j * n + i], up[(j - 1) * n + i]) : T(0);
+    wy[q] = v ? CellSum<T, S>::half(up[j * n + i], low[j * n + i - 1]) : T(0);
   });
 }
 
 // the reaction's edge weights: rx, ry as the stiffness weights of b (same two triangles per edge),
 // rd of the hypotenuse (i,j)-(i+1,j+1) = (b_low(i,j) + b_up(i,j)) / 2
 template <typename T, typename S>
-__device__ void reaction_weights(int n, const S* low, const S* up, T* rx, T* ry, T* rd) {
-  weights_from_cells<T, S>(n, low, up, rx, ry);
+__device__ void reaction_weights(int n, const S* low, const S* up, T* rx, T* ry, T* rd, T* lx = nullptr,
+                                 T* ly = nullptr, T* ld_ = nullptr) {
+  weights_from_cells<T, S>(n, low, up, rx, ry, lx, ly);
   const int ld = n + 1;
   for_all(gsz(n), [&](size_t q) {
     const int i = (int)(q % ld), j = (int)(q / ld);
-    rd[q] = (i <= n - 1 && j <= n - 1) ? T(0.5 * ((double)low[j * n + i] + (double)up[j * n + i])) : T(0);
+    const bool in = i <= n - 1 && j <= n - 1;
+    if constexpr (sizeof(T) == sizeof(float) && sizeof(S) == sizeof(double)) {
+      if (ld_) {
+        const df d = in ? df_add(df_split(low[j * n + i]), df_split(up[j * n + i])) : df{0.0f, 0.0f};
+        rd[q] = 0.5f * d.h, ld_[q] = 0.5f * d.l;
+        return;
+      }
+    }
+    rd[q] = in ? CellSum<T, S>::half(low[j * n + i], up[j * n + i]) : T(0);
   });
 }
 
@@ -313,14 +355,15 @@ __device__ void reaction_weights(int n, const S* low, const S* up, T* rx, T* ry,
 template <typename T, typename S>
 __device__ void lumped_reaction(int n, const S* low, const S* up, T* dr) {
   const int ld = n + 1;
-  const double f = 1.0 / (6.0 * (double)n * (double)n);
+  const T f = T(1) / (T(6) * T(n) * T(n));
+  using C = CellSum<T, S>;
   for_all(gsz(n), [&](size_t q) {
     const int i = (int)(q % ld), j = (int)(q / ld);
     T v = T(0);
     if (i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1) {
       const int c = j * n + i;
-      v = T(f * ((double)low[c] + (double)up[c] + (double)low[c - 1] + (double)up[c - n] + (double)low[c - n - 1] +
-                 (double)up[c - n - 1]));
+      v = f * (C::val(low[c]) + C::val(up[c]) + C::val(low[c - 1]) + C::val(up[c - n]) + C::val(low[c - n - 1]) +
+               C::val(up[c - n - 1]));
     }
     dr[q] = v;
   });
@@ -329,15 +372,16 @@ __device__ void lumped_reaction(int n, const S* low, const S* up, T* dr) {
 template <typename T, typename S>
 __device__ void coarsen_cells(int n, const S* low, const S* up, T* out) {
   const int m = n / 2;
+  using C = CellSum<T, S>;
   for_all((size_t)m * m, [&](size_t q) {
     const int I = (int)(q % m), J = (int)(q / m);
     const int i = 2 * I, j = 2 * J;
-    const double lo = (double)low[j * n + i] + (double)low[j * n + i + 1] + (double)low[(j + 1) * n + i + 1] +
-                      (double)up[j * n + i + 1];
-    const double hi = (double)up[j * n + i] + (double)up[(j + 1) * n + i + 1] + (double)up[(j + 1) * n + i] +
-                      (double)low[(j + 1) * n + i];
-    out[q] = T(0.25 * lo);
-    out[m * m + q] = T(0.25 * hi);
+    const T lo = C::val(low[j * n + i]) + C::val(low[j * n + i + 1]) + C::val(low[(j + 1) * n + i + 1]) +
+                 C::val(up[j * n + i + 1]);
+    const T hi = C::val(up[j * n + i]) + C::val(up[(j + 1) * n + i + 1]) + C::val(up[(j + 1) * n + i]) +
+                 C::val(low[(j + 1) * n + i]);
+    out[q] = T(0.25) * lo;
+    out[m * m + q] = T(0.25) * hi;
   });
 }
 
@@ -421,15 +465,17 @@ __device__ void coarse_inverse4(const T* wx, const T* wy, T* cinv, const T* dr =
 
 // Builds every level (weights, inverse diagonals) from the fine centroid coefficients a, and with
 // rb (hierarchy carved with the reaction arrays) the lumped reaction of every level from the
-// centroid values rb of the reaction coefficient.  Returns true when every a is positive
+// centroid values rb of the reaction coefficient (lx, ly: NULL, or the low parts of the finest weights, see
+// weights_from_cells).  Returns true when every a is positive
 // (Assumption A1) and every b nonnegative.
 template <typename T, typename S = double>
-__device__ bool build_mg(MGDesc<T>& d, const S* __restrict__ a, int n, double* red, const S* __restrict__ rb = nullptr) {
+__device__ bool build_mg(MGDesc<T>& d, const S* __restrict__ a, int n, double* red, const S* __restrict__ rb = nullptr,
+                         T* lx = nullptr, T* ly = nullptr) {
   int bad = 0;
   const bool rx = rb != nullptr && d.dr[0] != nullptr;
-  for_all((size_t)2 * n * n, [&](size_t q) { bad |= !(a[q] > S(0)); });
-  if (rx) for_all((size_t)2 * n * n, [&](size_t q) { bad |= !(rb[q] >= S(0)); });
-  weights_from_cells<T, S>(n, a, a + (size_t)n * n, d.wx[0], d.wy[0]);
+  for_all((size_t)2 * n * n, [&](size_t q) { bad |= cell_invalid(a[q], false); });
+  if (rx) for_all((size_t)2 * n * n, [&](size_t q) { bad |= cell_invalid(rb[q], true); });
+  weights_from_cells<T, S>(n, a, a + (size_t)n * n, d.wx[0], d.wy[0], lx, ly);
   if (d.L > 1) coarsen_cells<T, S>(n, a, a + (size_t)n * n, d.cell[0]);
   if (rx) {
     lumped_reaction<T, S>(n, rb, rb + (size_t)n * n, d.dr[0]);
@@ -452,9 +498,8 @@ __device__ bool build_mg(MGDesc<T>& d, const S* __restrict__ a, int n, double* r
   inverse_diagonal<T>(d.n[d.L - 1], d.wx[d.L - 1], d.wy[d.L - 1], d.dinv[d.L - 1], rx ? d.dr[d.L - 1] : nullptr);
   if (d.L >= 2 && threadIdx.x == 0)
     coarse_inverse4<T>(d.wx[d.L - 2], d.wy[d.L - 2], d.cinv, rx ? d.dr[d.L - 2] : nullptr);
-  double v[1] = {(double)bad}, o[1];
-  block_sum<1, double>(v, o, red);
-  return o[0] == 0.0;
+  (void)red;
+  return __syncthreads_or(bad) == 0;
 }
 
 // Symmetric V-cycle for A (A + D_B when the hierarchy holds a lumped reaction, which build_mg must

@@ -84,6 +84,38 @@ __host__ __device__ void carve_coarse(Carver& c, int nc, CoarseWS& ws, size_t* p
   carve_mg<float>(c, nc, ws.mg, reaction);
 }
 
+// Coarse eigensolve workspace of the FP32 kernel (lobpcg32): the iterate as a double-float pair, the
+// operator's weights as pairs (their high parts are the multigrid hierarchy's finest weights), the
+// search directions and their images in FP32.
+struct CoarseWS32 {
+  MGDesc<float> mg;
+  float *xh, *xl, *wxl, *wyl, *r, *w, *mw, *p, *ap, *mp;
+  float *rx, *ry, *rd, *rxl, *ryl, *rdl;  // reaction edge weights and their low parts (NULL without a reaction term)
+};
+
+// Meshes whose coarse problem the FP32 kernel solves with lobpcg32: its residual floor, about 2^-48 4 n / theta
+// relative, stays below every eigen-residual target in use (1e-12 at the least) up to 1/128.
+constexpr int kEig32Max = 128;
+
+// xh, xl come first: they hold the coarse eigenvector through the fine solves
+__host__ __device__ void carve_coarse32(Carver& c, int nc, CoarseWS32& ws, size_t* persist = nullptr,
+                                        bool reaction = false) {
+  const size_t V = gsz(nc);
+  ws.xh = c.take<float>(V);
+  ws.xl = c.take<float>(V);
+  if (persist) *persist = c.used();
+  float** const a[8] = {&ws.wxl, &ws.wyl, &ws.r, &ws.w, &ws.mw, &ws.p, &ws.ap, &ws.mp};
+  for (float** v : a) *v = c.take<float>(V);
+  float** const b[6] = {&ws.rx, &ws.ry, &ws.rd, &ws.rxl, &ws.ryl, &ws.rdl};
+  for (float** v : b) *v = reaction ? c.take<float>(V) : nullptr;
+  carve_mg<float>(c, nc, ws.mg, reaction, false);
+  // the coefficients of the coarser meshes are needed only while the hierarchy is built, before ap and mp are
+  ws.mg.cell[0] = ws.ap;
+  ws.mg.cell[1] = ws.mp;
+  ws.mg.rcell[0] = reaction ? ws.mw : nullptr;
+  ws.mg.rcell[1] = reaction ? c.take<float>((size_t)nc * nc / 2 + 1) : nullptr;
+}
+
 // Fine shifted-solve workspace: FP64 solution and right-hand side, inner vectors in T.
 template <typename T>
 struct FineWS {
@@ -130,9 +162,14 @@ __host__ __device__ size_t fine_bytes(int n, bool reaction = false) {
 template <typename T>
 __host__ __device__ size_t slab_size(int nf, int nc, int np, int mode_f = 0, int mode_p = 0, bool reaction = false) {
   Carver c(nullptr);
-  CoarseWS cw;
   size_t persist = 0;
-  carve_coarse(c, nc, cw, &persist, reaction);
+  if (sizeof(T) == sizeof(float) && nc <= kEig32Max) {
+    CoarseWS32 cw;
+    carve_coarse32(c, nc, cw, &persist, reaction);
+  } else {
+    CoarseWS cw;
+    carve_coarse(c, nc, cw, &persist, reaction);
+  }
   persist = (persist + 15) & ~(size_t)15;  // the fine region starts 16-byte aligned
   const size_t coarse = (c.used() + 15) & ~(size_t)15;
   auto need = [&](int n, int mode) -> size_t {
@@ -444,6 +481,292 @@ __device__ __noinline__ int lobpcg(CoarseWS& ws, int n, double tol, int maxit, i
   return conv ? it : -1;
 }
 
+// Block sum of NV double-floats (fixed order: deterministic); thread 0 runs ep(totals) before the closing
+// barrier.  red as in block_sum.
+template <int NV, class Ep>
+__device__ __forceinline__ void block_sum_df(df (&v)[NV], double* red, Ep ep) {
+  static_assert(NV <= 12, "block_sum_df reduces at most 12 values");
+  df* part = reinterpret_cast<df*>(red);
+  df* tot = part + 32 * 12;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int base = 0, c = NV;
+  DfButterfly<NV, 16>::run(v, lane, base, c);
+  if (c >= 1) part[wid * NV + base] = v[0];
+  __syncthreads();
+  if (wid == 0) {
+    if (lane < NV) {
+      df s = part[lane];
+      for (int w = 1; w < nw; ++w) s = df_add(s, part[w * NV + lane]);
+      tot[lane] = s;
+    }
+    __syncwarp();
+    if (lane == 0) {
+      df t[NV];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) t[i] = tot[i];
+      ep(t);
+    }
+  }
+  __syncthreads();
+}
+
+struct Eig32Shared {
+  df theta;        // shift of the residual: the predicted Rayleigh quotient
+  float delta;     // x.r / x.Mx: the Rayleigh quotient is theta + delta
+  float xmx;
+  float al, be;    // x += al w + be p
+  int conv, ok;
+  double lam, g, scale;
+};
+
+// Rayleigh-Ritz on the basis [x, w, p] (k = 3; [x, w] for k = 2) for lobpcg32, by one thread: the smallest
+// eigenpair of the pencil shifted by the Rayleigh quotient of x, so that x.Kx = 0.  With the scaled x as
+// first unit vector the eigenvector is (1, y), y = -C(mu)^{-1} g(mu), where C and g are the other block and
+// the coupling of K - mu M; the iteration mu <- Rayleigh quotient of (1, y) is Newton's on the Schur
+// complement, which decreases and is concave left of C's eigenvalues, so from mu = 0 it converges
+// monotonically to the smallest eigenvalue and quadratically (the shift is small by then).  Returns
+// false when C(0) is not safely positive definite or w and p are nearly parallel.
+__device__ bool ritz_newton(float m00, const float b[2], const float m0[2], const float K[3], const float M[3], int k,
+                            float& al, float& be, float& mu) {
+  // K, M: entries 11, 12, 22 of the block on w, p
+  if (!(m00 > 0.0f) || !(M[0] > 0.0f) || (k > 2 && !(M[2] > 0.0f))) return false;
+  const float d0 = rsqrtf(m00), d1 = rsqrtf(M[0]), d2 = k > 2 ? rsqrtf(M[2]) : 0.0f;
+  const float m12 = k > 2 ? M[1] * d1 * d2 : 0.0f, k11 = K[0] * d1 * d1;
+  const float k12 = k > 2 ? K[1] * d1 * d2 : 0.0f, k22 = k > 2 ? K[2] * d2 * d2 : 1.0f;
+  const float m22 = k > 2 ? 1.0f : 0.0f;
+  const float k01 = b[0] * d0 * d1, k02 = k > 2 ? b[1] * d0 * d2 : 0.0f;
+  const float m01 = m0[0] * d0 * d1, m02 = k > 2 ? m0[1] * d0 * d2 : 0.0f;
+  if (!(1.0f - m12 * m12 > 1e-5f)) return false;
+  if (!(k11 > 0.0f) || !(k22 > 0.0f) || !(k11 * k22 - k12 * k12 > 1e-5f * k11 * k22)) return false;
+  float y1 = 0.0f, y2 = 0.0f, m = 0.0f;
+#pragma unroll 1
+  for (int it = 0; it < 6; ++it) {
+    const float c11 = k11 - m, c12 = k12 - m * m12, c22 = k22 - m * m22;
+    const float g1 = k01 - m * m01, g2 = k02 - m * m02;
+    const float idet = 1.0f / (c11 * c22 - c12 * c12);
+    y1 = (c12 * g2 - c22 * g1) * idet;
+    y2 = (c12 * g1 - c11 * g2) * idet;
+    const float num = 2.0f * (k01 * y1 + k02 * y2) + k11 * y1 * y1 + 2.0f * k12 * y1 * y2 + (k > 2 ? k22 * y2 * y2 : 0.0f);
+    const float den = 1.0f + 2.0f * (m01 * y1 + m02 * y2) + y1 * y1 + 2.0f * m12 * y1 * y2 + m22 * y2 * y2;
+    if (!(den > 1e-3f)) return false;
+    const float mn = num / den;
+    const bool done = fabsf(mn - m) <= 1e-6f * fabsf(mn);
+    m = mn;
+    if (done) break;
+  }
+  mu = m;
+  al = y1 * d1 / d0;
+  be = y2 * d2 / d0;
+  return isfinite(al) && isfinite(be) && isfinite(mu);
+}
+
+// LOBPCG of the FP32 kernel: as lobpcg, with only the iterate and its residual r = A x - theta M x in more
+// than FP32.  The residual is formed afresh from x in double-floats each iteration (differences first, as
+// in the streaming tier's residual), with theta the Rayleigh quotient predicted by the last
+// Rayleigh-Ritz step; x.r gives the exact quotient.  Everything else -- the preconditioned residual w
+// (an FP32 V-cycle), the last correction p, their images and the Gram matrix of the shifted pencil --
+// only steers the correction x += al w + be p, whose FP32 rounding the next residual corrects.  The
+// FP64 form keeps nine FP64 vectors (one sample of mesh 1/32 per SM) and executes about 60 FP64
+// instructions per node and iteration, at sixteen clocks of an SM each; this one needs about 300 FP32
+// instructions and half the memory.  8,192 direct eigensolves on mesh 1/32 (a window of
+// the six-level workload's level 0): 15.8 -> 5.3 ms.  On return xh + xl is the M-normalised eigenvector with a positive sum, lam its Rayleigh quotient, g =
+// |integral of x|; the result is the iterations used or -1.
+__device__ __noinline__ int lobpcg32(CoarseWS32& ws, int n, double tol, int maxit, int nu, float omega, double* red,
+                                     Eig32Shared* sh, double lam0, double& lam, double& g) {
+  const int ld = n + 1;
+  const double hm64 = 1.0 / (12.0 * n * n);
+  const float h2 = 1.0f / ((float)n * (float)n), hm = h2 / 12.0f;
+  const df hmd = {(float)hm64, (float)(hm64 - (double)(float)hm64)};
+  const float* __restrict__ wxh = ws.mg.wx[0];
+  const float* __restrict__ wyh = ws.mg.wy[0];
+  float* __restrict__ aw = ws.mg.t[0];  // free outside the V-cycle
+  if (threadIdx.x == 0) {
+    sh->theta = df_split(lam0);
+    sh->conv = 0;
+  }
+  __syncthreads();
+  const float tol2 = (float)(tol * tol);
+  // r = A x - theta M x; sums x.r, x.x, x.S6, r.r, r.Mx, Mx.Mx; last: the Rayleigh quotient in FP64
+  auto residual = [&](bool last) {
+    const df th = sh->theta;
+    df c2 = df_mul(th, h2), c12 = df_mul(th, hmd);
+    c12 = fast_two_sum(c12.h, c12.l);
+    df acc[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) acc[k] = {0.0f, 0.0f};
+    for_interior(n, [&](int p, int, int) {
+      auto X = [&](int q) { return df{ws.xh[q], ws.xl[q]}; };
+      const df x = X(p);
+      const df dE = df_sub(x, X(p + 1)), dW = df_sub(x, X(p - 1)), dN = df_sub(x, X(p + ld)), dS = df_sub(x, X(p - ld));
+      const df dNE = df_sub(x, X(p + ld + 1)), dSW = df_sub(x, X(p - ld - 1));
+      df r = df_mul(df{wxh[p], ws.wxl[p]}, dE);
+      df_acc(r, df_mul(df{wxh[p - 1], ws.wxl[p - 1]}, dW));
+      df_acc(r, df_mul(df{wyh[p], ws.wyl[p]}, dN));
+      df_acc(r, df_mul(df{wyh[p - ld], ws.wyl[p - ld]}, dS));
+      df s6 = dE;
+      df_acc(s6, dW);
+      df_acc(s6, dN);
+      df_acc(s6, dS);
+      df_acc(s6, dNE);
+      df_acc(s6, dSW);
+      s6 = fast_two_sum(s6.h, s6.l);
+      if (ws.rx) {
+        // h^2/12 (2 x sum r_q - sum r_q d_q)
+        const int q[6] = {p, p - 1, p, p - ld, p, p - ld - 1};
+        const float* const h[6] = {ws.rx, ws.rx, ws.ry, ws.ry, ws.rd, ws.rd};
+        const float* const l[6] = {ws.rxl, ws.rxl, ws.ryl, ws.ryl, ws.rdl, ws.rdl};
+        const df d[6] = {dE, dW, dN, dS, dNE, dSW};
+        df rs = {0.0f, 0.0f}, rdq = {0.0f, 0.0f};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const df w = {h[k][q[k]], l[k][q[k]]};
+          df_acc(rs, w);
+          df_acc(rdq, df_mul(w, d[k]));
+        }
+        rs = fast_two_sum(rs.h, rs.l);
+        df bx = df_mul(rs, df{2.0f * x.h, 2.0f * x.l});
+        df_acc(bx, df_neg(rdq));
+        bx = fast_two_sum(bx.h, bx.l);
+        df_acc(r, df_mul(hmd, bx));
+      }
+      df_acc(r, df_neg(df_mul(c2, x)));
+      df_acc(r, df_mul(c12, s6));
+      r = fast_two_sum(r.h, r.l);
+      ws.r[p] = r.h;
+      const float mx = h2 * (x.h - s6.h * (1.0f / 12.0f));
+      df_acc(acc[0], df_mul(r, x));
+      df_acc(acc[1], df_mul(x, x));
+      df_acc(acc[2], df_mul(x, s6));
+      acc[3].h = fmaf(r.h, r.h, acc[3].h);
+      acc[4].h = fmaf(r.h, mx, acc[4].h);
+      acc[5].h = fmaf(mx, mx, acc[5].h);
+    });
+    block_sum_df<6>(acc, red, [&](const df* t) {
+      const float xmx = h2 * (t[1].h - t[2].h * (1.0f / 12.0f));
+      const float d = (t[0].h + t[0].l) / xmx;
+      sh->xmx = xmx;
+      sh->delta = d;
+      const float th1 = th.h + d, rr = t[3].h - 2.0f * d * t[4].h + d * d * t[5].h;
+      sh->conv = rr <= tol2 * th1 * th1 * t[5].h;
+      if (last || sh->conv) {
+        const double m = (df_double(t[1]) - df_double(t[2]) / 12.0) / ((double)n * n);
+        sh->lam = df_double(th) + df_double(t[0]) / m;
+        sh->scale = 1.0 / sqrt(m);
+      }
+    });
+  };
+  // the shift of a start vector is only a guess: one pass measures it
+  residual(false);
+  if (threadIdx.x == 0) sh->theta = df_add(sh->theta, df{sh->delta, 0.0f});
+  __syncthreads();
+  bool have_p = false;
+  int it = 0, conv = 0, evaluated = 0;
+  for (;; ++it) {
+    residual(it == maxit);
+    if (sh->conv) conv = 1;
+    if (conv || it == maxit) {
+      evaluated = 1;
+      break;
+    }
+    vcycle<float>(ws.mg, ws.r, ws.w, omega, nullptr, nu);
+    {
+      const float th = sh->theta.h + sh->delta;
+      float acc[10];
+      double o[10];
+#pragma unroll
+      for (int i = 0; i < 10; ++i) acc[i] = 0.0f;
+      for_interior(n, [&](int p, int, int) {
+        float a = stiff<float, float>(wxh, wyh, ws.w, p, ld);
+        if (ws.rx) a += hm * react7<float, float>(ws.rx, ws.ry, ws.rd, ws.w, p, ld);
+        const float m = hm * mass7(ws.w, p, ld);
+        aw[p] = a;
+        ws.mw[p] = m;
+        const float wv = ws.w[p], xv = ws.xh[p], rv = ws.r[p], kw = a - th * m;
+        acc[0] += wv * rv;
+        acc[1] += xv * m;
+        acc[2] += wv * kw;
+        acc[3] += wv * m;
+        if (have_p) {
+          const float pv = ws.p[p], pm = ws.mp[p];
+          acc[4] += pv * rv;
+          acc[5] += xv * pm;
+          acc[6] += pv * kw;
+          acc[7] += pv * m;
+          acc[8] += pv * (ws.ap[p] - th * pm);
+          acc[9] += pv * pm;
+        }
+      });
+      const bool hp = have_p;
+      block_sum<10, float>(acc, o, red, [&](const double* t) {
+        float v[10];
+        for (int i = 0; i < 10; ++i) v[i] = (float)t[i];
+        const float dl = sh->delta;
+        const float b[2] = {v[0] - dl * v[1], v[4] - dl * v[5]}, m0[2] = {v[1], v[5]};
+        const float K[3] = {v[2], v[6], v[8]}, M[3] = {v[3], v[7], v[9]};
+        float al = 0.0f, be = 0.0f, mu = 0.0f;
+        bool ok = (hp && ritz_newton(sh->xmx, b, m0, K, M, 3, al, be, mu)) || ritz_newton(sh->xmx, b, m0, K, M, 2, al, be, mu);
+        if (!ok) {
+          const float GA[3][3] = {{0.0f, b[0], b[1]}, {b[0], K[0], K[1]}, {b[1], K[1], K[2]}};
+          const float GM[3][3] = {{sh->xmx, m0[0], m0[1]}, {m0[0], M[0], M[1]}, {m0[1], M[1], M[2]}};
+          float c[3];
+          const int k = rayleigh_ritz_shifted(GA, GM, hp ? 3 : 2, c, mu);
+          ok = k > 0 && c[0] != 0.0f;
+          if (ok) {
+            al = c[1] / c[0];
+            be = k > 2 ? c[2] / c[0] : 0.0f;
+          }
+        }
+        sh->al = al;
+        sh->be = be;
+        sh->ok = ok;
+        sh->theta = df_add(sh->theta, two_sum(dl, mu));
+      });
+    }
+    if (!sh->ok) break;
+    const float al = sh->al, be = sh->be;
+    const bool use_p = have_p && be != 0.0f;
+    for_interior(n, [&](int p, int, int) {
+      const float pv = use_p ? ws.p[p] : 0.0f, apv = use_p ? ws.ap[p] : 0.0f, mpv = use_p ? ws.mp[p] : 0.0f;
+      const float d = fmaf(al, ws.w[p], be * pv);
+      const df x = df_add(df{ws.xh[p], ws.xl[p]}, df{d, 0.0f});
+      ws.xh[p] = x.h;
+      ws.xl[p] = x.l;
+      ws.p[p] = d;
+      ws.ap[p] = fmaf(al, aw[p], be * apv);
+      ws.mp[p] = fmaf(al, ws.mw[p], be * mpv);
+    });
+    __syncthreads();
+    have_p = true;
+  }
+  if (!evaluated) residual(true);
+  // normalisation and sign; the integral of a P1 function with zero boundary values is h^2 times the
+  // sum of its nodal values
+  df sacc[1] = {{0.0f, 0.0f}};
+  for_interior(n, [&](int p, int, int) { df_acc(sacc[0], df{ws.xh[p], ws.xl[p]}); });
+  block_sum_df<1>(sacc, red, [&](const df* t) {
+    const double sum = df_double(t[0]);
+    sh->g = fabs(sum) * sh->scale / ((double)n * n);
+    if (sum < 0.0) sh->scale = -sh->scale;
+  });
+  const df sc = df_split(sh->scale);
+  for_interior(n, [&](int p, int, int) {
+    const df v = df_mul(df{ws.xh[p], ws.xl[p]}, sc), x = fast_two_sum(v.h, v.l);
+    ws.xh[p] = x.h;
+    ws.xl[p] = x.l;
+  });
+  __syncthreads();
+  lam = sh->lam;
+  g = sh->g;
+  return conv ? it : -1;
+}
+
+// The coarse eigenvector as the fine solves read it: FP64 values, or double-float pairs.
+struct CoarseVec {
+  const double* d;
+  const float *h, *l;
+  __device__ double operator[](int q) const { return d ? d[q] : (double)h[q] + (double)l[q]; }
+};
+
 // MINRES scalars, owned by thread 0 and read by all threads after each reduction.  The
 // recurrences run in the inner precision T (FP32 on the mixed path), the refinement norms in FP64.
 template <typename T>
@@ -477,7 +800,7 @@ __host__ __device__ inline double residual_target(double tol, double bnorm, doub
 // and refinement steps; flags receives kFlag* bits.
 template <typename T>
 __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int n, const double* __restrict__ a,
-                               const double* __restrict__ rb, const double* uH, int nc, double sigma,
+                               const double* __restrict__ rb, const CoarseVec uH, int nc, double sigma,
                                const SampleLaunch& P, double* red, MinresShared<T>* ms, int& iters, int& outer,
                                int& flags, double& gq) {
   const int ld = n + 1;
@@ -777,6 +1100,8 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
   extern __shared__ __align__(16) char smem_dyn[];
   __shared__ double red[kRedSlots];
   __shared__ EigShared esh;
+  __shared__ Eig32Shared esh32;
+  __shared__ CoarseWS32 cws32;
   __shared__ MinresShared<T> msh;
   __shared__ MinresShared<double> msh64;
   __shared__ CoarseWS cws;
@@ -785,7 +1110,13 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
   char* base = P.use_smem ? smem_dyn : P.gscratch + (size_t)blockIdx.x * P.slab_bytes;
   size_t persist_bytes;
   const bool rxn = P.reaction != 0;
-  {
+  const bool e32 = sizeof(T) == sizeof(float) && P.nc <= kEig32Max;
+  if (e32) {
+    Carver c(base);
+    CoarseWS32 tmp;
+    carve_coarse32(c, P.nc, tmp, &persist_bytes, rxn);
+    if (threadIdx.x == 0) cws32 = tmp;
+  } else {
     Carver c(base);
     CoarseWS tmp;
     carve_coarse(c, P.nc, tmp, &persist_bytes, rxn);
@@ -798,8 +1129,15 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
   const int nchunks = cpr * P.R;
   const size_t ncT = (size_t)2 * nc * nc, nfT = (size_t)2 * P.nf * P.nf, npT = (size_t)2 * P.np * P.np;
   // the persistent coarse eigenvector: zero once (its ring stays zero)
-  zero_vec(cws.uprev, nc);
+  if (e32) {
+    zero_vec(cws32.xh, nc);
+    zero_vec(cws32.xl, nc);
+  } else {
+    zero_vec(cws.uprev, nc);
+  }
   __syncthreads();
+  const CoarseVec uH = e32 ? CoarseVec{nullptr, cws32.xh, cws32.xl} : CoarseVec{cws.uprev, nullptr, nullptr};
+  double lam_prev = 0.0;  // coarse eigenvalue of the previous point of the chain
   const float omega = (float)P.omega;
   for (int ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     const int r = ch / cpr;
@@ -815,7 +1153,16 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
       int eit = 0;
       if (P.u_in) {
         const size_t Vc = gsz(nc);
-        for_all(Vc, [&](size_t q) { cw.uprev[q] = P.u_in[b * Vc + q]; });
+        for_all(Vc, [&](size_t q) {
+          const double v = P.u_in[b * Vc + q];
+          if (e32) {
+            const df d = df_split(v);
+            cws32.xh[q] = d.h;
+            cws32.xl[q] = d.l;
+          } else {
+            cw.uprev[q] = v;
+          }
+        });
         lamH = P.out[b * 4 + 0];
         __syncthreads();
         if (P.qoi && (P.direct_f || (P.np > 0 && P.direct_p && !P.prev_given))) {
@@ -823,12 +1170,48 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
           const double hmc = 1.0 / (12.0 * nc * nc);
           double acc[2] = {0.0, 0.0}, o[2];
           for_interior(nc, [&](int p, int, int) {
-            acc[0] += cw.uprev[p];
-            acc[1] += cw.uprev[p] * hmc * mass7(cw.uprev, p, nc + 1);
+            const int ldc = nc + 1;
+            acc[0] += uH[p];
+            acc[1] += uH[p] * hmc * (6.0 * uH[p] + (uH[p + 1] + uH[p - 1]) + (uH[p + ldc] + uH[p - ldc]) +
+                                     (uH[p + ldc + 1] + uH[p - ldc - 1]));
           });
           block_sum<2, double>(acc, o, red);
           gH = fabs(o[0]) / ((double)nc * nc * sqrt(o[1]));
         }
+      } else if (e32) {
+        // the fine solves of the previous point reused this memory: clear the coarse vectors (the rings
+        // must be zero; interiors are written before use)
+        CoarseWS32& c32 = cws32;
+        float* const vs[8] = {c32.wxl, c32.wyl, c32.r, c32.w, c32.mw, c32.p, c32.ap, c32.mp};
+        for (int i = 0; i < 8; ++i) zero_vec(vs[i], nc);
+        zero_mg(c32.mg);
+        __syncthreads();
+        const double* ac = P.a_c + b * ncT;
+        const double* bc = rxn ? P.b_c + b * ncT : nullptr;
+        if (!build_mg<float>(c32.mg, ac, nc, red, bc, c32.wxl, c32.wyl)) flags |= kFlagBadCoef;
+        if (rxn)
+          reaction_weights<float, double>(nc, bc, bc + (size_t)nc * nc, c32.rx, c32.ry, c32.rd, c32.rxl, c32.ryl, c32.rdl);
+        if (kk == k0) {
+          const float inc = 1.0f / (float)nc;
+          for_interior(nc, [&](int p, int i, int j) {
+            c32.xh[p] = sinpif(i * inc) * sinpif(j * inc);
+            c32.xl[p] = 0.0f;
+          });
+        }
+        __syncthreads();
+        eit = lobpcg32(c32, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh32, kk == k0 ? 20.0 : lam_prev, lamH, gH);
+        lam_prev = lamH;
+        if (eit < 0) flags |= kFlagEigNoConv;
+        if (P.u_out) {
+          for_interior(nc, [&](int p, int i, int j) {
+            P.u_out[b * (size_t)(nc - 1) * (nc - 1) + (j - 1) * (nc - 1) + (i - 1)] = uH[p];
+          });
+        }
+        if (P.u_pad) {
+          const size_t Vc = gsz(nc);
+          for_all(Vc, [&](size_t q) { P.u_pad[b * Vc + q] = uH[(int)q]; });
+        }
+        __syncthreads();
       } else {
         // the fine solves of the previous point reused this memory: clear the coarse vectors
         // (rings must be zero; interiors are written before use)
@@ -881,10 +1264,10 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
       const double* rbp = rxn ? P.b_p + b * npT : nullptr;
       if (!P.direct_f) {
         if (P.mode_f == 0)
-          lf = twogrid_fine<T>(fws, fine_base, P.nf, P.a_f + b * nfT, rbf, cw.uprev, nc, lamH, P, red, &msh, itf, of,
+          lf = twogrid_fine<T>(fws, fine_base, P.nf, P.a_f + b * nfT, rbf, uH, nc, lamH, P, red, &msh, itf, of,
                                flags, gf);
         else if (P.mode_f == 1)
-          lf = twogrid_fine<double>(fws64, fine_base, P.nf, P.a_f + b * nfT, rbf, cw.uprev, nc, lamH, P, red, &msh64,
+          lf = twogrid_fine<double>(fws64, fine_base, P.nf, P.a_f + b * nfT, rbf, uH, nc, lamH, P, red, &msh64,
                                     itf, of, flags, gf);
         if (P.qoi && P.mode_f != 2) lf = gf;
       }
@@ -892,10 +1275,10 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
         lp = P.out[b * 4 + 2];  // every thread reads it before thread 0 rewrites the same value below
       } else if (P.np > 0 && !P.direct_p) {
         if (P.mode_p == 0)
-          lp = twogrid_fine<T>(fws, fine_base, P.np, P.a_p + b * npT, rbp, cw.uprev, nc, lamH, P, red, &msh, itp, op,
+          lp = twogrid_fine<T>(fws, fine_base, P.np, P.a_p + b * npT, rbp, uH, nc, lamH, P, red, &msh, itp, op,
                                flags, gp);
         else if (P.mode_p == 1)
-          lp = twogrid_fine<double>(fws64, fine_base, P.np, P.a_p + b * npT, rbp, cw.uprev, nc, lamH, P, red, &msh64,
+          lp = twogrid_fine<double>(fws64, fine_base, P.np, P.a_p + b * npT, rbp, uH, nc, lamH, P, red, &msh64,
                                     itp, op, flags, gp);
         if (P.qoi && P.mode_p != 2) lp = gp;
       }
