@@ -468,7 +468,8 @@ mq_status mq_apply_operator_device(mq_ctx* ctx, int32_t n, int32_t B, const doub
  * target tol_linear (1e-10 by default), inner reduction per refinement step 1e-5 (mixed) or
  * tol_linear / 10 (FP64), at most 500 inner iterations and 10 (mixed) or 4 (FP64) refinement
  * steps, V(2,2) damped Jacobi (omega 0.8).  A solve on the coarse mesh itself (n_fine or n_prev
- * equal to n_coarse) is nearly singular and uses an FP64 inner solve in either precision.  These
+ * equal to n_coarse) is nearly singular: in mixed precision it is solved for the change of the
+ * eigenvector, and again in FP64 where that does not converge.  These
  * targets are tighter than mq_eval_level's defaults, so on larger coarse meshes a sample can hit
  * the eigensolver cap (flag 1) where mq_eval_level converges.
  *

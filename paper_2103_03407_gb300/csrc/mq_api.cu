@@ -115,6 +115,7 @@ struct mq_ctx {
 
   DevBuf Y, af, ac, ap, out, stat, outer, scratch, sums_d, flags_d, uout, misc, upad, arena, ysl, tc_err;
   DevBuf bf, bc, bp;  // reaction coefficients of the fine, coarse and previous meshes (family 2)
+  DevBuf fscratch;    // per-sample kernel: workspaces of the FP64 fallback solves
   DevBuf tsl, sepw;   // separable evaluation: stage-1 slices, table scratch
   int stream_min = 0;  // fine meshes 1/n with n >= stream_min use the streaming tier (0: default)
   mq_stats stats{};
@@ -483,8 +484,19 @@ bool streams(const mq_ctx* c, const LevelGeom& g) {
   return g.nf >= stream_threshold(c);
 }
 
+// Points per warm-start chain: as long as possible with the chains a multiple of the resident blocks (occ per
+// SM) and at least four per SM, so that uneven chains even out.  Four chains per SM whatever the block
+// size left half of each SM empty on the smallest meshes (64 threads, seven blocks resident), and
+// 1.3 waves of chains where three blocks fit.
+int chunk_for(const mq_ctx* c, int R, int npts, int occ) {
+  const long want = (long)c->sm_count * occ * ((3 + occ) / occ);
+  const long ch = ((long)R * npts + want - 1) / want;
+  return (int)std::max(1L, std::min<long>(ch, 64));
+}
+
 // Runs the per-sample pipeline on B = R * npts samples whose parameters are in c->Y (ldy = s).
-// Writes c->out / c->stat / c->outer; returns timings in stats.  In the reuse scheme, `level`
+// Writes c->out / c->stat / c->outer; returns timings in stats.  chunk: points per warm-start chain, 0 for
+// the default.  In the reuse scheme, `level`
 // and the first point `kbase` of the pass locate the stored level-0 pairs and lower-level values:
 // levels l >= 1 take them instead of solving the coarse problem and the previous-level problem.
 mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk, bool want_u, int level = -1,
@@ -539,12 +551,12 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   mq::SampleLaunch p{};
   // Where each fine solve runs.  A solve on the coarse mesh itself (h = H with a longer
   // truncation) is nearly singular -- lambda_H differs from the fine eigenvalue only by the
-  // truncation -- so it always runs in the per-sample kernel with an FP64 inner solve.
+  // truncation -- so it always runs in the per-sample kernel, which then solves for the change of
+  // the eigenvector instead.
   const bool stream = streams(c, g);
   auto mode_of = [&](int n, bool direct) {
     if (direct || n == 0) return 0;
-    if (n == g.nc) return mixed ? 1 : 0;
-    return stream ? 2 : 0;
+    return stream && n != g.nc ? 2 : 0;
   };
   p.mode_f = mode_of(g.nf, g.direct_f);
   p.mode_p = given ? 0 : mode_of(g.np, g.direct_p);
@@ -557,7 +569,6 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   p.direct_p = g.direct_p;
   p.R = R;
   p.npts = npts;
-  p.chunk = chunk;
   p.a_f = (const double*)c->af.p;
   p.a_c = (const double*)c->ac.p;
   p.a_p = (const double*)c->ap.p;
@@ -623,7 +634,8 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   const int np_k = given ? 0 : g.np;  // the previous-level solve runs here only without the store
   const int in_kernel_n = std::max(p.mode_f != 2 && !g.direct_f ? g.nf : 0, p.mode_p != 2 && !g.direct_p ? np_k : 0);
   const int threads = g.threads > 0 ? g.threads : threads_for(in_kernel_n, g.nc);
-  const size_t slab = mq::sample_slab_bytes(g.nf, g.nc, np_k, mixed, p.mode_f, p.mode_p, p.reaction);
+  const size_t slab = mq::sample_slab_bytes(g.nf, g.nc, np_k, mixed, g.direct_f ? 2 : p.mode_f, g.direct_p ? 2 : p.mode_p,
+                                            p.reaction);
   const int static_smem = mq::sample_static_smem(mixed);
   const size_t smem_cap = (size_t)std::max(0, c->smem_optin - static_smem - 1024);
   const bool use_smem = slab <= smem_cap;
@@ -631,12 +643,24 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   if (use_smem) MQ_CUDA(c, mq::set_sample_smem(mixed, (int)smem));
   int occ = mq::sample_occupancy(mixed, threads, smem);
   if (occ < 1) occ = 1;
+  if (chunk <= 0) chunk = chunk_for(c, R, npts, occ);
+  p.chunk = chunk;
   const int cpr = (npts + chunk - 1) / chunk;
   const long nchunks = (long)cpr * R;
   int blocks = (int)std::min<long>(nchunks, (long)c->sm_count * occ);
   if (blocks < 1) blocks = 1;
+  // global workspaces: of blocks whose own does not fit in shared memory, and of the FP64 solves behind those on
+  // the coarse mesh itself; large ones (fine coarse meshes) get two blocks per SM
+  const bool near = mixed && ((!g.direct_f && g.nf == g.nc) || (np_k == g.nc && !g.direct_p));
+  const size_t fslab = near ? mq::sample_fallback_bytes(g.nc, rxn) : 0;
+  if (((use_smem ? 0 : slab) + fslab) * (size_t)blocks > (size_t)48 << 30) blocks = std::min(blocks, 2 * c->sm_count);
   if (!use_smem) {
     if ((st = grow(c, c->scratch, (size_t)blocks * slab)) != MQ_OK) return st;
+  }
+  if (near) {
+    if ((st = grow(c, c->fscratch, (size_t)blocks * fslab)) != MQ_OK) return st;
+    p.fscratch = (char*)c->fscratch.p;
+    p.fslab_bytes = fslab;
   }
   p.gscratch = (char*)c->scratch.p;
   p.slab_bytes = slab;
@@ -783,13 +807,6 @@ int points_per_pass(const mq_ctx* c, const LevelGeom& g, int R, int npts) {
   return (int)std::min<size_t>(pts, (size_t)npts);
 }
 
-int chunk_for(const mq_ctx* c, int R, int npts) {
-  // points per warm-start chain: enough chains to fill the GPU, chains as long as possible
-  const long want = (long)c->sm_count * 4;
-  long ch = ((long)R * npts + want - 1) / want;
-  return (int)std::max(1L, std::min<long>(ch, 64));
-}
-
 mq_status eval_level_impl(mq_ctx* c, int level, uint32_t k0, uint32_t k1, double* per_sample, double* shift_sums,
                           double* d_per_sample, double* d_shift_sums) {
   mq_status st = check_level_ready(c, level);
@@ -826,7 +843,7 @@ mq_status eval_level_impl(mq_ctx* c, int level, uint32_t k0, uint32_t k1, double
     const int mb = c->mbits[level];
     MQ_LAUNCH(c, mq::launch_lattice_points(c->d_z[level], mb ? (1u << mb) : lv.N, c->d_delta[level], R, g.s, k0 + p0,
                                          pn, mb, (double*)c->Y.p, c->stream, kshift(c)));
-    if ((st = run_samples(c, g, R, pn, chunk_for(c, R, pn), false, level, k0 + p0)) != MQ_OK) return st;
+    if ((st = run_samples(c, g, R, pn, 0, false, level, k0 + p0)) != MQ_OK) return st;
     if (c->reuse) {
       const mq_level& l0 = c->levels[0];
       const size_t V0 = (size_t)(l0.n_fine + 1) * (l0.n_fine + 1);
@@ -971,7 +988,7 @@ mq_status mq_destroy(mq_ctx* c) {
     if (b->p) cudaFree(b->p);
   for (DevBuf* b : {&c->Y, &c->af, &c->ac, &c->ap, &c->out, &c->stat, &c->outer, &c->scratch, &c->sums_d,
                     &c->flags_d, &c->uout, &c->misc, &c->upad, &c->arena, &c->ysl, &c->tc_err, &c->bf, &c->bc,
-                    &c->bp, &c->tsl, &c->sepw})
+                    &c->bp, &c->tsl, &c->sepw, &c->fscratch})
     if (b->p) cudaFree(b->p);
   release_tables(c);
   free_reuse(c);

@@ -150,7 +150,8 @@ __device__ __forceinline__ void for_all(size_t count, F f) {
 }
 
 // size of the shared reduction buffer every block_sum caller must provide
-constexpr int kRedSlots = 32 * 12 + 12;
+constexpr int kRedWarps = 16;  // warps of the largest block (512 threads)
+constexpr int kRedSlots = kRedWarps * 12 + 12;
 
 struct NoEp {
   __device__ void operator()(const double*) const {}
@@ -197,13 +198,13 @@ template <int NV, typename A, class Ep = NoEp>
 __device__ __forceinline__ void block_sum(A (&v)[NV], double (&out)[NV], double* red, Ep ep = Ep(),
                                           int nact = 1 << 30) {
   static_assert(NV <= 12, "block_sum reduces at most 12 values");
-  // red: kRedSlots doubles = 32 * 12 partial slots followed by 12 total slots.  The totals never
+  // red: kRedSlots doubles = kRedWarps * 12 partial slots followed by 12 total slots.  The totals never
   // overlap the partials, so two barriers suffice: the next call writes partials only after
   // passing this call's second barrier, and writes totals only after its own first barrier
   // (every thread has read ours).
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = min((int)(blockDim.x >> 5), (nact + 31) >> 5);
-  double* tot = red + 32 * 12;
+  double* tot = red + kRedWarps * 12;
   if (wid < nw) {
     int base = 0, c = NV;
     Butterfly<NV, 16, A>::run(v, lane, base, c);

@@ -26,6 +26,8 @@ struct SampleLaunch {
   double* u_out;           // NULL or [B][(nc-1)^2] coarse eigenvectors
   char* gscratch;          // per-CTA workspace slabs when they do not fit in shared memory
   size_t slab_bytes;
+  char* fscratch;          // NULL, or per-CTA workspaces of the FP64 fallback of solves on the coarse mesh itself
+  size_t fslab_bytes;      // (sample_fallback_bytes; FP32 kernel only)
   int use_smem;
   double tol_eig;
   int max_eig_it;
@@ -40,8 +42,7 @@ struct SampleLaunch {
   const double* u_in;      // NULL or [B][(nc+1)^2]: coarse pairs given (no coarse eigensolve), with
                            // lambda_H in out[b][0] (the reuse scheme across levels)
   int prev_given;          // lambda^{l-1} given in out[b][2] (no previous-level solve)
-  int mode_f, mode_p;      // fine / previous-fine solve: 0 in the kernel (inner precision T),
-                           // 1 in the kernel with an FP64 inner solve, 2 elsewhere (streaming)
+  int mode_f, mode_p;      // fine / previous-fine solve: 0 in the kernel, 2 elsewhere (streaming)
   int reaction;            // the operator has a reaction term b u (b_f, b_c, b_p hold b)
   const double* b_f;       // [B][2 nf^2] centroid values of the reaction coefficient, like a_f
   const double* b_c;
@@ -152,6 +153,7 @@ enum : int {
 };
 
 size_t sample_slab_bytes(int nf, int nc, int np, int mixed);
+size_t sample_fallback_bytes(int n, int reaction);
 size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int mode_f, int mode_p, int reaction = 0);
 cudaError_t launch_sample(const SampleLaunch& p, int mixed, int blocks, int threads, size_t smem,
                           cudaStream_t st);

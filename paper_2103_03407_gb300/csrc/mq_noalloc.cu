@@ -91,14 +91,13 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   if (B == 0) return MQ_OK;
   if (!d_a_coarse || !d_out || !d_stat || !d_outer) return MQ_EINVAL;
   const int mixed = precision == MQ_PREC_MIXED;
-  // A solve on the coarse mesh itself (n == n_coarse with a longer truncation) is nearly
-  // singular -- the shift is an eigenvalue of a nearby operator -- so in mixed precision it runs
-  // with an FP64 inner solve (mode 1), as in mq_eval_level; every other solve uses the inner
-  // precision of the mode (mode 0).  The workspace is sized for the modes actually used.
-  const int mode_f = (mixed && n_fine == n_coarse && d_a_fine) ? 1 : 0;
-  const int mode_p = (mixed && n_prev == n_coarse && d_a_prev) ? 1 : 0;
+  // the workspace is sized for the solves performed (mode 2: none)
+  const int mode_f = d_a_fine ? 0 : 2, mode_p = d_a_prev ? 0 : 2;
   const size_t slab = mq::sample_slab_bytes(n_fine, n_coarse, n_prev, mixed, mode_f, mode_p);
-  if (slab > kNoAllocScratchBytes) return MQ_EINVAL;  // one block's workspace exceeds the fixed array
+  // a solve on the coarse mesh itself may fall back to FP64 (see mq_sample.cu)
+  const bool near = mixed && ((d_a_fine && n_fine == n_coarse) || (d_a_prev && n_prev == n_coarse));
+  const size_t fslab = near ? mq::sample_fallback_bytes(n_coarse, 0) : 0;
+  if (slab + fslab > kNoAllocScratchBytes) return MQ_EINVAL;  // one block's workspace exceeds the fixed array
 
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kMaxDevices) return MQ_ECUDA;
@@ -110,7 +109,7 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   const int threads = n_fine <= 16 ? 128 : 256;
   int occ = mq::sample_occupancy(mixed, threads, 0);
   if (occ < 1) occ = 1;
-  const long fit = (long)(kNoAllocScratchBytes / slab);
+  const long fit = (long)(kNoAllocScratchBytes / (slab + fslab));
   const long blocks = std::max(1L, std::min<long>({(long)B, (long)sms * occ, fit}));
   const int chunk = (int)((B + blocks - 1) / blocks);
 
@@ -132,6 +131,8 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   p.u_out = nullptr;
   p.gscratch = (char*)scratch;
   p.slab_bytes = slab;
+  p.fscratch = near ? (char*)scratch + (size_t)blocks * slab : nullptr;
+  p.fslab_bytes = fslab;
   p.use_smem = 0;
   p.tol_eig = 1e-12;
   p.max_eig_it = 200;
@@ -141,8 +142,6 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   p.max_inner_it = 500;
   p.nu = 2;
   p.omega = 0.8;
-  p.mode_f = mode_f;
-  p.mode_p = mode_p;
   const cudaError_t e = mq::launch_sample(p, mixed, (int)blocks, threads, 0, (cudaStream_t)cuda_stream);
   return e == cudaSuccess ? MQ_OK : MQ_ECUDA;
 }

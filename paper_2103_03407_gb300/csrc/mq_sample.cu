@@ -116,11 +116,14 @@ __host__ __device__ void carve_coarse32(Carver& c, int nc, CoarseWS32& ws, size_
   ws.mg.rcell[1] = reaction ? c.take<float>((size_t)nc * nc / 2 + 1) : nullptr;
 }
 
-// Fine shifted-solve workspace: FP64 solution and right-hand side, inner vectors in T.
+// Fine shifted-solve workspace: solution and right-hand side beyond FP32, inner vectors in T.
 template <typename T>
 struct FineWS {
   MGDesc<T> mg;
-  double *x64, *b64;
+  double *x64, *b64;  // FP64 kernel
+  // FP32 kernel: solution and right-hand side as double-floats, the low parts of the edge weights (and of
+  // the reaction's)
+  float *xh, *xl, *bh, *bl, *wxl, *wyl, *rxl, *ryl, *rdl;
   T *vo, *v, *z, *zn, *wo, *w, *q, *xi;
   T *rx, *ry, *rd;  // reaction edge weights in the inner precision (NULL without a reaction term)
 };
@@ -128,8 +131,13 @@ struct FineWS {
 template <typename T>
 __host__ __device__ void carve_fine(Carver& c, int n, FineWS<T>& ws, bool reaction = false) {
   const size_t V = gsz(n);
-  ws.x64 = c.take<double>(V);
-  ws.b64 = c.take<double>(V);
+  const bool f32 = sizeof(T) == sizeof(float);
+  ws.x64 = f32 ? nullptr : c.take<double>(V);
+  ws.b64 = f32 ? nullptr : c.take<double>(V);
+  float** const pr[6] = {&ws.xh, &ws.xl, &ws.bh, &ws.bl, &ws.wxl, &ws.wyl};
+  for (float** v : pr) *v = f32 ? c.take<float>(V) : nullptr;
+  float** const rl[3] = {&ws.rxl, &ws.ryl, &ws.rdl};
+  for (float** v : rl) *v = f32 && reaction ? c.take<float>(V) : nullptr;
   ws.vo = c.take<T>(V);
   ws.v = c.take<T>(V);
   ws.z = c.take<T>(V);
@@ -154,8 +162,7 @@ __host__ __device__ size_t fine_bytes(int n, bool reaction = false) {
 }
 
 // workspace of one CTA: the persistent head, then the larger of the rest of the coarse region
-// and the largest fine solve it performs in place (mode 0: inner precision T, mode 1: FP64 inner
-// solve, 2: not in this kernel).  A multiple of 256 bytes: the slabs of a global scratch lie back
+// and the largest fine solve it performs in place (mode 2: not in this kernel).  A multiple of 256 bytes: the slabs of a global scratch lie back
 // to back, so every slab then starts as aligned as the scratch itself and the kernel carves it
 // exactly as sized here (an unaligned slab start would shift its arrays by up to 15 bytes into
 // the next slab).
@@ -173,8 +180,9 @@ __host__ __device__ size_t slab_size(int nf, int nc, int np, int mode_f = 0, int
   persist = (persist + 15) & ~(size_t)15;  // the fine region starts 16-byte aligned
   const size_t coarse = (c.used() + 15) & ~(size_t)15;
   auto need = [&](int n, int mode) -> size_t {
-    if (mode == 2) return 0;
-    return mode == 1 ? fine_bytes<double>(n, reaction) : fine_bytes<T>(n, reaction);
+    // (the FP32 kernel's FP64 solve on a large coarse mesh itself has its own workspace)
+    if (mode == 2 || (sizeof(T) == sizeof(float) && n == nc && nc > kEig32Max)) return 0;
+    return fine_bytes<T>(n, reaction);
   };
   size_t m = coarse - persist;
   const size_t a = need(nf, mode_f), b = need(np, mode_p);
@@ -487,7 +495,7 @@ template <int NV, class Ep>
 __device__ __forceinline__ void block_sum_df(df (&v)[NV], double* red, Ep ep) {
   static_assert(NV <= 12, "block_sum_df reduces at most 12 values");
   df* part = reinterpret_cast<df*>(red);
-  df* tot = part + 32 * 12;
+  df* tot = part + kRedWarps * 12;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int base = 0, c = NV;
   DfButterfly<NV, 16>::run(v, lane, base, c);
@@ -508,6 +516,26 @@ __device__ __forceinline__ void block_sum_df(df (&v)[NV], double* red, Ep ep) {
     }
   }
   __syncthreads();
+}
+
+// 12 / h^2 times the reaction's value at node p, 2 x sum r_q - sum r_q d_q over the six neighbours, from the
+// edge weights r (pairs) and the differences d_q = x_p - x_q
+__device__ __forceinline__ df reaction_df(const float* rx, const float* ry, const float* rd, const float* rxl,
+                                          const float* ryl, const float* rdl, int p, int ld, df x, df dE, df dW, df dN,
+                                          df dS, df dNE, df dSW) {
+  const df w[6] = {{rx[p], rxl[p]},           {rx[p - 1], rxl[p - 1]}, {ry[p], ryl[p]},
+                   {ry[p - ld], ryl[p - ld]}, {rd[p], rdl[p]},         {rd[p - ld - 1], rdl[p - ld - 1]}};
+  const df d[6] = {dE, dW, dN, dS, dNE, dSW};
+  df rs = {0.0f, 0.0f}, rdq = {0.0f, 0.0f};
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    df_acc(rs, w[k]);
+    df_acc(rdq, df_mul(w[k], d[k]));
+  }
+  rs = fast_two_sum(rs.h, rs.l);
+  df bx = df_mul(rs, df{2.0f * x.h, 2.0f * x.l});
+  df_acc(bx, df_neg(rdq));
+  return fast_two_sum(bx.h, bx.l);
 }
 
 struct Eig32Shared {
@@ -610,25 +638,8 @@ __device__ __noinline__ int lobpcg32(CoarseWS32& ws, int n, double tol, int maxi
       df_acc(s6, dNE);
       df_acc(s6, dSW);
       s6 = fast_two_sum(s6.h, s6.l);
-      if (ws.rx) {
-        // h^2/12 (2 x sum r_q - sum r_q d_q)
-        const int q[6] = {p, p - 1, p, p - ld, p, p - ld - 1};
-        const float* const h[6] = {ws.rx, ws.rx, ws.ry, ws.ry, ws.rd, ws.rd};
-        const float* const l[6] = {ws.rxl, ws.rxl, ws.ryl, ws.ryl, ws.rdl, ws.rdl};
-        const df d[6] = {dE, dW, dN, dS, dNE, dSW};
-        df rs = {0.0f, 0.0f}, rdq = {0.0f, 0.0f};
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          const df w = {h[k][q[k]], l[k][q[k]]};
-          df_acc(rs, w);
-          df_acc(rdq, df_mul(w, d[k]));
-        }
-        rs = fast_two_sum(rs.h, rs.l);
-        df bx = df_mul(rs, df{2.0f * x.h, 2.0f * x.l});
-        df_acc(bx, df_neg(rdq));
-        bx = fast_two_sum(bx.h, bx.l);
-        df_acc(r, df_mul(hmd, bx));
-      }
+      if (ws.rx)
+        df_acc(r, df_mul(hmd, reaction_df(ws.rx, ws.ry, ws.rd, ws.rxl, ws.ryl, ws.rdl, p, ld, x, dE, dW, dN, dS, dNE, dSW)));
       df_acc(r, df_neg(df_mul(c2, x)));
       df_acc(r, df_mul(c12, s6));
       r = fast_two_sum(r.h, r.l);
@@ -760,11 +771,14 @@ __device__ __noinline__ int lobpcg32(CoarseWS32& ws, int n, double tol, int maxi
   return conv ? it : -1;
 }
 
+constexpr int kNearInner = 24;  // MINRES iterations per correction of a solve on the coarse mesh itself
+
 // The coarse eigenvector as the fine solves read it: FP64 values, or double-float pairs.
 struct CoarseVec {
   const double* d;
   const float *h, *l;
   __device__ double operator[](int q) const { return d ? d[q] : (double)h[q] + (double)l[q]; }
+  __device__ df pair(int q) const { return d ? df_split(d[q]) : df{h[q], l[q]}; }
 };
 
 // MINRES scalars, owned by thread 0 and read by all threads after each reduction.  The
@@ -781,6 +795,7 @@ struct MinresShared {
   double knorm, xnorm;  // ||A - sigma M|| bound and ||x|| for the FP64 residual floor
   double xax, xmx;      // x.Ax and x.Mx of the last FP64 residual pass (the Rayleigh quotient)
   double xsum;          // sum of the nodal values of x in that pass (h^2 xsum = integral of x)
+  double tau;           // factor of the right-hand side (1 except in a solve on the coarse mesh itself)
   int done, breakdown;
 };
 
@@ -803,6 +818,9 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
                                const double* __restrict__ rb, const CoarseVec uH, int nc, double sigma,
                                const SampleLaunch& P, double* red, MinresShared<T>* ms, int& iters, int& outer,
                                int& flags, double& gq) {
+  constexpr bool kF32 = sizeof(T) == sizeof(float);
+  // A solve on the coarse mesh itself (a longer truncation on the mesh of the coarse pair): see `near` below
+  const bool near = kF32 && n == nc;
   const int ld = n + 1;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -811,8 +829,13 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
   }
   __syncthreads();
   const double hm = 1.0 / (12.0 * n * n);
-  zero_vec(ws.x64, n);
-  zero_vec(ws.b64, n);
+  if constexpr (kF32) {
+    float* const pr[4] = {ws.xh, ws.xl, ws.bh, ws.bl};
+    for (float* v : pr) zero_vec(v, n);
+  } else {
+    zero_vec(ws.x64, n);
+    zero_vec(ws.b64, n);
+  }
   zero_vec(ws.vo, n);
   zero_vec(ws.v, n);
   zero_vec(ws.z, n);
@@ -828,23 +851,29 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
   }
   zero_mg(ws.mg);
   __syncthreads();
-  if (!build_mg<T>(ws.mg, a, n, red, rb)) flags |= kFlagBadCoef;
-  if (rb) reaction_weights<T, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd);
+  if constexpr (kF32) {
+    if (!build_mg<T>(ws.mg, a, n, red, rb, ws.wxl, ws.wyl)) flags |= kFlagBadCoef;
+    if (rb)
+      reaction_weights<T, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd, ws.rxl, ws.ryl, ws.rdl);
+  } else {
+    if (!build_mg<T>(ws.mg, a, n, red, rb)) flags |= kFlagBadCoef;
+    if (rb) reaction_weights<T, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd);
+  }
   {
     // ||A + B - sigma M||_inf <= 8 max a + (max b + sigma) h^2 (row sums of the edge form, of the
-    // reaction and of the mass)
-    double amax = 0.0, bmax = 0.0;
+    // reaction and of the mass); positive doubles order as their bit patterns (integer units)
+    long long amax = 0, bmax = 0;
     for_all((size_t)2 * n * n, [&](size_t q) {
-      amax = fmax(amax, a[q]);
-      if (rb) bmax = fmax(bmax, rb[q]);
+      amax = max(amax, __double_as_longlong(a[q]));
+      if (rb) bmax = max(bmax, __double_as_longlong(rb[q]));
     });
     for (int off = 16; off > 0; off >>= 1) {
-      amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-      bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
+      amax = max(amax, (long long)__shfl_xor_sync(0xffffffffu, amax, off));
+      bmax = max(bmax, (long long)__shfl_xor_sync(0xffffffffu, bmax, off));
     }
     if ((threadIdx.x & 31) == 0) {
-      red[threadIdx.x >> 5] = amax;
-      red[32 + (threadIdx.x >> 5)] = bmax;
+      red[threadIdx.x >> 5] = __longlong_as_double(amax);
+      red[32 + (threadIdx.x >> 5)] = __longlong_as_double(bmax);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -856,22 +885,108 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
       ms->knorm = 8.0 * m + (mb + sigma) / ((double)n * n);
       ms->xnorm = 0.0;
       ms->xax = ms->xmx = 0.0;
+      ms->tau = 1.0;
     }
     __syncthreads();
   }
-  // FP64 operator for the residual and the Rayleigh quotient: the FP64 weights of level 0 when the
-  // inner precision is FP64, otherwise weights formed on the fly from the centroid coefficients
-  const bool w64 = sizeof(T) == sizeof(double);
+  // FP64 kernel: the operator of the residual from the FP64 weights of level 0
   const double* wx64 = (const double*)ws.mg.wx[0];
   const double* wy64 = (const double*)ws.mg.wy[0];
-  auto K64 = [&](const double* x, int p, int i, int j) {
-    double k = w64 ? stiff<double, double>(wx64, wy64, x, p, ld) : stiff_cells(a, n, x, p, ld, i, j);
-    if (rb)
-      k += hm * (w64 ? react7<double, double>((const double*)ws.rx, (const double*)ws.ry, (const double*)ws.rd, x, p, ld)
-                     : react_cells(rb, n, x, p, ld, i, j));
+  auto K64 = [&](const double* x, int p) {
+    double k = stiff<double, double>(wx64, wy64, x, p, ld);
+    if (rb) k += hm * react7<double, double>((const double*)ws.rx, (const double*)ws.ry, (const double*)ws.rd, x, p, ld);
     return k;
   };
-  // b = M P u_H  (P: P1 interpolation from the nested coarse mesh); x64 holds P u_H for a moment
+  const df hmd = {(float)hm, (float)(hm - (double)(float)hm)};
+  // FP32 kernel: the residual of the current x in double-floats (as the streaming tier's: see k_residual4), and
+  // with it x.Kx, x.x, x.S6 and sum x.  With `near` the right-hand side is tau b with tau = x.Kx / x.b,
+  // r orthogonal to x: a solve on the coarse mesh itself has its shift at an eigenvalue
+  // of a nearby operator, K w = b a solution w that is almost a multiple of u_H and may be
+  // arbitrarily long, and only its direction matters.  Written as w = (u_H + v) / tau the unknown
+  // v is as small as the change of the coefficient, and FP32 corrections converge for any distance
+  // of the shift from the eigenvalue (x soon is the near-null direction itself, and r orthogonal
+  // to it leaves that direction out of the correction).  The residual of w relative to ||b|| is ||tau b - K (u_H + v)|| / (|tau| ||b||).
+  auto residual32 = [&](bool first_pass) {
+    if constexpr (kF32) {
+      const double c12d = sigma / ((double)n * n);
+      const df c12 = df_split(c12d), cs = df_split(sigma * hm);
+      df acc[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) acc[k] = {0.0f, 0.0f};
+      const float* __restrict__ wxh = (const float*)ws.mg.wx[0];
+      const float* __restrict__ wyh = (const float*)ws.mg.wy[0];
+      for_interior(n, [&](int p, int, int) {
+        auto X = [&](int q) { return df{ws.xh[q], ws.xl[q]}; };
+        const df x = X(p);
+        const df dE = df_sub(x, X(p + 1)), dW = df_sub(x, X(p - 1)), dN = df_sub(x, X(p + ld)), dS = df_sub(x, X(p - ld));
+        const df dNE = df_sub(x, X(p + ld + 1)), dSW = df_sub(x, X(p - ld - 1));
+        df k = df_mul(df{wxh[p], ws.wxl[p]}, dE);
+        df_acc(k, df_mul(df{wxh[p - 1], ws.wxl[p - 1]}, dW));
+        df_acc(k, df_mul(df{wyh[p], ws.wyl[p]}, dN));
+        df_acc(k, df_mul(df{wyh[p - ld], ws.wyl[p - ld]}, dS));
+        df s6 = dE;
+        df_acc(s6, dW);
+        df_acc(s6, dN);
+        df_acc(s6, dS);
+        df_acc(s6, dNE);
+        df_acc(s6, dSW);
+        s6 = fast_two_sum(s6.h, s6.l);
+        if (ws.rx) df_acc(k, df_mul(hmd, reaction_df(ws.rx, ws.ry, ws.rd, ws.rxl, ws.ryl, ws.rdl, p, ld, x, dE, dW, dN, dS, dNE, dSW)));
+        df_acc(k, df_neg(df_mul(c12, x)));
+        df_acc(k, df_mul(cs, s6));
+        k = fast_two_sum(k.h, k.l);
+        const df bv = {ws.bh[p], ws.bl[p]};
+        if (near) {
+          ws.q[p] = k.h;
+          ws.vo[p] = k.l;
+          df_acc(acc[5], df_mul(bv, x));
+        } else {
+          df r = bv;
+          df_acc(r, df_neg(k));
+          const float rf = r.h + r.l;
+          ws.v[p] = rf;
+          acc[0].h = fmaf(rf, rf, acc[0].h);
+        }
+        df_acc(acc[1], df_mul(x, x));
+        df_acc(acc[2], df_mul(x, k));
+        df_acc(acc[3], df_mul(x, s6));
+        df_acc(acc[4], x);
+      });
+      auto finish = [&](double rr) {
+        const double rnew = sqrt(rr);
+        // no progress: stop refining (not after the first step, whose FP32 rounding noise can
+        // leave a residual above ||b|| on fine meshes)
+        ms->done = !first_pass && outer > 0 && !(rnew < 0.5 * ms->rnorm);
+        ms->rnorm = rnew;
+        ms->rs = T(1.0 / rnew);
+      };
+      block_sum_df<6>(acc, red, [&](const df* t) {
+        const double x2 = df_double(t[1]), xk = df_double(t[2]), x6 = df_double(t[3]);
+        ms->xnorm = sqrt(x2);
+        ms->xmx = (x2 - x6 / 12.0) / ((double)n * n);
+        ms->xax = xk + sigma * ms->xmx;
+        ms->xsum = df_double(t[4]);
+        if (near)
+          ms->tau = xk / df_double(t[5]);
+        else
+          finish(df_double(t[0]));
+      });
+      if (near) {
+        const df tau = df_split(ms->tau);
+        df acc1[1] = {{0.0f, 0.0f}};
+        for_interior(n, [&](int p, int, int) {
+          df r = df_mul(tau, df{ws.bh[p], ws.bl[p]});
+          df_acc(r, df{-ws.q[p], -ws.vo[p]});
+          const float rf = r.h + r.l;
+          ws.v[p] = rf;
+          acc1[0].h = fmaf(rf, rf, acc1[0].h);
+        });
+        block_sum_df<1>(acc1, red, [&](const df* t) { finish(df_double(t[0])); });
+      }
+    }
+  };
+  // b = M P u_H  (P: P1 interpolation from the nested coarse mesh); x holds P u_H for a moment (with `near`
+  // it stays there)
   {
     const int lr = ilog2(n / nc);
     const int rm = (1 << lr) - 1;
@@ -879,32 +994,73 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
     const double inv = 1.0 / (double)(1 << lr);
     for_interior(n, [&](int p, int i, int j) {
       const int I = i >> lr, J = j >> lr;
-      const double xi_ = (double)(i & rm) * inv, et = (double)(j & rm) * inv;
       const int c0 = J * ldc + I;
-      double v;
-      if (xi_ >= et)
-        v = (1.0 - xi_) * uH[c0] + (xi_ - et) * uH[c0 + 1] + et * uH[c0 + ldc + 1];
-      else
-        v = (1.0 - et) * uH[c0] + (et - xi_) * uH[c0 + ldc] + xi_ * uH[c0 + ldc + 1];
-      ws.x64[p] = v;
+      if constexpr (kF32) {
+        const int ki = i & rm, kj = j & rm;
+        const bool lower = ki >= kj;
+        const df u00 = uH.pair(c0), u11 = uH.pair(c0 + ldc + 1), uc = uH.pair(lower ? c0 + 1 : c0 + ldc);
+        const float s1 = (float)(lower ? ki : kj) * (float)inv, s2 = (float)(lower ? kj : ki) * (float)inv;
+        const df v = df_add(df_add(u00, df_mul(df_sub(uc, u00), s1)), df_mul(df_sub(u11, uc), s2));
+        ws.xh[p] = v.h;
+        ws.xl[p] = v.l;
+      } else {
+        const double xi_ = (double)(i & rm) * inv, et = (double)(j & rm) * inv;
+        double v;
+        if (xi_ >= et)
+          v = (1.0 - xi_) * uH[c0] + (xi_ - et) * uH[c0 + 1] + et * uH[c0 + ldc + 1];
+        else
+          v = (1.0 - et) * uH[c0] + (et - xi_) * uH[c0 + ldc] + xi_ * uH[c0 + ldc + 1];
+        ws.x64[p] = v;
+      }
     });
     __syncthreads();
     double acc[1] = {0.0}, o[1];
+    float acc32[1] = {0.0f};
     for_interior(n, [&](int p, int, int) {
-      const double bv = hm * mass7(ws.x64, p, ld);
-      ws.b64[p] = bv;
-      ws.v[p] = T(bv);
-      acc[0] += bv * bv;
+      if constexpr (kF32) {
+        df m = df_mul(df{ws.xh[p], ws.xl[p]}, 6.0f);
+        const int q[6] = {p + 1, p - 1, p + ld, p - ld, p + ld + 1, p - ld - 1};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) df_acc(m, df{ws.xh[q[k]], ws.xl[q[k]]});
+        df bv = df_mul(m, hmd);
+        bv = fast_two_sum(bv.h, bv.l);
+        ws.bh[p] = bv.h;
+        ws.bl[p] = bv.l;
+        ws.v[p] = bv.h;
+        acc32[0] = fmaf(bv.h, bv.h, acc32[0]);
+      } else {
+        const double bv = hm * mass7(ws.x64, p, ld);
+        ws.b64[p] = bv;
+        ws.v[p] = T(bv);
+        acc[0] += bv * bv;
+      }
     });
-    block_sum<1, double>(acc, o, red, [&](const double* t) {
+    auto start = [&](const double* t) {
       ms->bnorm = ms->rnorm = sqrt(t[0]);
       ms->rs = T(1.0 / ms->rnorm);
-    });
-    for_interior(n, [&](int p, int, int) { ws.x64[p] = 0.0; });
-    __syncthreads();
+    };
+    if constexpr (kF32)
+      block_sum<1, float>(acc32, o, red, start);
+    else
+      block_sum<1, double>(acc, o, red, start);
+    if (!near) {
+      for_interior(n, [&](int p, int, int) {
+        if constexpr (kF32)
+          ws.xh[p] = ws.xl[p] = 0.0f;
+        else
+          ws.x64[p] = 0.0;
+      });
+      __syncthreads();
+    } else {
+      residual32(true);
+    }
   }
   outer = 0;
   iters = 0;
+  // with the shift within FP32 rounding of the eigenvalue, a correction cannot reduce what r has along the
+  // near-null direction before x has turned into it: such solves end early and the next one goes on
+  const bool early = near && P.max_inner_it > kNearInner;
+  const int max_inner = early ? kNearInner : P.max_inner_it;
   const T sigm = T(sigma * hm);
   const T hmt = T(hm);
   const T om = T(P.omega);
@@ -914,7 +1070,7 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
   const T* try_ = ws.ry;
   const T* trd = ws.rd;
   for (; outer < P.max_outer; ++outer) {
-    if (!(ms->rnorm > residual_target(P.tol_lin, ms->bnorm, ms->knorm, ms->xnorm, 16.0))) break;
+    if (!(ms->rnorm > residual_target(P.tol_lin, fabs(ms->tau) * ms->bnorm, ms->knorm, ms->xnorm, 16.0))) break;
     // inner: MINRES on (A - sigma M) xi = r / ||r|| in precision T, preconditioned by the V-cycle;
     // v holds r (unscaled)
     const T rs = ms->rs;
@@ -954,7 +1110,7 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
     }
     int j = 0;
     bool pending = false;
-    for (; j < P.max_inner_it && !ms->done; ++j) {
+    for (; j < max_inner && !ms->done; ++j) {
       // [pending w/x update of the previous iteration] + q = K z / gamma, delta
       {
         T acc1[1] = {T(0)};
@@ -1047,66 +1203,81 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
     }
     iters += j;
     if (ms->breakdown) flags |= kFlagBreakdown;
-    if (!ms->done) flags |= kFlagLinNoConv;
-    // x64 += ||r|| xi ; r = b - (A - sigma M) x64 in FP64, stored (unscaled) in v
+    if (!ms->done && !early) flags |= kFlagLinNoConv;
+    // x += ||r|| xi ; r = b - (A - sigma M) x beyond FP32, stored (unscaled) in v.  The same pass forms x.Ax,
+    // x.Mx and sum(x): the last one gives the Rayleigh quotient and the functional of the result
     const double rn = ms->rnorm;
-    for_interior(n, [&](int p, int, int) { ws.x64[p] += rn * (double)ws.xi[p]; });
-    __syncthreads();
-    // the same pass forms x.Ax, x.Mx and sum(x): the last one gives the Rayleigh quotient and the
-    // functional of the result
-    double acc2[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, o2[5];
-    for_interior(n, [&](int p, int i, int j) {
-      const double xv = ws.x64[p];
-      const double ax = K64(ws.x64, p, i, j);
-      const double mx = hm * mass7(ws.x64, p, ld);
-      const double rv = ws.b64[p] - (ax - sigma * mx);
-      ws.v[p] = T(rv);
-      acc2[0] += rv * rv;
-      acc2[1] += xv * xv;
-      acc2[2] += xv * ax;
-      acc2[3] += xv * mx;
-      acc2[4] += xv;
-    });
-    int stalled = 0;
-    const int first = outer == 0;
-    block_sum<5, double>(acc2, o2, red, [&](const double* t) {
-      const double rnew = sqrt(t[0]);
-      ms->xnorm = sqrt(t[1]);
-      ms->xax = t[2];
-      ms->xmx = t[3];
-      ms->xsum = t[4];
-      // no progress: stop refining (not after the first step, whose FP32 rounding noise can
-      // leave a residual above ||b|| on fine meshes)
-      ms->done = !first && !(rnew < 0.5 * ms->rnorm);
-      ms->rnorm = rnew;
-      ms->rs = T(1.0 / rnew);
-    });
-    stalled = ms->done;
+    if constexpr (kF32) {
+      const df rnd = df_split(rn);
+      for_interior(n, [&](int p, int, int) {
+        const df x = df_add(df{ws.xh[p], ws.xl[p]}, df_mul(rnd, ws.xi[p]));
+        ws.xh[p] = x.h;
+        ws.xl[p] = x.l;
+      });
+      __syncthreads();
+      residual32(false);
+    } else {
+      for_interior(n, [&](int p, int, int) { ws.x64[p] += rn * (double)ws.xi[p]; });
+      __syncthreads();
+      double acc2[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, o2[5];
+      for_interior(n, [&](int p, int, int) {
+        const double xv = ws.x64[p];
+        const double ax = K64(ws.x64, p);
+        const double mx = hm * mass7(ws.x64, p, ld);
+        const double rv = ws.b64[p] - (ax - sigma * mx);
+        ws.v[p] = T(rv);
+        acc2[0] += rv * rv;
+        acc2[1] += xv * xv;
+        acc2[2] += xv * ax;
+        acc2[3] += xv * mx;
+        acc2[4] += xv;
+      });
+      const int first = outer == 0;
+      block_sum<5, double>(acc2, o2, red, [&](const double* t) {
+        const double rnew = sqrt(t[0]);
+        ms->xnorm = sqrt(t[1]);
+        ms->xax = t[2];
+        ms->xmx = t[3];
+        ms->xsum = t[4];
+        // no progress: stop refining (not after the first step, whose FP32 rounding noise can
+        // leave a residual above ||b|| on fine meshes)
+        ms->done = !first && !(rnew < 0.5 * ms->rnorm);
+        ms->rnorm = rnew;
+        ms->rs = T(1.0 / rnew);
+      });
+    }
+    const int stalled = ms->done;
     if (stalled) {
       ++outer;
       break;
     }
   }
   // flagged only well above the target (or the FP64 floor): the refinement may stop a little short
-  if (!(ms->rnorm <= residual_target(fmax(1e-5, 10.0 * P.tol_lin), ms->bnorm, ms->knorm, ms->xnorm, 256.0)))
+  if (!(ms->rnorm <= residual_target(fmax(1e-5, 10.0 * P.tol_lin), fabs(ms->tau) * ms->bnorm, ms->knorm, ms->xnorm, 256.0)))
     flags |= kFlagLinNoConv;
   // Rayleigh quotient and functional in FP64, from the residual pass over the final iterate
   gq = fabs(ms->xsum) / ((double)n * n * sqrt(ms->xmx));
   return ms->xax / ms->xmx;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
+// MAXT: threads per block at most.  Up to 256 threads the FP32 kernel is compiled for three blocks of 256 per SM (80
+// registers): its phases are short and end in block-wide barriers, which other blocks then fill.
+template <typename T, int MAXT>
+__global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 256 ? 3 : 1) sample_kernel(SampleLaunch P) {
   extern __shared__ __align__(16) char smem_dyn[];
   __shared__ double red[kRedSlots];
   __shared__ EigShared esh;
   __shared__ Eig32Shared esh32;
-  __shared__ CoarseWS32 cws32;
   __shared__ MinresShared<T> msh;
-  __shared__ MinresShared<double> msh64;
-  __shared__ CoarseWS cws;
+  // one of the two coarse workspaces is in use (e32 below)
+  __shared__ union CoarseBoth {
+    CoarseWS f64;
+    CoarseWS32 f32;
+    __device__ CoarseBoth() {}
+  } both;
+  CoarseWS& cws = both.f64;
+  CoarseWS32& cws32 = both.f32;
   __shared__ FineWS<T> fws;
-  __shared__ FineWS<double> fws64;
   char* base = P.use_smem ? smem_dyn : P.gscratch + (size_t)blockIdx.x * P.slab_bytes;
   size_t persist_bytes;
   const bool rxn = P.reaction != 0;
@@ -1138,6 +1309,26 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
   __syncthreads();
   const CoarseVec uH = e32 ? CoarseVec{nullptr, cws32.xh, cws32.xl} : CoarseVec{cws.uprev, nullptr, nullptr};
   double lam_prev = 0.0;  // coarse eigenvalue of the previous point of the chain
+  // a fine solve; one on the coarse mesh itself that FP32 corrections could not finish (the shift meets the
+  // eigenvalue by accident) runs again in FP64, its workspace in global memory
+  auto fine = [&](int n, const double* a, const double* rb, double lamH, int& it, int& outer, int& flags, double& gq) {
+    int fl = 0;
+    double v = 0.0;
+    const bool f64 = sizeof(T) == sizeof(float) && n == P.nc && P.nc > kEig32Max;  // beyond the FP32 form's reach
+    if (!f64) v = twogrid_fine<T>(fws, fine_base, n, a, rb, uH, P.nc, lamH, P, red, &msh, it, outer, fl, gq);
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (f64 || (n == P.nc && (fl & (kFlagLinNoConv | kFlagBreakdown)))) {
+        Carver c(P.fscratch + (size_t)blockIdx.x * P.fslab_bytes);
+        FineWS<double>& ws = *c.take<FineWS<double>>(1);
+        MinresShared<double>* ms = c.take<MinresShared<double>>(1);
+        char* base64 = (char*)c.take<double2>(1);
+        fl &= kFlagBadCoef;
+        v = twogrid_fine<double>(ws, base64, n, a, rb, uH, P.nc, lamH, P, red, ms, it, outer, fl, gq);
+      }
+    }
+    flags |= fl;
+    return v;
+  };
   const float omega = (float)P.omega;
   for (int ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     const int r = ch / cpr;
@@ -1263,23 +1454,13 @@ __global__ void __launch_bounds__(512) sample_kernel(SampleLaunch P) {
       const double* rbf = rxn ? P.b_f + b * nfT : nullptr;
       const double* rbp = rxn ? P.b_p + b * npT : nullptr;
       if (!P.direct_f) {
-        if (P.mode_f == 0)
-          lf = twogrid_fine<T>(fws, fine_base, P.nf, P.a_f + b * nfT, rbf, uH, nc, lamH, P, red, &msh, itf, of,
-                               flags, gf);
-        else if (P.mode_f == 1)
-          lf = twogrid_fine<double>(fws64, fine_base, P.nf, P.a_f + b * nfT, rbf, uH, nc, lamH, P, red, &msh64,
-                                    itf, of, flags, gf);
+        if (P.mode_f != 2) lf = fine(P.nf, P.a_f + b * nfT, rbf, lamH, itf, of, flags, gf);
         if (P.qoi && P.mode_f != 2) lf = gf;
       }
       if (P.prev_given) {
         lp = P.out[b * 4 + 2];  // every thread reads it before thread 0 rewrites the same value below
       } else if (P.np > 0 && !P.direct_p) {
-        if (P.mode_p == 0)
-          lp = twogrid_fine<T>(fws, fine_base, P.np, P.a_p + b * npT, rbp, uH, nc, lamH, P, red, &msh, itp, op,
-                               flags, gp);
-        else if (P.mode_p == 1)
-          lp = twogrid_fine<double>(fws64, fine_base, P.np, P.a_p + b * npT, rbp, uH, nc, lamH, P, red, &msh64,
-                                    itp, op, flags, gp);
+        if (P.mode_p != 2) lp = fine(P.np, P.a_p + b * npT, rbp, lamH, itp, op, flags, gp);
         if (P.qoi && P.mode_p != 2) lp = gp;
       }
       if (threadIdx.x == 0) {
@@ -1418,6 +1599,14 @@ cudaError_t launch_reuse_scatter(int R, int npts, uint32_t k0, size_t V, const d
   return cudaGetLastError();
 }
 
+size_t sample_fallback_bytes(int n, int reaction) {
+  Carver c(nullptr);
+  c.take<FineWS<double>>(1);
+  c.take<MinresShared<double>>(1);
+  c.take<double2>(1);
+  return (c.used() + fine_bytes<double>(n, reaction != 0) + 255) & ~(size_t)255;
+}
+
 size_t sample_slab_bytes(int nf, int nc, int np, int mixed) {
   return mixed ? slab_size<float>(nf, nc, np) : slab_size<double>(nf, nc, np);
 }
@@ -1427,16 +1616,22 @@ size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int mode_f, int mode
                : slab_size<double>(nf, nc, np, mode_f, mode_p, reaction != 0);
 }
 
+namespace {
+using SampleFn = void (*)(SampleLaunch);
+SampleFn sample_fn(int mixed, int threads) {
+  return mixed ? (threads <= 256 ? sample_kernel<float, 256> : sample_kernel<float, 512>) : sample_kernel<double, 512>;
+}
+}  // namespace
+
 int sample_occupancy(int mixed, int threads, size_t smem) {
   int nb = 0;
-  cudaError_t e = mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sample_kernel<float>, threads, smem)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sample_kernel<double>, threads, smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sample_fn(mixed, threads), threads, smem);
   return e == cudaSuccess ? nb : 0;
 }
 
 int sample_static_smem(int mixed) {
   cudaFuncAttributes fa;
-  cudaError_t e = mixed ? cudaFuncGetAttributes(&fa, sample_kernel<float>) : cudaFuncGetAttributes(&fa, sample_kernel<double>);
+  const cudaError_t e = cudaFuncGetAttributes(&fa, sample_fn(mixed, 512));
   return e == cudaSuccess ? (int)fa.sharedSizeBytes : 8192;
 }
 
@@ -1455,8 +1650,8 @@ cudaError_t raise_smem_limit(const void* func, int bytes) {
 }
 
 cudaError_t set_sample_smem(int mixed, int bytes) {
-  return mixed ? raise_smem_limit((const void*)sample_kernel<float>, bytes)
-               : raise_smem_limit((const void*)sample_kernel<double>, bytes);
+  const cudaError_t e = raise_smem_limit((const void*)sample_fn(mixed, 256), bytes);
+  return e == cudaSuccess ? raise_smem_limit((const void*)sample_fn(mixed, 512), bytes) : e;
 }
 
 cudaError_t launch_apply_operator(int n, int B, const double* d_a, int which, double sigma, const double* d_x,
@@ -1474,10 +1669,7 @@ cudaError_t launch_shift_sums(const double* d_out, const int* d_stat, int R, int
 }
 
 cudaError_t launch_sample(const SampleLaunch& p, int mixed, int blocks, int threads, size_t smem, cudaStream_t st) {
-  if (mixed)
-    sample_kernel<float><<<blocks, threads, smem, st>>>(p);
-  else
-    sample_kernel<double><<<blocks, threads, smem, st>>>(p);
+  sample_fn(mixed, threads)<<<blocks, threads, smem, st>>>(p);
   return cudaGetLastError();
 }
 
