@@ -598,15 +598,16 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   // 1e-6 keeps lambda^h within ~3e-13 of the exact two-grid value.  The mixed path refines
   // twice whatever the targets (the FP32 rounding of the first correction, which is
   // amplified by the near-singular shift, leaves a residual of ~1e-4): inner reductions of 1e-4
-  // and a target of 1e-5 leave lambda^h within ~2e-13 (1e-5 inner reductions above mesh 1/128).
+  // and a target of 1e-5 leave lambda^h within ~2e-13.
   // The functional G(u_H) of a direct level is first order in the eigenvector error, which the
   // eigen-residual bounds only to ~tol_eig (lambda_H is second order): it takes 1e-11.
   p.tol_eig = c->opt_tol_eig > 0 ? c->opt_tol_eig : (c->qoi == MQ_QOI_FUNCTIONAL ? 1e-11 : (want_u || rxn ? 1e-8 : 1e-6));
   p.max_eig_it = c->opt_max_eig > 0 ? c->opt_max_eig : 200;
   p.tol_lin = c->tol_lin > 0 ? c->tol_lin : (mixed ? 1e-5 : 1e-6);
   if (mixed) {
-    // the preconditioned residual MINRES reduces understates the 2-norm one by a factor growing
-    // like 1/h: finer meshes take a smaller inner reduction per refinement step
+    // (in the per-sample kernel; the streaming tier chooses the reduction of each solve)  The preconditioned
+    // residual MINRES reduces understates the 2-norm one by a factor growing like 1/h: finer meshes
+    // take a smaller inner reduction per refinement step
     p.tol_inner = g.nf > 128 ? 1e-5 : 1e-4;
     p.max_outer = 10;
   } else {
@@ -687,7 +688,10 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
     s.flags = (int*)c->stat.p + 3;
     s.flags_stride = 4;
     s.tol_lin = p.tol_lin;
-    s.tol_inner = p.tol_inner;
+    // reductions chosen step by step end closer to the residual target; the functional is first order in the
+    // residual, and on the islands (unresolved coarse mesh) lambda^h moves ~1e4 times more with it than
+    // for the sine families, so both keep fixed reductions that end further below
+    s.tol_inner = mixed && !(c->opt_tol_inner > 0) && !rxn && c->qoi == MQ_QOI_EIGENVALUE ? 0.0 : p.tol_inner;
     s.max_inner = p.max_inner_it;
     s.max_outer = p.max_outer;
     s.omega = p.omega;

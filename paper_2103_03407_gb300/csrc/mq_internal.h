@@ -80,7 +80,8 @@ struct StreamSolve {
   int outer_stride;
   int* flags;              // OR-ed with kFlag* bits
   int flags_stride;
-  double tol_lin, tol_inner;
+  double tol_lin;
+  double tol_inner;        // reduction of every inner solve; 0: chosen for each (FP32 path)
   int max_inner, max_outer;
   double omega;
   int nu;                  // Jacobi sweeps before and after each coarse-grid correction (1 or 2)
