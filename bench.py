@@ -470,9 +470,13 @@ def percta_fp64_flops(wl, level, st, prec, samples):
 #   per solve: 20 e + 72 bytes (clearing 8 e + 16, FP32 and FP64 weights 3 e + 32, interpolation
 #   and right-hand side e + 24, operators of the coarser levels ~8 e).
 def stream_bytes(wl, level, st, prec, samples):
+    # bytes per fine node.  Mixed path: per iteration the operator sweep 16, the Lanczos update 16, the vector's share of the
+    # combination 4 and the V(1,1) cycle 27 on the finest mesh (restriction 11, prolongation and smoothing
+    # 16) plus its coarser meshes; per refinement step another cycle, the scaling 8, the solution 16 and the
+    # residual 36; setup 74.  FP64 path: every array in FP64, w and x updated per iteration.
     e = 4 if prec == "mixed" else 8
     lv = wl.levels[level]
-    vcyc = 11.5 * e + 10.5 * e * (1 / 4 + 1 / 16)
+    vcyc = 27 * (1 + 1 / 4 + 1 / 16) if prec == "mixed" else 11.5 * e + 10.5 * e * (1 / 4 + 1 / 16)
     I, O = st["fine_iters_mean"], st["outer_iters_mean"]
     solves = []
     if lv.n_fine >= stream_min_default(prec) and not (lv.n_fine == lv.n_coarse and lv.s == lv.S):
@@ -483,7 +487,10 @@ def stream_bytes(wl, level, st, prec, samples):
             solves.append(pv.n_fine)
     per = 0.0
     for n in solves:
-        per += (n - 1) ** 2 * ((14 * e + vcyc) * I + (12 * e + 48 + vcyc) * O + 20 * e + 72)
+        if prec == "mixed":
+            per += (n - 1) ** 2 * ((36 + vcyc) * I + (60 + vcyc) * O + 74)
+        else:
+            per += (n - 1) ** 2 * ((14 * e + vcyc) * I + (12 * e + 48 + vcyc) * O + 20 * e + 56)
     return per * samples
 
 
@@ -494,12 +501,11 @@ SAMPLE_KERNEL_TRAFFIC = {"source_sha256": "5cfd76dfb86a1cec2d451c0ddf255b8e942fe
                          "level": 1, "precision": "mixed", "bytes_per_launch": 141.982720e6 + 95.710208e6}
 
 
-# ncu DRAM traffic of the operator sweep k_minres_q per algorithmic byte: one launch with the pending
-# MINRES update (10 arrays per node) on mesh 1/1024, 16 samples of the six-level workload's finest
-# level (summarised under profiles/), scaled to a launch by its algorithmic bytes; valid only for
-# the kernel source it was measured on
-KMINRES_TRAFFIC = {"source_sha256": "544ec7444614d4ab700b9665f19c3a860cc656f51459c999e0266c26273cc0c7",
-                   "dram_per_algorithmic": (471.794432e6 + 170.729984e6) / (16 * 1023 * 1023 * 40)}
+# ncu DRAM traffic of the operator sweep k_minres_q per algorithmic byte: one launch (4 arrays per node) on mesh
+# 1/1024, 16 samples of the six-level workload's finest level (summarised under profiles/), scaled to a
+# launch by its algorithmic bytes; valid only for the kernel source it was measured on
+KMINRES_TRAFFIC = {"source_sha256": "380ceaad2c828e22cbcfea23016c39d197e23e784370136009120356eafeaa9a",
+                   "dram_per_algorithmic": (202.488576e6 + 48.444672e6) / (16 * 1023 * 1023 * 16)}
 
 
 def _stream_source_hash():
@@ -517,7 +523,7 @@ def _stream_source_hash():
 def kminres_roofline(probe, steps):
     """Roofline of the largest kernel of the step: the streaming operator sweep, timed live with
     CUDA events around its launches over the timed region; algorithmic bytes counted on the device
-    (per active sample and node: 4 arrays, 10 with the pending MINRES update)."""
+    (per active sample and node: 4 arrays, 7 with a reaction term)."""
     ms, launches, nbytes = probe
     if launches == 0 or ms <= 0:
         return None

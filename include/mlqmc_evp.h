@@ -296,10 +296,10 @@ mq_status mq_graph_capture(mq_ctx* ctx, int32_t nranges, const int32_t* levels, 
                            const uint32_t* k1s, double* const* d_per_sample, double* const* d_shift_sums);
 mq_status mq_graph_launch(mq_ctx* ctx, const uint32_t* k0s);
 /* Live timing of the streaming tier's operator sweep (its largest kernel: the MINRES operator
- * application with the pending update, once per inner iteration): with on = 1, every later
+ * application, once per inner iteration): with on = 1, every later
  * host-driven streaming solve records CUDA events on the context stream around each launch of
  * that kernel and counts on the device the algorithmic bytes the launches move (per active sample
- * and interior node: weights and operand 4 arrays, plus 6 for the pending MINRES update).  Turning
+ * and interior node: 4 arrays, 7 with a reaction term; in FP64 plus 6 for the pending update).  Turning
  * it on (or off) clears the totals.  mq_get_kernel_probe returns the summed launch time (ms), the
  * launches and the algorithmic bytes since then (any output may be NULL).  Graph launches are not
  * timed. */

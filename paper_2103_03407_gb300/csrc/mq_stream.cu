@@ -6,9 +6,11 @@
 // grid-wide kernel over [sample][node] arrays instead, so the whole GPU streams every array with
 // full memory-level parallelism:
 //   * MINRES (preconditioned, symmetric indefinite) in the inner precision T, one iteration =
-//     K1 (pending w/x update, q = (A - sigma M) z / gamma, partial <q, z>), S1 (scalars),
-//     K2 (v_new; z_j is normalised inside the next pending update), the V-cycle, S2 (Givens
-//     rotation, convergence);
+//     K1 (q = (A - sigma M) z / gamma, partial <q, z>), S1 (scalars), K2 (v_new), the V-cycle, S2 (Givens
+//     rotation, convergence).  On the FP32 path the directions w_j are not formed: the preconditioned
+//     Lanczos vectors z_j are kept, S2 carries the coefficients of the solution (and of the last two
+//     directions) over them, and the solution is combined once per solve (or every kBasis
+//     iterations).  The FP64 path updates w and x with K1 of the next iteration;
 //   * the V-cycle (nu = 1 or 2 Jacobi steps before and after, Galerkin coarse levels) streams the
 //     meshes finer than 1/32.  nu = 2: four kernels per level -- two fused smoothing steps from
 //     zero, residual + restriction, prolongation + correction + one smoothing step, one smoothing
@@ -21,6 +23,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <initializer_list>
@@ -92,6 +95,9 @@ __device__ __forceinline__ void for_tile(int n, int ch, F f) {
   }
 }
 
+// FP32 path: Lanczos vectors kept between combinations (even: the graph mode runs iterations in pairs)
+constexpr int kBasis = 12;
+
 template <typename T>
 struct SS {  // per-sample solver scalars
   T gam, gam_old, eta, eta0, c, c_old, s, s_old, ig, c1, c2, cx, ia1, a2, a3, delta, rs;
@@ -109,6 +115,21 @@ struct SS {  // per-sample solver scalars
   int act;        // inner MINRES running
   int pend;       // a w/x update is pending
   int iters, outer, flags;
+  // FP32 path: coefficients of the inner solution and of the directions w_{j-1}, w_{j-2} over the vectors z of
+  // iterations j0 .. j0 + nb - 1 and (last two) the directions stored by the last combination
+  float cxs[kBasis + 2], cw1[kBasis + 2], cw2[kBasis + 2];
+  int j0, nb;
+  int combined;  // the coefficients have been applied (a combination inside the solve)
+};
+
+// FP32 path: the Lanczos vector of iteration j + (jc ? *jc : 0), kept in a ring of kBasis + 1 slots of
+// `stride` entries (jc: the device iteration counter of the graph mode); base NULL: a plain vector
+struct ZSlot {
+  float* base;
+  size_t stride;
+  const int* jc;
+  int j;
+  __device__ float* get() const { return base + stride * (size_t)(((jc ? *jc : 0) + j) % (kBasis + 1)); }
 };
 
 // block reduction of NV partial sums to part[(b * nch + ch) * NV + i] (butterfly within each warp,
@@ -394,6 +415,7 @@ __global__ void k_inner_init(int n, int B, const int* __restrict__ act, const SS
   const size_t off = (size_t)b * ssz(n);
   for_tile(n, ch, [&](int p, int, int) {
     v[off + p] *= rs;
+    if (!vo) return;  // FP32 path: nothing else is read before it is written
     vo[off + p] = T(0);
     w[off + p] = T(0);
     wo[off + p] = T(0);
@@ -709,9 +731,9 @@ __global__ void __launch_bounds__(kThreads) k_sub_build(int ns, int B, const T* 
 template <typename T>
 __global__ void __launch_bounds__(kSubThreads) k_subcycle(int ns, int B, const int* __restrict__ act,
                                                        const char* __restrict__ subw, size_t wbytes,
-                                                       const T* __restrict__ bin, T* __restrict__ xout, int ldio,
+                                                       const T* __restrict__ bin, T* xout, int ldio,
                                                        int nu, T om, double* part, const T* __restrict__ dotv,
-                                                       int rxn) {
+                                                       int rxn, ZSlot zs) {
   // bin / xout: rows of ldio entries (ns + 1 for the sub-cycle's own arrays, sld(ns) when the
   // whole V-cycle of a streamed mesh runs here); the shared-memory copies have rows of ns + 1
   extern __shared__ __align__(16) char sm[];
@@ -742,7 +764,7 @@ __global__ void __launch_bounds__(kSubThreads) k_subcycle(int ns, int B, const i
   __syncthreads();
   // with dotv (the right-hand side itself, copied to b0) also <v, x>
   T acc[1] = {vcycle<T>(mg, b0, x0, om, dotv ? b0 : nullptr, nu)};
-  T* dst = xout + (size_t)b * (size_t)(ns + 1) * ldio;
+  T* dst = (zs.base ? (T*)zs.get() : xout) + (size_t)b * (size_t)(ns + 1) * ldio;
   for_all(V, [&](size_t q) {
     const int i = (int)(q % ld), j = (int)(q / ld);
     dst[j * ldio + i] = x0[q];
@@ -818,26 +840,29 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ float at(const float4& v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
 
-// K1, vectorised: the pending w/x update, q = (A - sigma M) z * ig and the partial <q, z>; with RX
-// the operator is A + B - sigma M, B the reaction matrix from its edge weights rx, ry, rd (edges to
-// E, N and NE)
+// K1 of the FP32 path: q = (A - sigma M) z * ig and the partial <q, z>; with RX the operator is A + B - sigma
+// M, B the reaction matrix from its edge weights rx, ry, rd (edges to E, N and NE).  Bound by memory: 16 B
+// per node (28 B with a reaction).  With the update of w and x in this kernel it moved 40 B; the kept
+// vectors cost 4 B per iteration when they are combined.  16 samples of mesh 1/1024: 109 -> 66 us per
+// launch in ncu.
+// work: NULL, or a device counter of the algorithmic bytes moved
 template <bool RX>
 __global__ void k_minres_q4(int n, int B, const int* __restrict__ act, const SS<float>* __restrict__ ss,
-                            const float* __restrict__ wx, const float* __restrict__ wy, const float* __restrict__ z,
-                            const float* __restrict__ zp, float* __restrict__ wo, const float* __restrict__ w,
-                            float* __restrict__ xi, float* __restrict__ qv, double* part, unsigned long long* work,
+                            const float* __restrict__ wx, const float* __restrict__ wy, ZSlot zs,
+                            float* __restrict__ qv, double* part, unsigned long long* work,
                             const float* __restrict__ rx, const float* __restrict__ ry, const float* __restrict__ rd) {
   const int nt = tiles_vec(n);
   const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
   if (b >= B || !act[b]) return;
-  const SS<float> S = ss[b];
+  const float sigm = ss[b].sigm, ig = ss[b].ig;
+  const float* __restrict__ z = zs.get();
   if (work && threadIdx.x == 0) {
     const long tot = (long)(n - 1) * (n / kVec);
     const long g0 = (long)ch * kThreads, g1 = g0 + kThreads < tot ? g0 + kThreads : tot;
     // interior nodes of the tile: four per thread, minus the boundary column of each row start
     const long per_row = n / kVec;
     const long nodes = kVec * (g1 - g0) - ((g1 + per_row - 1) / per_row - (g0 + per_row - 1) / per_row);
-    atomicAdd(work, (unsigned long long)(nodes * ((S.pend ? 10 : 4) + (RX ? 3 : 0)) * (long)sizeof(float)));
+    atomicAdd(work, (unsigned long long)(nodes * (4 + (RX ? 3 : 0)) * (long)sizeof(float)));
   }
   const int ld = sld(n);
   const size_t off = (size_t)b * ssz(n);
@@ -845,21 +870,6 @@ __global__ void k_minres_q4(int n, int B, const int* __restrict__ act, const SS<
   int j, c0;
   if (vec_walk(n, ch, j, c0)) {
     const size_t p = off + (size_t)j * ld + c0;
-    if (S.pend) {
-      const float4 a = ld4(zp + p), o = ld4(wo + p), ww = ld4(w + p);
-      float4 x = ld4(xi + p);
-      float4 wn;
-      wn.x = (a.x * S.igp - S.a3 * o.x - S.a2 * ww.x) * S.ia1;
-      wn.y = (a.y * S.igp - S.a3 * o.y - S.a2 * ww.y) * S.ia1;
-      wn.z = (a.z * S.igp - S.a3 * o.z - S.a2 * ww.z) * S.ia1;
-      wn.w = (a.w * S.igp - S.a3 * o.w - S.a2 * ww.w) * S.ia1;
-      x.x += S.cx * wn.x;
-      x.y += S.cx * wn.y;
-      x.z += S.cx * wn.z;
-      x.w += S.cx * wn.w;
-      st4(wo + p, wn);
-      st4(xi + p, x);
-    }
     const float4 zc = ld4(z + p), zn = ld4(z + p + ld), zs = ld4(z + p - ld);
     const float4 wc = ld4(wx + p), yc = ld4(wy + p), ys = ld4(wy + p - ld);
     const bool first = c0 == 0;
@@ -887,13 +897,13 @@ __global__ void k_minres_q4(int n, int B, const int* __restrict__ act, const SS<
       const float we = at(wc, k), wwv = k > 0 ? at(wc, k - 1) : wwest;
       const float st = we * (xp - xe) + wwv * (xp - xw) + at(yc, k) * (xp - xn) + at(ys, k) * (xp - xs);
       const float ms = 6.0f * xp + (xe + xw) + (xn + xs) + (xne + xsw);
-      float kz = st - S.sigm * ms;
+      float kz = st - sigm * ms;
       if (RX) {
         const float rw = k > 0 ? at(rxc, k - 1) : rxw, rsw = k > 0 ? at(rds, k - 1) : rdsw;
         kz += hmf * (at(rxc, k) * (xp + xe) + rw * (xp + xw) + at(ryc, k) * (xp + xn) + at(rys, k) * (xp + xs) +
                      at(rdc, k) * (xp + xne) + rsw * (xp + xsw));
       }
-      kz *= S.ig;
+      kz *= ig;
       q[k] = (first && k == 0) ? 0.0f : kz;
       acc[0] += q[k] * xp;
     }
@@ -912,7 +922,8 @@ __global__ void k_minres_v4(int n, int B, const int* __restrict__ act, const SS<
   int j, c0;
   if (!vec_walk(n, ch, j, c0)) return;
   const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
-  const float4 a = ld4(q + p), bv = ld4(v + p), o = ld4(vo + p);
+  // (c2 = 0 in the first iteration, when vo holds nothing)
+  const float4 a = ld4(q + p), bv = ld4(v + p), o = c2 != 0.0f ? ld4(vo + p) : make_float4(0.f, 0.f, 0.f, 0.f);
   st4(vo + p, make_float4(a.x - c1 * bv.x - c2 * o.x, a.y - c1 * bv.y - c2 * o.y, a.z - c1 * bv.z - c2 * o.z,
                           a.w - c1 * bv.w - c2 * o.w));
 }
@@ -1210,25 +1221,61 @@ __global__ void __launch_bounds__(kThreads) k_rhs4(int n, int B, const float* __
   tile_partials_df<1>(acc, part, (size_t)b * nt + ch);
 }
 
-// x += ||r|| xi (double-float x) for samples that ran an inner solve this step
-__global__ void __launch_bounds__(kThreads) k_outer_update4(int n, int B, const SS<float>* __restrict__ ss,
-                                                            const int* __restrict__ ran, const float* __restrict__ xi,
-                                                            float* __restrict__ xh, float* __restrict__ xl) {
+// x += ||r|| xi (double-float x) with xi combined from the kept Lanczos vectors.  FLUSH = false: at the end of a
+// refinement step, for the samples that ran an inner solve.  FLUSH = true: inside a solve, when the vectors
+// of kBasis iterations are complete (jc: graph mode, the device iteration counter; the launch does
+// nothing in the other iterations), for the samples still iterating; also combines the last two directions
+// into w1, w0.
+template <bool FLUSH>
+__global__ void __launch_bounds__(kThreads) k_combine4(int n, int B, SS<float>* __restrict__ ss,
+                                                       const int* __restrict__ on, ZSlot zs, float* __restrict__ w0,
+                                                       float* __restrict__ w1, float* __restrict__ xh,
+                                                       float* __restrict__ xl) {
+  if (FLUSH && zs.jc && (*zs.jc + zs.j + 1) % kBasis != 0) return;
   const int nt = tiles_vec(n);
-  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
-  int j, c0;
-  if (b >= B || !ran[b] || !vec_walk(n, ch, j, c0)) return;
-  const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
-  const df rn = df_split(ss[b].rnorm);
-  const float4 d = ld4(xi + p), a = ld4(xh + p), c = ld4(xl + p);
-  float h[kVec], l[kVec];
+  for (int t = blockIdx.x; t < B * nt; t += gridDim.x) {
+    const int b = t / nt, ch = t % nt;
+    int j, c0;
+    if (!on[b]) continue;
+    const SS<float>& S = ss[b];
+    const int nb = S.nb, j0 = S.j0;
+    if (FLUSH ? nb != kBasis : S.combined != 0) continue;
+    if (FLUSH && ch == 0 && threadIdx.x == 0) ss[b].combined = 1;  // read by later launches only
+    if (!vec_walk(n, ch, j, c0)) continue;
+    const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
+    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f), a1 = xi, a2 = xi;
+    auto add = [](float4& s, float c, const float4& z) {
+      s.x = fmaf(c, z.x, s.x), s.y = fmaf(c, z.y, s.y), s.z = fmaf(c, z.z, s.z), s.w = fmaf(c, z.w, s.w);
+    };
+    auto term = [&](int k, const float* z) {
+      const float4 v = ld4(z + p);
+      add(xi, S.cxs[k], v);
+      if (FLUSH) {
+        add(a1, S.cw1[k], v);
+        add(a2, S.cw2[k], v);
+      }
+    };
+#pragma unroll 4
+    for (int k = 0; k < nb; ++k) term(k, zs.base + zs.stride * (size_t)((j0 + k) % (kBasis + 1)));
+    if (j0) {
+      term(kBasis, w0);
+      term(kBasis + 1, w1);
+    }
+    const df rn = df_split(S.rnorm);
+    const float4 a = ld4(xh + p), c = ld4(xl + p);
+    float h[kVec], l[kVec];
 #pragma unroll
-  for (int k = 0; k < kVec; ++k) {
-    const df v = df_add(df{at(a, k), at(c, k)}, df_mul(rn, at(d, k)));
-    h[k] = v.h, l[k] = v.l;
+    for (int k = 0; k < kVec; ++k) {
+      const df v = df_add(df{at(a, k), at(c, k)}, df_mul(rn, at(xi, k)));
+      h[k] = v.h, l[k] = v.l;
+    }
+    st4v(xh + p, h);
+    st4v(xl + p, l);
+    if (FLUSH) {
+      st4(w1 + p, a1);
+      st4(w0 + p, a2);
+    }
   }
-  st4v(xh + p, h);
-  st4v(xl + p, l);
 }
 
 // Residual r = b - K x, K = A (+ B) - sigma M, in double-float arithmetic; v = r rounded to FP32.
@@ -1490,7 +1537,7 @@ template <bool DOT, typename WT = float, bool RX = false>
 __global__ void k_prolong_smooth1_4(int n, int B, const int* __restrict__ act, const WT* __restrict__ wx,
                                     const WT* __restrict__ wy, const WT* __restrict__ dinv,
                                     const float* __restrict__ bb, const float* __restrict__ xc, int ldc,
-                                    float* __restrict__ out, const float* __restrict__ dotv, double* part,
+                                    float* out, const float* __restrict__ dotv, double* part, ZSlot zs,
                                     const WT* __restrict__ dr = nullptr) {
   const int nt = tiles_vec(n);
   const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
@@ -1498,6 +1545,7 @@ __global__ void k_prolong_smooth1_4(int n, int B, const int* __restrict__ act, c
   const int ld = sld(n);
   const size_t off = (size_t)b * ssz(n);
   const float* __restrict__ XC = xc + (size_t)b * (size_t)(n / 2 + 1) * ldc;
+  float* __restrict__ O = zs.base ? zs.get() : out;
   float acc[1] = {0.0f};
   int j, c0;
   if (vec_walk(n, ch, j, c0)) {
@@ -1557,7 +1605,7 @@ __global__ void k_prolong_smooth1_4(int n, int B, const int* __restrict__ act, c
       if (RX) ax += at(drc, k) * tp;
       o[k] = (first && k == 0) ? 0.0f : tp + at(dc, k) * (at(rc, k) - ax);
     }
-    st4(out + p, make_float4(o[0], o[1], o[2], o[3]));
+    st4(O + p, make_float4(o[0], o[1], o[2], o[3]));
     if (DOT) {
       const float4 dv = ld4(dotv + p);
       acc[0] = dv.x * o[0] + dv.y * o[1] + dv.z * o[2] + dv.w * o[3];
@@ -1615,11 +1663,16 @@ __global__ void k_sc_gamma0(int B, int nch, const double* part, const int* act, 
   S.ig = T(1) / g;
   S.pend = 0;
   if (brk) S.flags |= kFlagBreakdown;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    for (int k = 0; k < kBasis + 2; ++k) S.cxs[k] = S.cw1[k] = S.cw2[k] = 0.0f;
+    S.j0 = S.nb = S.combined = 0;
+  }
 }
 
 template <typename T>
-__global__ void k_sc_delta(int B, int nch, const double* part, const int* act, SS<T>* ss) {
+__global__ void k_sc_delta(int B, int nch, const double* part, const int* act, SS<T>* ss, int* count) {
   const int b = warp_sample();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;  // of the Givens kernel that follows
   if (b >= B || !act[b]) return;
   double t[1];
   warp_sum_slots<1>(part, b, nch, t);
@@ -1629,11 +1682,14 @@ __global__ void k_sc_delta(int B, int nch, const double* part, const int* act, S
   const T delta = T(s) * S.ig;
   S.c1 = delta * S.ig;
   S.c2 = S.gam / S.gam_old;
+  if constexpr (sizeof(T) == sizeof(float))
+    if (S.j0 == 0 && S.nb == 0) S.c2 = 0.0f;  // the first iteration of a solve: there is no v_old yet
   S.delta = delta;
 }
 
-// Givens step; a converged sample keeps its pending update and leaves the active set after the
-// next K1 (which applies it)
+// Givens step.  FP64 path: a converged sample keeps its pending update and leaves the active set after the
+// next K1 (which applies it).  FP32 path: the step's direction w_j = (z_j / gamma_j - a3 w_{j-2} - a2 w_{j-1})
+// / a1 enters the coefficients, and a converged sample leaves at once.
 // jc (graph mode): the device iteration counter of the inner loop; iteration *jc + joff is the
 // last one allowed when it reaches max_inner - 1, and every sample then counts as done (its pending
 // update is applied by the next operator sweep, as the host loop's final update would)
@@ -1672,13 +1728,32 @@ __global__ void k_sc_givens(int B, int nch, const double* part, int* act, SS<T>*
   S.gam_old = gam;
   S.gam = gnew;
   S.igp = S.ig;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    if (S.combined) {  // the last kBasis vectors have been combined: start from the stored directions
+      for (int k = 0; k < kBasis + 2; ++k) S.cxs[k] = S.cw1[k] = S.cw2[k] = 0.0f;
+      S.cw2[kBasis] = S.cw1[kBasis + 1] = 1.0f;
+      S.j0 += kBasis;
+      S.nb = S.combined = 0;
+    }
+    for (int k = 0; k < kBasis + 2; ++k) {
+      const float w = ((k == S.nb ? S.igp : 0.0f) - al3 * S.cw2[k] - al2 * S.cw1[k]) * ia1;
+      S.cxs[k] += S.cx * w;
+      S.cw2[k] = S.cw1[k];
+      S.cw1[k] = w;
+    }
+    S.nb += 1;
+  }
   S.ig = gnew > T(0) ? T(1) / gnew : T(0);
   S.pend = 1;
   S.iters += 1;
   const bool capped = jc && *jc + joff + 1 >= max_inner;
   const bool done = fabs(S.eta) <= S.tol * S.eta0 || gnew == T(0) || capped;
-  if (done) S.act = 0;  // leaves after the next K1
-  else atomicAdd(count, 1);
+  if (!done)
+    atomicAdd(count, 1);
+  else if constexpr (sizeof(T) == sizeof(float))
+    act[b] = 0;
+  else
+    S.act = 0;  // leaves after the next K1
 }
 
 // samples that converged in the last Givens step leave the active set (K1 applied their update)
@@ -1795,6 +1870,41 @@ __global__ void k_cond_inner(cudaGraphConditionalHandle h, int* counter, const i
   cudaGraphSetConditional(h, (*count > 0 && *counter < max_iter) ? 1u : 0u);
 }
 
+__global__ void k_to_slot(int n, int B, const int* __restrict__ act, const float* __restrict__ x, ZSlot zs) {
+  const int nt = tiles_vec(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  int j, c0;
+  if (b >= B || !act[b] || !vec_walk(n, ch, j, c0)) return;
+  const size_t p = (size_t)b * ssz(n) + (size_t)j * sld(n) + c0;
+  st4(zs.get() + p, ld4(x + p));
+}
+
+// zeros on the boundary ring (and the padding columns) of up to 24 node arrays of mesh n: the sweeps write the
+// interiors before they read them
+struct RingList {
+  float* a[24];
+  int count;
+};
+__global__ void k_zero_ring(int n, int B, RingList L) {
+  const int ld = sld(n), per = 2 * ld + (n - 1) * 5;
+  const size_t tot = (size_t)B * per;
+  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += (size_t)gridDim.x * blockDim.x) {
+    const size_t b = q / per;
+    const int e = (int)(q % per);
+    int i, j;
+    if (e < 2 * ld) {
+      j = e < ld ? 0 : n;
+      i = e % ld;
+    } else {
+      const int f = (e - 2 * ld) % 5;
+      j = 1 + (e - 2 * ld) / 5;
+      i = f ? n - 1 + f : 0;
+    }
+    const size_t p = b * ssz(n) + (size_t)j * ld + i;
+    for (int k = 0; k < L.count; ++k) L.a[k][p] = 0.0f;
+  }
+}
+
 template <typename T>
 __global__ void k_zero(size_t count, T* p) {
   for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < count; q += (size_t)gridDim.x * blockDim.x)
@@ -1809,28 +1919,17 @@ __global__ void k_set_int(int B, int* p, int v) {
 
 // ---------------------------------------------------------------------------------------------
 // host driver
-// The operator sweep and the Lanczos update: vectorised kernels for FP32, the row-mapped ones for
-// FP64.  Returns the number of partial-sum slots per sample the sweep wrote (for k_sc_delta).
-template <typename T>
-int launch_minres_q(int n, int B, const int* act, const SS<T>* ss, const T* wx, const T* wy, const double* lamH,
-                    int lam_stride, const T* z, const T* zp, T* wo, const T* w, T* xi, T* q, double* part,
-                    unsigned long long* work, cudaStream_t st, const T* rx = nullptr, const T* ry = nullptr,
-                    const T* rd = nullptr) {
-  if constexpr (sizeof(T) == sizeof(float)) {
-    (void)lamH;
-    (void)lam_stride;
-    if (rx)
-      k_minres_q4<true><<<B * tiles_vec(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, z, zp, wo, w, xi, q, part, work,
-                                                              rx, ry, rd);
-    else
-      k_minres_q4<false><<<B * tiles_vec(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, z, zp, wo, w, xi, q, part, work,
-                                                               nullptr, nullptr, nullptr);
-    return tiles_vec(n);
-  } else {
-    k_minres_q<T><<<B * tiles_interior(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, lamH, lam_stride, z, zp, wo, w,
-                                                            xi, q, part, work);
-    return tiles_interior(n);
-  }
+// The operator sweep of the FP32 path (zs: the Lanczos vector it applies to); returns the partial-sum slots per
+// sample (for k_sc_delta)
+int launch_minres_q4(int n, int B, const int* act, const SS<float>* ss, const float* wx, const float* wy, ZSlot zs,
+                     float* q, double* part, unsigned long long* work, cudaStream_t st, const float* rx, const float* ry,
+                     const float* rd) {
+  if (rx)
+    k_minres_q4<true><<<B * tiles_vec(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, zs, q, part, work, rx, ry, rd);
+  else
+    k_minres_q4<false><<<B * tiles_vec(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, zs, q, part, work, nullptr, nullptr,
+                                                             nullptr);
+  return tiles_vec(n);
 }
 
 template <typename T>
@@ -1851,7 +1950,8 @@ struct Arena {
   int n, B, Ls;  // Ls streaming multigrid levels (meshes n .. > kSub)
   int nu;        // Jacobi sweeps per side of the V-cycle (1 or 2)
   size_t V0;
-  T *v, *vo, *z, *zn, *w, *wo, *q, *xi;
+  T *v, *vo, *z, *zn, *w, *wo, *q, *xi;  // (z, zn, xi: FP64 path; w, wo of the FP32 path: stored directions)
+  float* zb;            // FP32 path: the kept Lanczos vectors, kBasis + 1 slots of B V0 entries
   double *x64, *b64;  // FP64 path: solution and right-hand side
   // FP32 path: the same as double-floats, and the low parts of the finest mesh's edge weights
   float *xh, *xl, *bh, *bl, *wxl, *wyl;
@@ -1882,15 +1982,10 @@ size_t carve_arena(void* base, int n, int B, Arena<T>& A, bool rxn = false) {
   A.rxn = rxn ? 1 : 0;
   A.V0 = ssz(n);
   const size_t Bz = (size_t)B;
-  A.v = c.take<T>(Bz * A.V0);
-  A.vo = c.take<T>(Bz * A.V0);
-  A.z = c.take<T>(Bz * A.V0);
-  A.zn = c.take<T>(Bz * A.V0);
-  A.w = c.take<T>(Bz * A.V0);
-  A.wo = c.take<T>(Bz * A.V0);
-  A.q = c.take<T>(Bz * A.V0);
-  A.xi = c.take<T>(Bz * A.V0);
   const bool f32 = sizeof(T) == sizeof(float);
+  T** const vecs[8] = {&A.v, &A.vo, &A.q, &A.w, &A.wo, &A.z, &A.zn, &A.xi};
+  for (int k = 0; k < 8; ++k) *vecs[k] = f32 && k >= 5 ? nullptr : c.take<T>(Bz * A.V0);
+  A.zb = f32 ? c.take<float>(Bz * A.V0 * (kBasis + 1)) : nullptr;
   A.x64 = f32 ? nullptr : c.take<double>(Bz * A.V0);
   A.b64 = f32 ? nullptr : c.take<double>(Bz * A.V0);
   float** const pairs[6] = {&A.xh, &A.xl, &A.bh, &A.bl, &A.wxl, &A.wyl};
@@ -1950,11 +2045,12 @@ size_t carve_arena(void* base, int n, int B, Arena<T>& A, bool rxn = false) {
 // V-cycle over the arena hierarchy: x0 = B^{-1} b0; with dotv, partial <dotv, x0> into part
 template <typename T>
 cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om, const T* dotv, double* part,
-                          size_t sub_smem, cudaStream_t st) {
+                          size_t sub_smem, cudaStream_t st, ZSlot zs = ZSlot{}) {
   const int n = A.n, B = A.B;
+  const ZSlot plain{};
   if (A.Ls == 0) {
     ++tl_launches, k_subcycle<T><<<B, kSubThreads, sub_smem, st>>>(n, B, act, A.subw, A.subw_bytes, b0, x0, sld(n), A.nu,
-                                                                   om, part, dotv, A.rxn);
+                                                                   om, part, dotv, A.rxn, zs);
     LAUNCH_CHECK();
     return cudaSuccess;
   }
@@ -1986,7 +2082,7 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
     }
     const int ns = n >> A.Ls;
     ++tl_launches, k_subcycle<T><<<B, kSubThreads, sub_smem, st>>>(ns, B, act, A.subw, A.subw_bytes, A.bsub, A.xsub,
-                                                                   ns + 1, 1, om, nullptr, nullptr, A.rxn);
+                                                                   ns + 1, 1, om, nullptr, nullptr, A.rxn, plain);
     LAUNCH_CHECK();
     for (int l = A.Ls - 1; l >= 0; --l) {
       const int nl = n >> l;
@@ -1998,16 +2094,16 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
         if (A.hr[l]) {
           if (l == 0 && dotv)
             ++tl_launches, k_prolong_smooth1_4<true, __nv_bfloat16, true><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, A.hr[l]);
+                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, l ? plain : zs, A.hr[l]);
           else
             ++tl_launches, k_prolong_smooth1_4<false, __nv_bfloat16, true><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, A.hr[l]);
+                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, l ? plain : zs, A.hr[l]);
         } else if (l == 0 && dotv) {
           ++tl_launches, k_prolong_smooth1_4<true, __nv_bfloat16><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part);
+              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, l ? plain : zs);
         } else {
           ++tl_launches, k_prolong_smooth1_4<false, __nv_bfloat16><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr);
+              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, l ? plain : zs);
         }
       } else {
         if (l == 0 && dotv)
@@ -2036,7 +2132,7 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
   }
   const int ns = n >> A.Ls;
   ++tl_launches, k_subcycle<T><<<B, kSubThreads, sub_smem, st>>>(ns, B, act, A.subw, A.subw_bytes, A.bsub, A.xsub, ns + 1,
-                                                                 A.nu, om, nullptr, nullptr, A.rxn);
+                                                                 A.nu, om, nullptr, nullptr, A.rxn, plain);
   LAUNCH_CHECK();
   for (int l = A.Ls - 1; l >= 0; --l) {
     const int nl = n >> l;
@@ -2053,6 +2149,10 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
     else
       ++tl_launches, k_smooth<T, false><<<B * tiles_interior(nl), kThreads, 0, st>>>(nl, B, act, A.wx[l], A.wy[l], A.dinv[l], b,
                                                                      A.t[l], xa, nullptr, nullptr);
+    LAUNCH_CHECK();
+  }
+  if (zs.base) {  // V(2,2) on the FP32 path works in x0 = q, free here (its sweeps take plain pointers): move the result
+    ++tl_launches, k_to_slot<<<B * tiles_vec(n), kThreads, 0, st>>>(n, B, act, (const float*)x0, zs);
     LAUNCH_CHECK();
   }
   return cudaSuccess;
@@ -2109,10 +2209,12 @@ cudaError_t close_while(cudaStream_t body) {
 template <typename T>
 cudaError_t outer_pass(const StreamSolve& s, Arena<T>& A, df hm, cudaStream_t st) {
   const int n = s.n, B = s.B, gw = (B + 7) / 8;
+  const size_t Bz0 = (size_t)B * A.V0;
   if constexpr (sizeof(T) == sizeof(float)) {
     const int nt = tiles_vec(n);
     const ResidualIn W{A.wx[0], A.wy[0], A.wxl, A.wyl, A.rx, A.ry, A.rd, A.rxl, A.ryl, A.rdl};
-    ++tl_launches, k_outer_update4<<<B * nt, kThreads, 0, st>>>(n, B, A.ss, A.ran, A.xi, A.xh, A.xl);
+    ++tl_launches, k_combine4<false><<<B * nt, kThreads, 0, st>>>(n, B, A.ss, A.ran, ZSlot{A.zb, Bz0, nullptr, 0}, A.wo,
+                                                                 A.w, A.xh, A.xl);
     LAUNCH_CHECK();
     ++tl_launches;
     if (A.rxn)
@@ -2148,6 +2250,8 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   const T om = T(s.omega);
   const double hm64 = 1.0 / (12.0 * n * n);
   const df hm{(float)hm64, (float)(hm64 - (double)(float)hm64)};
+  auto slot = [&](const int* jc, int j) { return ZSlot{A.zb, Bz * A.V0, jc, j}; };
+  const int gc = std::min(B * tiles_vec(n), 152 * 8);  // combinations inside a solve: mostly nothing to do in graph mode
   const int ns = n >> A.Ls;
   const size_t sub_smem = sub_vectors_bytes<T>(ns, A.rxn != 0);
   cudaError_t e = raise_smem_limit((const void*)k_subcycle<T>, (int)sub_smem);
@@ -2158,23 +2262,41 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   const int gw = (B + 7) / 8;  // warp-per-sample scalar kernels: 8 samples per 256-thread block
   // ---- clear vectors (boundary rings must be zero), build the operators
   const size_t V0 = A.V0;
-  T* const vecs[8] = {A.v, A.vo, A.z, A.zn, A.w, A.wo, A.q, A.xi};
-  for (int k = 0; k < 8; ++k) {
-    ++tl_launches, k_zero<T><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, vecs[k]);
-    LAUNCH_CHECK();
-  }
   if constexpr (kF32) {
-    float* const pairs[4] = {A.xh, A.xl, A.bh, A.bl};
-    for (float* a : pairs) ++tl_launches, k_zero<float><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, a);
+    // the solution starts at zero; of the other vectors only the rings are read before they are written
+    float* const xs[2] = {A.xh, A.xl};
+    for (float* a : xs) ++tl_launches, k_zero<float><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, a);
+    for (int l = 0; l < (A.Ls > 1 ? A.Ls : 1); ++l) {
+      RingList L{};
+      auto put = [&](float* a) {
+        if (a) L.a[L.count++] = a;
+      };
+      if (l == 0) {
+        float* const vecs[5] = {A.v, A.vo, A.q, A.w, A.wo};
+        for (float* a : vecs) put(a);
+        for (int k = 0; k <= kBasis; ++k) put(A.zb + (size_t)k * Bz * V0);
+      }
+      put(A.t[l]);
+      put(A.x[l]);
+      put(A.b[l]);
+      const int nl = n >> l;
+      ++tl_launches, k_zero_ring<<<grid1(Bz * (size_t)(7 * nl + 3)), 256, 0, st>>>(nl, B, L);
+      LAUNCH_CHECK();
+    }
   } else {
+    T* const vecs[8] = {A.v, A.vo, A.z, A.zn, A.w, A.wo, A.q, A.xi};
+    for (int k = 0; k < 8; ++k) {
+      ++tl_launches, k_zero<T><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, vecs[k]);
+      LAUNCH_CHECK();
+    }
     ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.x64);
     ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.b64);
-  }
-  for (int l = 0; l < A.Ls; ++l) {
-    const size_t V = ssz(n >> l);
-    T* const lv[3] = {A.t[l], A.x[l], A.b[l]};
-    for (int k = 0; k < 3; ++k)
-      if (lv[k]) ++tl_launches, k_zero<T><<<grid1(Bz * V), 256, 0, st>>>(Bz * V, lv[k]);
+    for (int l = 0; l < A.Ls; ++l) {
+      const size_t V = ssz(n >> l);
+      T* const lv[3] = {A.t[l], A.x[l], A.b[l]};
+      for (int k = 0; k < 3; ++k)
+        if (lv[k]) ++tl_launches, k_zero<T><<<grid1(Bz * V), 256, 0, st>>>(Bz * V, lv[k]);
+    }
   }
   if (A.Ls) {
     ++tl_launches, k_zero<T><<<grid1(Bz * gsz(ns)), 256, 0, st>>>(Bz * gsz(ns), A.bsub);
@@ -2241,11 +2363,11 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   // ---- right-hand side b = M P u_H
   int nts = nt;  // partial slots per sample of ||b||^2 and of the residual's sums
   if constexpr (kF32) {
-    // q and xi hold P u_H for a moment (their rings are zero; the first sweep overwrites them)
+    // q and the first Lanczos vector hold P u_H for a moment (their rings are zero; both are written again first)
     nts = tiles_vec(n);
-    ++tl_launches, k_interp4<<<B * nts, kThreads, 0, st>>>(n, s.nc, B, s.uH, A.q, A.xi);
+    ++tl_launches, k_interp4<<<B * nts, kThreads, 0, st>>>(n, s.nc, B, s.uH, A.q, A.zb);
     LAUNCH_CHECK();
-    ++tl_launches, k_rhs4<<<B * nts, kThreads, 0, st>>>(n, B, A.q, A.xi, A.bh, A.bl, A.v, hm, A.part);
+    ++tl_launches, k_rhs4<<<B * nts, kThreads, 0, st>>>(n, B, A.q, A.zb, A.bh, A.bl, A.v, hm, A.part);
   } else {
     ++tl_launches, k_interp<T><<<B * nt, kThreads, 0, st>>>(n, s.nc, B, s.uH, A.x64);
     LAUNCH_CHECK();
@@ -2277,10 +2399,13 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     ++tl_launches, k_sc_outer_begin<T><<<gs, 256, 0, b0>>>(B, n, s.lamH, s.lam_stride, s.tol_lin, s.tol_inner, A.ss, A.act, cnt_o);
     LAUNCH_CHECK();
     if ((e = cudaMemcpyAsync(A.ran, A.act, Bz * sizeof(int), cudaMemcpyDeviceToDevice, b0)) != cudaSuccess) return e;
-    ++tl_launches, k_inner_init<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.act, A.ss, A.v, A.vo, A.w, A.wo, A.xi);
+    ++tl_launches, k_inner_init<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.act, A.ss, A.v, kF32 ? nullptr : A.vo, A.w, A.wo, A.xi);
     LAUNCH_CHECK();
     T *v = A.v, *vo = A.vo, *z = A.z, *zn = A.zn, *w = A.w, *wo = A.wo;
-    if ((e = vcycle_stream<T>(A, v, z, A.act, om, v, A.part, sub_smem, b0)) != cudaSuccess) return e;
+    const ZSlot none{};
+    if ((e = vcycle_stream<T>(A, v, kF32 ? A.q : z, A.act, om, v, A.part, sub_smem, b0, kF32 ? slot(nullptr, 0) : none)) !=
+        cudaSuccess)
+      return e;
     // partial slots per sample of <v, z> (written by the V-cycle's last sweep: the vectorised one for
     // FP32 with V(1,1), the row-mapped one otherwise; one slot when the sub-cycle does it all)
     const int nchd = A.Ls ? ((sizeof(T) == sizeof(float) && A.nu == 1) ? tiles_vec(n) : nt) : 1;
@@ -2291,28 +2416,40 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     LAUNCH_CHECK();
     if ((e = open_while(b0, b1, hi)) != cudaSuccess) return e;
     for (int half = 0; half < 2; ++half) {
-      const int nq = launch_minres_q<T>(n, B, A.act, A.ss, A.wx[0], A.wy[0], s.lamH, s.lam_stride, z, zn, wo, w, A.xi,
-                                        A.q, A.part, nullptr, b1, A.rx, A.ry, A.rd);
+      int nq = 0;
       ++tl_launches;
+      if constexpr (kF32) {
+        nq = launch_minres_q4(n, B, A.act, A.ss, A.wx[0], A.wy[0], slot(ic, half), A.q, A.part, nullptr, b1, A.rx, A.ry, A.rd);
+      } else {
+        nq = nt;
+        k_minres_q<T><<<B * nt, kThreads, 0, b1>>>(n, B, A.act, A.ss, A.wx[0], A.wy[0], s.lamH, s.lam_stride, z, zn, wo, w,
+                                                  A.xi, A.q, A.part, nullptr);
+        LAUNCH_CHECK();
+        ++tl_launches, k_sc_retire<T><<<gs, 256, 0, b1>>>(B, A.act, A.ss);
+      }
       LAUNCH_CHECK();
-      ++tl_launches, k_sc_retire<T><<<gs, 256, 0, b1>>>(B, A.act, A.ss);
       { T* tt = wo; wo = w; w = tt; }
-      ++tl_launches, k_sc_delta<T><<<gw, 256, 0, b1>>>(B, nq, A.part, A.act, A.ss);
+      ++tl_launches, k_sc_delta<T><<<gw, 256, 0, b1>>>(B, nq, A.part, A.act, A.ss, cnt_i);
       ++tl_launches, launch_minres_v<T>(n, B, A.act, A.ss, A.q, v, vo, b1);
       LAUNCH_CHECK();
       { T* tt = vo; vo = v; v = tt; }
-      if ((e = vcycle_stream<T>(A, v, zn, A.act, om, v, A.part, sub_smem, b1)) != cudaSuccess) return e;
-      if ((e = cudaMemsetAsync(cnt_i, 0, sizeof(int), b1)) != cudaSuccess) return e;
+      if ((e = vcycle_stream<T>(A, v, kF32 ? A.q : zn, A.act, om, v, A.part, sub_smem, b1,
+                                kF32 ? slot(ic, half + 1) : none)) != cudaSuccess)
+        return e;
       ++tl_launches, k_sc_givens<T><<<gw, 256, 0, b1>>>(B, nchd, A.part, A.act, A.ss, cnt_i, ic, half,
                                                        s.max_inner);
       LAUNCH_CHECK();
       { T* tt = z; z = zn; zn = tt; }
     }
+    if constexpr (kF32) {
+      ++tl_launches, k_combine4<true><<<gc, kThreads, 0, b1>>>(n, B, A.ss, A.act, slot(ic, 1), A.wo, A.w, A.xh, A.xl);
+      LAUNCH_CHECK();
+    }
     ++tl_launches, k_cond_inner<<<1, 1, 0, b1>>>(hi, ic, cnt_i, s.max_inner);
     LAUNCH_CHECK();
     if ((e = close_while(b1)) != cudaSuccess) return e;
     // an even number of iterations: the rotating vectors are back where they started
-    ++tl_launches, k_minres_finish<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.ran, A.ss, zn, wo, w, A.xi);
+    if constexpr (!kF32) ++tl_launches, k_minres_finish<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.ran, A.ss, zn, wo, w, A.xi);
     if ((e = outer_pass<T>(s, A, hm, b0)) != cudaSuccess) return e;
     ++tl_launches, k_cond_outer<<<1, 1, 0, b0>>>(ho, oc, cnt_o, s.max_outer);
     LAUNCH_CHECK();
@@ -2327,10 +2464,11 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     if (e != cudaSuccess) return e;
     if (active == 0) break;
     cudaMemcpyAsync(A.ran, A.act, Bz * sizeof(int), cudaMemcpyDeviceToDevice, st);
-    ++tl_launches, k_inner_init<T><<<B * nt, kThreads, 0, st>>>(n, B, A.act, A.ss, A.v, A.vo, A.w, A.wo, A.xi);
+    ++tl_launches, k_inner_init<T><<<B * nt, kThreads, 0, st>>>(n, B, A.act, A.ss, A.v, kF32 ? nullptr : A.vo, A.w, A.wo, A.xi);
     LAUNCH_CHECK();
     T *v = A.v, *vo = A.vo, *z = A.z, *zn = A.zn, *w = A.w, *wo = A.wo;
-    e = vcycle_stream<T>(A, v, z, A.act, om, v, A.part, sub_smem, st);
+    const ZSlot none{};
+    e = vcycle_stream<T>(A, v, kF32 ? A.q : z, A.act, om, v, A.part, sub_smem, st, kF32 ? slot(nullptr, 0) : none);
     if (e != cudaSuccess) return e;
     // partial slots per sample of <v, z> (written by the V-cycle's last sweep: the vectorised one for
     // FP32 with V(1,1), the row-mapped one otherwise; one slot when the sub-cycle does it all)
@@ -2343,32 +2481,41 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
         if ((e = s.probe->next(&pe)) != cudaSuccess) return e;
         cudaEventRecord(pe->first, st);
       }
-      const int nq = launch_minres_q<T>(n, B, A.act, A.ss, A.wx[0], A.wy[0], s.lamH, s.lam_stride, z, zn, wo, w, A.xi,
-                                        A.q, A.part, s.probe ? s.probe->d_bytes : nullptr, st, A.rx, A.ry, A.rd);
+      int nq = nt;
+      unsigned long long* work = s.probe ? s.probe->d_bytes : nullptr;
       ++tl_launches;
+      if constexpr (kF32)
+        nq = launch_minres_q4(n, B, A.act, A.ss, A.wx[0], A.wy[0], slot(nullptr, j), A.q, A.part, work, st, A.rx, A.ry, A.rd);
+      else
+        k_minres_q<T><<<B * nt, kThreads, 0, st>>>(n, B, A.act, A.ss, A.wx[0], A.wy[0], s.lamH, s.lam_stride, z, zn, wo, w,
+                                                  A.xi, A.q, A.part, work);
       LAUNCH_CHECK();
       if (pe) cudaEventRecord(pe->second, st);
-      // samples that converged in the previous Givens step have now applied their update
-      ++tl_launches, k_sc_retire<T><<<gs, 256, 0, st>>>(B, A.act, A.ss);
+      // (FP64 path: samples that converged in the previous Givens step have now applied their update)
+      if constexpr (!kF32) ++tl_launches, k_sc_retire<T><<<gs, 256, 0, st>>>(B, A.act, A.ss);
       { T* tt = wo; wo = w; w = tt; }
-      ++tl_launches, k_sc_delta<T><<<gw, 256, 0, st>>>(B, nq, A.part, A.act, A.ss);
+      ++tl_launches, k_sc_delta<T><<<gw, 256, 0, st>>>(B, nq, A.part, A.act, A.ss, A.count);
       ++tl_launches, launch_minres_v<T>(n, B, A.act, A.ss, A.q, v, vo, st);
       LAUNCH_CHECK();
       { T* tt = vo; vo = v; v = tt; }
-      e = vcycle_stream<T>(A, v, zn, A.act, om, v, A.part, sub_smem, st);
+      e = vcycle_stream<T>(A, v, kF32 ? A.q : zn, A.act, om, v, A.part, sub_smem, st, kF32 ? slot(nullptr, j + 1) : none);
       if (e != cudaSuccess) return e;
-      cudaMemsetAsync(A.count, 0, sizeof(int), st);
       ++tl_launches, k_sc_givens<T><<<gw, 256, 0, st>>>(B, nchd, A.part, A.act, A.ss, A.count);
       LAUNCH_CHECK();
       { T* tt = z; z = zn; zn = tt; }
+      if constexpr (kF32)
+        if ((j + 1) % kBasis == 0) {
+          ++tl_launches, k_combine4<true><<<gc, kThreads, 0, st>>>(n, B, A.ss, A.act, slot(nullptr, j), A.wo, A.w, A.xh, A.xl);
+          LAUNCH_CHECK();
+        }
       if ((j & 3) == 3 || j + 1 == s.max_inner) {
         active = read_count(A.count, st, e);
         if (e != cudaSuccess) return e;
         if (active == 0) break;
       }
     }
-    // apply the pending updates of every sample that ran this step (converged or capped)
-    ++tl_launches, k_minres_finish<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, A.ss, zn, wo, w, A.xi);
+    // FP64 path: apply the pending updates of every sample that ran this step (converged or capped)
+    if constexpr (!kF32) ++tl_launches, k_minres_finish<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, A.ss, zn, wo, w, A.xi);
     LAUNCH_CHECK();
     if ((e = outer_pass<T>(s, A, hm, st)) != cudaSuccess) return e;
   }
