@@ -115,6 +115,7 @@ struct SS {  // per-sample solver scalars
   int act;        // inner MINRES running
   int pend;       // a w/x update is pending
   int iters, outer, flags;
+  int strict;     // reductions of the inner solves are fixed (given, or after a step without progress)
   // FP32 path: coefficients of the inner solution and of the directions w_{j-1}, w_{j-2} over the vectors z of
   // iterations j0 .. j0 + nb - 1 and (last two) the directions stored by the last combination
   float cxs[kBasis + 2], cw1[kBasis + 2], cw2[kBasis + 2];
@@ -326,7 +327,7 @@ __device__ __forceinline__ int warp_sample() { return (int)((blockIdx.x * blockD
 
 template <typename T>
 __global__ void k_sc_start(int B, int n, const double* sigma, int sig_stride, int nch, const double* part,
-                           SS<T>* ss) {
+                           SS<T>* ss, int strict) {
   const int b = warp_sample();
   if (b >= B) return;
   double t[1];
@@ -344,6 +345,7 @@ __global__ void k_sc_start(int B, int n, const double* sigma, int sig_stride, in
   S.pend = 0;
   S.iters = 0;
   S.outer = 0;
+  S.strict = strict;
 }
 
 // a refinement step of sample S ends with residual norm rnew and ||x|| = xn
@@ -352,8 +354,12 @@ __device__ __forceinline__ void outer_step_done(SS<T>& S, double rnew, double xn
   S.xnorm = xn;
   // No progress: stop refining.  Not on the first step: on fine meshes the FP32 rounding of the
   // first inner solution alone leaves an FP64 residual above ||b|| (the operator amplifies its
-  // high-frequency part by O(h^-2)); the next step removes it.
-  if (S.outer >= 1 && !(rnew < 0.5 * S.rnorm)) S.act_outer = 0;
+  // high-frequency part by O(h^-2)); the next step removes it.  A sample whose shift nearly meets the
+  // eigenvalue needs more of each solve than the reductions chosen from the residual ask for: it first goes on with a fixed one.
+  if (S.outer >= 1 && !(rnew < 0.5 * S.rnorm)) {
+    if (S.strict) S.act_outer = 0;
+    S.strict = 1;
+  }
   S.rnorm = rnew;
   S.rs = T(1.0 / rnew);
   S.outer += 1;
@@ -397,7 +403,7 @@ __global__ void k_sc_outer_begin(int B, int n, const double* sigma, int sig_stri
   const double kn = knorm_of(S, n, sigma[(size_t)b * sig_stride]);
   const double target = residual_target(tol_lin, S.bnorm, kn, S.xnorm, 16.0);
   const int a = S.act_outer && (S.rnorm > target);
-  S.tol = T(tol_inner > 0.0 ? tol_inner : inner_reduction(n, S.outer, S.rnorm, S.bnorm, target));
+  S.tol = T(tol_inner > 0.0 ? tol_inner : S.strict ? 1e-5 : inner_reduction(n, S.outer, S.rnorm, S.bnorm, target));
   if (!a) S.act_outer = 0;
   S.act = a;
   act[b] = a;
@@ -2376,7 +2382,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     ++tl_launches, k_zero<double><<<grid1(Bz * V0), 256, 0, st>>>(Bz * V0, A.x64);
   }
   LAUNCH_CHECK();
-  ++tl_launches, k_sc_start<T><<<gw, 256, 0, st>>>(B, n, s.lamH, s.lam_stride, nts, A.part, A.ss);
+  ++tl_launches, k_sc_start<T><<<gw, 256, 0, st>>>(B, n, s.lamH, s.lam_stride, nts, A.part, A.ss, s.tol_inner > 0.0);
   LAUNCH_CHECK();
   if (sg) {
     // ---- refinement loop as nested WHILE nodes: no host reads.  The inner loop runs iterations in
