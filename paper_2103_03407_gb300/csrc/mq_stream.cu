@@ -1620,6 +1620,207 @@ __global__ void k_prolong_smooth1_4(int n, int B, const int* __restrict__ act, c
   if (DOT) tile_partials<1, float>(acc, part, (size_t)b * nt + ch);
 }
 
+// ---- the V(1,1) sweeps on large launches: a thread walks kRows rows (down: kRows coarse rows) of its columns and
+// keeps a window of rows in registers.  The kernels above read, convert and multiply every row three times
+// (up: 3 rows of t per row of nodes; down: 5 rows of x1 per coarse row), which left them bound by
+// instruction issue; a window of four rows needs 1.5 rows of t per row and 2.75 rows of x1 per coarse row, and
+// the residual on the odd rows is shared by the two coarse rows beside it.  Values are formed by the
+// same expressions (only the partial sums of <v, z> are grouped differently).  128 samples of mesh 1/1024: 70.8 ->
+// 65.0 ms (66.4 without the bound of four blocks per SM, 65.9 with two rows), 2,048 of mesh 1/256: 61.6 -> 56.1 ms.
+constexpr int kRows = 4;
+
+// CTAs per sample: column groups x groups of kRows rows (down: of coarse rows)
+__host__ __device__ inline int tiles_rows(int n) {
+  const long t = (long)((n - 1 + kRows - 1) / kRows) * (n / kVec);
+  return (int)((t + kThreads - 1) / kThreads);
+}
+__host__ __device__ inline int tiles_pair_rows(int m) {
+  const long t = (long)((m - 1 + kRows - 1) / kRows) * (m / 2);
+  return (int)((t + kThreads - 1) / kThreads);
+}
+
+// the fewest nodes of a launch that uses them: below, a quarter of the threads with longer chains lose (all launches
+// by rows: 2^23 nodes 3 to 5 % slower, 2^18 12 to 15 %; from 2^24 nodes on 2 to 9 % faster)
+constexpr long kRowsMinNodes = 1L << 24;
+inline bool up_by_rows(int n, int B) { return (long)B * n * n >= kRowsMinNodes; }
+inline int tiles_up(int n, int B) { return up_by_rows(n, B) ? tiles_rows(n) : tiles_vec(n); }
+inline bool down_by_rows(int m, int B) { return (long)B * 4 * m * m >= kRowsMinNodes; }
+
+template <bool DOT, typename WT, bool RX = false>
+__global__ void __launch_bounds__(kThreads, 4) k_prolong_smooth1_rows(
+    int n, int B, const int* __restrict__ act, const WT* __restrict__ wx, const WT* __restrict__ wy,
+    const WT* __restrict__ dinv, const float* __restrict__ bb, const float* __restrict__ xc, int ldc, float* out,
+    double* part, ZSlot zs, const WT* __restrict__ dr = nullptr) {
+  const int nt = tiles_rows(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  if (b >= B || !act[b]) return;
+  const int ld = sld(n), lgp = ilog2(n) - 2, mh = n >> 1;
+  const size_t off = (size_t)b * ssz(n);
+  float* __restrict__ O = (zs.base ? zs.get() : out) + off;
+  float acc[1] = {0.0f};
+  const int g = ch * kThreads + threadIdx.x;
+  const int j0 = (g >> lgp) * kRows + 1, c0 = (g & ((1 << lgp) - 1)) * kVec;
+  if (j0 < n) {
+    const float* __restrict__ XC = xc + (size_t)b * (size_t)(mh + 1) * ldc;
+    const bool first = c0 == 0;
+    // coarse rows J0 .. J0 + kRows/2 + 1 under the fine rows j0 - 1 .. j0 + kRows (j0 - 1 is even), columns as in
+    // k_prolong_smooth1_4; rows beyond the mesh (the last group) are clamped, their values unused
+    const int J0 = (j0 - 1) >> 1, cb = (c0 >> 1) - 1;
+    float X[kRows / 2 + 2][4];
+#pragma unroll
+    for (int r = 0; r < kRows / 2 + 2; ++r) {
+      const float* row = XC + (size_t)min(J0 + r, mh) * ldc + cb;
+      X[r][0] = first ? 0.0f : row[0];
+#pragma unroll
+      for (int q = 1; q < 4; ++q) X[r][q] = row[q];
+    }
+    // P xc at fine row j0 - 1 + r, column c0 + k (k = -1 .. 4)
+    auto pc = [&](int r, int k) {
+      const int q = ((k + 4) >> 1) - 1, o = k & 1;
+      return 0.5f * (X[r >> 1][q] + X[(r >> 1) + (r & 1)][q + o]);
+    };
+    // t = om D^-1 b + P xc along fine row j0 - 1 + r (r = 0 .. kRows + 1) at columns c0-1 .. c0+4
+    auto trow = [&](int r, float (&t)[kVec + 2], float4& d, float4& rv) {
+      const size_t p = off + (size_t)min(j0 - 1 + r, n) * ld + c0;
+      d = ldw4(dinv + p);
+      rv = ld4(bb + p);
+#pragma unroll
+      for (int k = 0; k < kVec; ++k) t[k + 1] = at(d, k) * at(rv, k) + pc(r, k);
+      if (r >= 1 && r <= kRows) {
+        t[0] = first ? 0.0f : wget<float>(dinv + p - 1) * bb[p - 1] + pc(r, -1);
+        t[kVec + 1] = wget<float>(dinv + p + kVec) * bb[p + kVec] + pc(r, kVec);
+      }
+    };
+    float ts[kVec + 2], tr[kVec + 2], tn[kVec + 2];
+    float4 dc, rc, dn, rn;
+    trow(0, ts, dn, rn);
+    trow(1, tr, dc, rc);
+    float4 ys = ldw4(wy + off + (size_t)(j0 - 1) * ld + c0);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      trow(r + 2, tn, dn, rn);
+      const int j = min(j0 + r, n);
+      const size_t p = off + (size_t)j * ld + c0;
+      const float4 wc = ldw4(wx + p), yc = ldw4(wy + p);
+      const float wwest = first ? 0.0f : wget<float>(wx + p - 1);
+      const float4 drc = RX ? ldw4(dr + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float o[kVec];
+#pragma unroll
+      for (int k = 0; k < kVec; ++k) {
+        const float tp = tr[k + 1];
+        const float wwv = k > 0 ? at(wc, k - 1) : wwest;
+        float ax = at(wc, k) * (tp - tr[k + 2]) + wwv * (tp - tr[k]) + at(yc, k) * (tp - tn[k + 1]) +
+                   at(ys, k) * (tp - ts[k + 1]);
+        if (RX) ax += at(drc, k) * tp;
+        o[k] = (first && k == 0) ? 0.0f : tp + at(dc, k) * (at(rc, k) - ax);
+      }
+      if (j < n) {
+        st4(O + (size_t)j * ld + c0, make_float4(o[0], o[1], o[2], o[3]));
+        if (DOT) acc[0] += rc.x * o[0] + rc.y * o[1] + rc.z * o[2] + rc.w * o[3];
+      }
+#pragma unroll
+      for (int k = 0; k < kVec + 2; ++k) {
+        ts[k] = tr[k];
+        tr[k] = tn[k];
+      }
+      dc = dn;
+      rc = rn;
+      ys = yc;
+    }
+  }
+  if (DOT) tile_partials<1, float>(acc, part, (size_t)b * nt + ch);
+}
+
+template <typename WT, bool RX = false>
+__global__ void __launch_bounds__(kThreads, 4) k_restrict1_rows(int n, int B, const int* __restrict__ act,
+                                                             const WT* __restrict__ wx, const WT* __restrict__ wy,
+                                                             const WT* __restrict__ dinv, const float* __restrict__ bb,
+                                                             float* __restrict__ bc, int ldo,
+                                                             const WT* __restrict__ dr = nullptr) {
+  const int m = n / 2;
+  const int nt = tiles_pair_rows(m);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  if (b >= B || !act[b]) return;
+  const int g = ch * kThreads + threadIdx.x, lgp = ilog2(m) - 1;
+  const int Jb = (g >> lgp) * kRows + 1, t = g & ((1 << lgp) - 1);
+  if (Jb > m - 1) return;
+  const int ld = sld(n), c = 4 * t;
+  const size_t off = (size_t)b * ssz(n);
+  // columns c-2 .. c+4 (index 0..6) of x1 = om D^-1 b and of b on fine row i; c-2 .. c+3 (index 0..5) of the
+  // weights.  Rows beyond the mesh (the last group) are clamped, their values unused.
+  auto xrow = [&](int i, float (&x)[7], float (&r)[7]) {
+    const size_t p = off + (size_t)min(i, n) * ld + c;
+    const float4 d1 = ldw4(dinv + p), r1 = ld4(bb + p);
+    const float dl0 = c ? wget<float>(dinv + p - 2) : 0.0f, dl1 = c ? wget<float>(dinv + p - 1) : 0.0f;
+    const float2 rl = c ? *reinterpret_cast<const float2*>(bb + p - 2) : make_float2(0.f, 0.f);
+    const float dv[7] = {dl0, dl1, d1.x, d1.y, d1.z, d1.w, wget<float>(dinv + p + 4)};
+    const float rv[7] = {rl.x, rl.y, r1.x, r1.y, r1.z, r1.w, bb[p + 4]};
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      x[q] = dv[q] * rv[q];
+      r[q] = rv[q];
+    }
+  };
+  auto wrow = [&](const WT* __restrict__ w, int i, float (&v)[6]) {
+    const size_t p = off + (size_t)min(i, n) * ld + c;
+    const float4 a = ldw4(w + p);
+    v[0] = c ? wget<float>(w + p - 2) : 0.0f;
+    v[1] = c ? wget<float>(w + p - 1) : 0.0f;
+    v[2] = a.x, v[3] = a.y, v[4] = a.z, v[5] = a.w;
+  };
+  float xs[7], xm[7], xn[7], rm[7], rn[7], ys[6], yc[6];
+  int i = 2 * Jb - 1;
+  xrow(i - 1, xs, rn);
+  xrow(i, xm, rm);
+  wrow(wy, i - 1, ys);
+  // residual b - A x1 on row i at index 1..5; the window moves to row i + 1
+  auto residual = [&](float (&e)[6]) {
+    float w[6], d[6];
+    xrow(i + 1, xn, rn);
+    wrow(wx, i, w);
+    wrow(wy, i, yc);
+    if (RX) wrow(dr, i, d);
+#pragma unroll
+    for (int q = 1; q < 6; ++q) {
+      const float xq = xm[q];
+      float ax = w[q] * (xq - xm[q + 1]) + w[q - 1] * (xq - xm[q - 1]) + yc[q] * (xq - xn[q]) + ys[q] * (xq - xs[q]);
+      if (RX) ax += d[q] * xq;
+      e[q] = rm[q] - ax;
+    }
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      xs[q] = xm[q];
+      xm[q] = xn[q];
+      rm[q] = rn[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) ys[q] = yc[q];
+    ++i;
+  };
+  float lo[6], mi[6], hi[6];
+  residual(lo);
+  float* __restrict__ C = bc + (size_t)b * (size_t)(m + 1) * ldo;
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) {
+    residual(mi);
+    residual(hi);
+    const int J = Jb + r;
+    if (J < m) {
+      // coarse node 2t (fine column c: q = 2) and 2t + 1 (fine column c + 2: q = 4)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int q = 2 + 2 * h;
+        const int I = 2 * t + h;
+        if (I >= 1)
+          C[(size_t)J * ldo + I] =
+              mi[q] + 0.5f * ((mi[q + 1] + mi[q - 1]) + (hi[q] + lo[q]) + (hi[q + 1] + lo[q - 1]));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) lo[q] = hi[q];
+  }
+}
+
 // K2: v_new = q - c1 v - c2 v_old (into vo).  z_j stays unnormalised: the next pending update
 // scales it by 1 / gamma_j (saves a read and a write of z per step)
 template <typename T>
@@ -2068,7 +2269,15 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
       const int ldo = (l + 1 < A.Ls) ? sld(nl / 2) : nl / 2 + 1;
       if constexpr (sizeof(T) == sizeof(float)) {
         if (A.hx[l]) {
-          if (A.hr[l])
+          if (down_by_rows(nl / 2, B)) {
+            ++tl_launches;
+            if (A.hr[l])
+              k_restrict1_rows<__nv_bfloat16, true><<<B * tiles_pair_rows(nl / 2), kThreads, 0, st>>>(
+                  nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, bc, ldo, A.hr[l]);
+            else
+              k_restrict1_rows<__nv_bfloat16><<<B * tiles_pair_rows(nl / 2), kThreads, 0, st>>>(
+                  nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, bc, ldo);
+          } else if (A.hr[l])
             ++tl_launches, k_restrict1_4<__nv_bfloat16, true><<<B * tiles_pairs(nl / 2), kThreads, 0, st>>>(
                 nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, bc, ldo, A.hr[l]);
           else
@@ -2097,19 +2306,37 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
       const T* xc = (l + 1 < A.Ls) ? A.x[l + 1] : A.xsub;
       const int ldc = (l + 1 < A.Ls) ? sld(nl / 2) : nl / 2 + 1;
       if constexpr (sizeof(T) == sizeof(float)) {
-        if (A.hr[l]) {
+        const ZSlot to = l ? plain : zs;
+        if (up_by_rows(nl, B)) {
+          const int nr = B * tiles_rows(nl);
+          ++tl_launches;
+          if (l == 0 && dotv) {  // (dotv is the right-hand side itself)
+            if (A.hr[l])
+              k_prolong_smooth1_rows<true, __nv_bfloat16, true><<<nr, kThreads, 0, st>>>(
+                  nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, part, to, A.hr[l]);
+            else
+              k_prolong_smooth1_rows<true, __nv_bfloat16><<<nr, kThreads, 0, st>>>(nl, B, act, A.hx[l], A.hy[l], A.hd[l],
+                                                                                 b, xc, ldc, xa, part, to);
+          } else if (A.hr[l]) {
+            k_prolong_smooth1_rows<false, __nv_bfloat16, true><<<nr, kThreads, 0, st>>>(
+                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, to, A.hr[l]);
+          } else {
+            k_prolong_smooth1_rows<false, __nv_bfloat16><<<nr, kThreads, 0, st>>>(nl, B, act, A.hx[l], A.hy[l], A.hd[l],
+                                                                                b, xc, ldc, xa, nullptr, to);
+          }
+        } else if (A.hr[l]) {
           if (l == 0 && dotv)
             ++tl_launches, k_prolong_smooth1_4<true, __nv_bfloat16, true><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, l ? plain : zs, A.hr[l]);
+                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, to, A.hr[l]);
           else
             ++tl_launches, k_prolong_smooth1_4<false, __nv_bfloat16, true><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, l ? plain : zs, A.hr[l]);
+                nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, to, A.hr[l]);
         } else if (l == 0 && dotv) {
           ++tl_launches, k_prolong_smooth1_4<true, __nv_bfloat16><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, l ? plain : zs);
+              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, dotv, part, to);
         } else {
           ++tl_launches, k_prolong_smooth1_4<false, __nv_bfloat16><<<B * tiles_vec(nl), kThreads, 0, st>>>(
-              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, l ? plain : zs);
+              nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, xc, ldc, xa, nullptr, nullptr, to);
         }
       } else {
         if (l == 0 && dotv)
@@ -2414,7 +2641,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
       return e;
     // partial slots per sample of <v, z> (written by the V-cycle's last sweep: the vectorised one for
     // FP32 with V(1,1), the row-mapped one otherwise; one slot when the sub-cycle does it all)
-    const int nchd = A.Ls ? ((sizeof(T) == sizeof(float) && A.nu == 1) ? tiles_vec(n) : nt) : 1;
+    const int nchd = A.Ls ? ((sizeof(T) == sizeof(float) && A.nu == 1) ? tiles_up(n, B) : nt) : 1;
     ++tl_launches, k_sc_gamma0<T><<<gw, 256, 0, b0>>>(B, nchd, A.part, A.act, A.ss);
     LAUNCH_CHECK();
     if ((e = make_handle(b0, &hi)) != cudaSuccess) return e;
@@ -2478,7 +2705,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     if (e != cudaSuccess) return e;
     // partial slots per sample of <v, z> (written by the V-cycle's last sweep: the vectorised one for
     // FP32 with V(1,1), the row-mapped one otherwise; one slot when the sub-cycle does it all)
-    const int nchd = A.Ls ? ((sizeof(T) == sizeof(float) && A.nu == 1) ? tiles_vec(n) : nt) : 1;
+    const int nchd = A.Ls ? ((sizeof(T) == sizeof(float) && A.nu == 1) ? tiles_up(n, B) : nt) : 1;
     ++tl_launches, k_sc_gamma0<T><<<gw, 256, 0, st>>>(B, nchd, A.part, A.act, A.ss);
     LAUNCH_CHECK();
     for (int j = 0; j < s.max_inner; ++j) {
