@@ -97,7 +97,9 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   // a solve on the coarse mesh itself may fall back to FP64 (see mq_sample.cu)
   const bool near = mixed && ((d_a_fine && n_fine == n_coarse) || (d_a_prev && n_prev == n_coarse));
   const size_t fslab = near ? mq::sample_fallback_bytes(n_coarse, 0) : 0;
-  if (slab + fslab > kNoAllocScratchBytes) return MQ_EINVAL;  // one block's workspace exceeds the fixed array
+  // one block's workspace, with every solve the meshes allow, has to fit in the fixed array (FP64: fine meshes up to 1/256)
+  const size_t full = mq::sample_slab_bytes(n_fine, n_coarse, n_prev, mixed, 0, 0);
+  if (std::max(slab + fslab, full) > kNoAllocScratchBytes || (!mixed && n_fine > 256)) return MQ_EINVAL;
 
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kMaxDevices) return MQ_ECUDA;
