@@ -497,8 +497,8 @@ def stream_bytes(wl, level, st, prec, samples):
 # ncu DRAM traffic of the per-sample kernel's launch on a level (one launch of the benchmark's size:
 # level 1 of the six-level workload, 4,096 samples; summarised under profiles/), valid only for the
 # kernel source it was measured on
-SAMPLE_KERNEL_TRAFFIC = {"source_sha256": "5cfd76dfb86a1cec2d451c0ddf255b8e942fe61bd808a6d51ab2ab5e09d1f482",
-                         "level": 1, "precision": "mixed", "bytes_per_launch": 141.982720e6 + 95.710208e6}
+SAMPLE_KERNEL_TRAFFIC = {"source_sha256": "cae22eaf7366879df4462bca057dc450f994f83a49f22a9cea16a178ae050441",
+                         "level": 1, "precision": "mixed", "bytes_per_launch": 141.686016e6 + 93.218816e6}
 
 
 # ncu DRAM traffic of the operator sweep k_minres_q per algorithmic byte: one launch (4 arrays per node) on mesh

@@ -436,8 +436,8 @@ int stream_threshold(const mq_ctx* c) {
 }
 
 // Threads per CTA of the per-sample kernel: n_fine is the largest mesh solved inside the kernel
-// (0: coarse eigensolves only).  Meshes up to 1/16 run with two warps: their workspace (~24 KB)
-// lets seven samples share an SM, which hides the barrier latency of the small phases better
+// (0: coarse eigensolves only).  Meshes up to 1/16 run with two warps: their workspace (~23 KB)
+// lets eight samples share an SM, which hides the barrier latency of the small phases better
 // than more threads per sample (measured on GB300).
 int threads_for(int n_fine, int n_coarse) {
   if (n_fine > 0 && n_fine <= 16) return 64;
