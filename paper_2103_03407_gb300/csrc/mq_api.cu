@@ -1110,14 +1110,12 @@ mq_status set_terms(mq_ctx* c, double a0, int32_t s_max, int32_t family, double 
     const int kp = mq::tc_pad_k(k1m);
     // start[v] .. start[v + 1] lists the terms of k1 = v / 2 + 1 with even (v even) or odd k2
     std::vector<int> start(2 * kp + 1, 0);
-    std::vector<int2> list;
-    list.reserve(m);
-    for (int v = 0; v < 2 * kp; ++v) {
-      start[v] = (int)list.size();
-      for (int t = 0; t < m; ++t)
-        if (k1[t] == v / 2 + 1 && (k2[t] & 1) == (v & 1)) list.push_back(make_int2(t, k2[t]));
-    }
-    start[2 * kp] = (int)list.size();
+    std::vector<int2> list(m);
+    auto slot = [&](int t) { return 2 * (k1[t] - 1) + (k2[t] & 1); };
+    for (int t = 0; t < m; ++t) ++start[slot(t) + 1];
+    for (int v = 0; v < 2 * kp; ++v) start[v + 1] += start[v];
+    std::vector<int> at(start.begin(), start.end() - 1);
+    for (int t = 0; t < m; ++t) list[at[slot(t)]++] = make_int2(t, k2[t]);
     MQ_CUDA(c, cudaMalloc(&c->d_k1start, start.size() * sizeof(int)));
     MQ_CUDA(c, cudaMalloc(&c->d_tlist, std::max<size_t>(list.size(), 1) * sizeof(int2)));
     MQ_CUDA(c, cudaMemcpy(c->d_k1start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice));
