@@ -418,22 +418,25 @@ def cpu_baseline(wl, seconds_budget, zs, ds):
 # ------------------------------------------------------------------------------------------
 # Roofline models.
 #
-# Per-sample kernel (one CTA per sample, workspace on chip): bounded by the FP64 units, whose
-# peak is 152 SMs x 2 FP64 FMA lanes per cycle x 2 flops x the SM clock.  FP64 operations
-# counted from the kernel source (a fused multiply-add counts two):
+# Per-sample kernel (one CTA per sample, workspace on chip): on the FP64 path bounded by the FP64 units,
+# whose peak is 152 SMs x 2 FP64 FMA lanes per cycle x 2 flops x the SM clock.  FP64 operations
+# counted from the FP64 kernel's source (a fused multiply-add counts two).  The mixed path does the same work
+# beyond FP32 in double-floats on the FP32 units: its line counts the FP64 operations they stand for, and is bound
+# by the latency of short phases rather than by the FP64 rate it is set against.
 #   coarse LOBPCG: 73 per coarse unknown and iteration (residual 6, A w and M w 19, Gram matrix
 #   24, update of x, Ax, Mx, p, Ap, Mp 24) + 46 per unknown and eigensolve (two operator
 #   applications with normalisation);
 #   fine solve with FP32 inner iterations: 23 per fine unknown (interpolation and right-hand side
 #   19, FP64 edge weights of the preconditioner 4) + 40 per unknown and refinement step (solution
 #   update 2, FP64 residual with the Rayleigh-quotient partials 38);
-#   fine solve with FP64 inner iterations (FP64 path, same-mesh solves): + 135 per unknown and
+#   fine solve with FP64 inner iterations (FP64 path): + 135 per unknown and
 #   inner iteration (operator 24, MINRES updates 12, V-cycle 99).
 FP64_EIG_IT, FP64_EIG_CALL, FP64_FINE_SETUP, FP64_FINE_OUTER, FP64_INNER = 73, 46, 23, 40, 135
 
 
-def stream_min_default(prec):
-    return 32 if prec == "mixed" else 256
+def streams_by_default(prec, n, samples):
+    """Whether the library solves fine meshes 1/n of a call of that many samples in the streaming tier."""
+    return n >= 32 if prec == "mixed" else n >= 128 or (n >= 32 and samples * n * n >= 1 << 21)
 
 
 def percta_fp64_flops(wl, level, st, prec, samples):
@@ -449,26 +452,19 @@ def percta_fp64_flops(wl, level, st, prec, samples):
         if not (pv.n_fine == nc and pv.s == lv.S):
             solves.append(pv.n_fine)
     I, O = st["fine_iters_mean"], st["outer_iters_mean"]
-    streamed = lv.n_fine >= stream_min_default(prec) and not (lv.n_fine == nc and lv.s == lv.S)
+    streamed = streams_by_default(prec, lv.n_fine, samples) and not (lv.n_fine == nc and lv.s == lv.S)
     for n in solves:
         if streamed and n != nc:
             continue  # batched streaming tier
-        inner64 = prec == "fp64" or n == nc
-        per += (n - 1) ** 2 * (FP64_FINE_SETUP + FP64_FINE_OUTER * O + (FP64_INNER * I if inner64 else 0))
+        per += (n - 1) ** 2 * (FP64_FINE_SETUP + FP64_FINE_OUTER * O + (FP64_INNER * I if prec == "fp64" else 0))
     return per * samples
 
 
-# Streaming tier (fine meshes >= 1/32 mixed): bounded by HBM.  Bytes per fine unknown with every
-# kernel reading and writing each of its arrays once (e = 4 bytes, FP32 inner vectors; the
-# default V(1,1) smoothing of this tier):
-#   per inner MINRES iteration: MINRES sweeps 14 e (operator + pending update 10 e, Lanczos
-#   vector 4 e) + V-cycle 11.5 e on the fine level (restriction of the first sweep's residual
-#   4.25 e, prolongation + sweep + dot 7.25 e) + 10.5 e / 4 and / 16 on the coarser streamed
-#   levels (the on-chip sub-cycle below 1/32 is not counted);
-#   per refinement step: 12 e + 48 bytes (inner start 6 e, final update 5 e, FP64 solution update
-#   e + 16, FP64 residual with FP64 weights e + 32) + one V-cycle;
-#   per solve: 20 e + 72 bytes (clearing 8 e + 16, FP32 and FP64 weights 3 e + 32, interpolation
-#   and right-hand side e + 24, operators of the coarser levels ~8 e).
+# Streaming tier: bounded by HBM.  Bytes per fine unknown with every kernel reading and writing each of
+# its arrays once (the default V(1,1) smoothing of this tier; the on-chip sub-cycle below 1/32 is not
+# counted).  FP64 path (e = 8 bytes): per inner MINRES iteration 14 e (operator + pending update 10 e,
+# Lanczos vector 4 e) + V-cycle 11.5 e on the fine level + 10.5 e / 4 and / 16 on the coarser
+# ones; per refinement step 12 e + 48 + one V-cycle; per solve 20 e + 56.
 def stream_bytes(wl, level, st, prec, samples):
     # bytes per fine node.  Mixed path: per iteration the operator sweep 16, the Lanczos update 16, the vector's share of the
     # combination 4 and the V(1,1) cycle 27 on the finest mesh (restriction 11, prolongation and smoothing
@@ -479,11 +475,11 @@ def stream_bytes(wl, level, st, prec, samples):
     vcyc = 27 * (1 + 1 / 4 + 1 / 16) if prec == "mixed" else 11.5 * e + 10.5 * e * (1 / 4 + 1 / 16)
     I, O = st["fine_iters_mean"], st["outer_iters_mean"]
     solves = []
-    if lv.n_fine >= stream_min_default(prec) and not (lv.n_fine == lv.n_coarse and lv.s == lv.S):
+    if streams_by_default(prec, lv.n_fine, samples) and not (lv.n_fine == lv.n_coarse and lv.s == lv.S):
         solves.append(lv.n_fine)
     if level > 0:
         pv = wl.levels[level - 1]
-        if lv.n_fine >= stream_min_default(prec) and pv.n_fine != lv.n_coarse:
+        if streams_by_default(prec, lv.n_fine, samples) and pv.n_fine != lv.n_coarse:
             solves.append(pv.n_fine)
     per = 0.0
     for n in solves:
@@ -578,8 +574,8 @@ def percta_roofline(wl, level, st, prec, ms_per_launch, sm_max_mhz, samples, mea
     traffic = None
     if t["source_sha256"] == _percta_source_hash() and t["level"] == level and t["precision"] == prec:
         traffic = t["bytes_per_launch"]
-    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": traffic,
+    return {"bound": "alu" if prec == "fp64" else "latency", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak, "traffic": traffic,
             "kernel": f"sample_kernel (level {level}: {samples} samples per launch, "
                       f"{ms_per_launch:.2f} ms per launch)",
             "algorithmic_flops": flops,

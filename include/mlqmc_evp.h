@@ -209,7 +209,7 @@ mq_status mq_set_smoothing(mq_ctx* ctx, int32_t nu);
  * the batched streaming tier (one kernel per sweep over all samples of a pass, lockstep across
  * samples); coarser ones run inside the per-sample kernel (one CTA per sample, workspace in
  * shared memory when it fits).  Both tiers compute the same values to rounding.  Default (or
- * stream_min_n = 0): 32 in MQ_PREC_MIXED, 256 in MQ_PREC_FP64. */
+ * stream_min_n = 0): 32 in MQ_PREC_MIXED; in MQ_PREC_FP64 128, or 32 in calls of at least 2^21 fine nodes. */
 mq_status mq_set_tier(mq_ctx* ctx, int32_t stream_min_n);
 
 /* Threads per CTA of the per-sample kernel (one CTA per sample) on level `level` (0 <= level < 64):

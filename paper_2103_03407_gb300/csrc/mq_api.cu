@@ -427,14 +427,6 @@ mq_status check_level_ready(mq_ctx* c, int level) {
   return MQ_OK;
 }
 
-// Default tier threshold (measured on GB300, 4-level workload): with FP32 inner solves the
-// streaming tier wins from 1/32 on (the per-sample kernel fits only two samples of mesh 1/32 per
-// SM); the FP64 path is FP64-throughput bound and keeps the per-sample kernel up to 1/128.
-int stream_threshold(const mq_ctx* c) {
-  if (c->stream_min > 0) return c->stream_min;
-  return c->prec == MQ_PREC_MIXED ? 32 : 256;
-}
-
 // Threads per CTA of the per-sample kernel: n_fine is the largest mesh solved inside the kernel
 // (0: coarse eigensolves only).  Meshes up to 1/16 run with two warps: their workspace (~23 KB)
 // lets eight samples share an SM, which hides the barrier latency of the small phases better
@@ -450,11 +442,13 @@ struct LevelGeom {
   int threads;  // requested threads per CTA of the per-sample kernel (0: default)
   int tier;     // -1: by mesh size; 0: fine solves in the per-sample kernel; 1: streaming tier
   int nu;       // Jacobi sweeps per side of the V-cycle for this level (0: default)
+  long B;       // samples of the call
 };
 
 LevelGeom geom(const mq_ctx* c, int level) {
   const mq_level& lv = c->levels[level];
   LevelGeom g{};
+  g.B = 1;
   g.nf = lv.n_fine;
   g.nc = lv.n_coarse;
   g.s = lv.s;
@@ -481,7 +475,14 @@ bool streams(const mq_ctx* c, const LevelGeom& g) {
   if (g.direct_f) return false;
   if (c->family == 2 && !(c->prec == MQ_PREC_MIXED && stream_nu(c, g) == 1)) return false;
   if (g.tier >= 0) return g.tier == 1;
-  return g.nf >= stream_threshold(c);
+  if (c->stream_min > 0) return g.nf >= c->stream_min;
+  // (measured on GB300, 4-level workload) with FP32 inner solves the streaming tier wins from 1/32 on
+  if (c->prec == MQ_PREC_MIXED) return g.nf >= 32;
+  // FP64: from mesh 1/128 on the workspace of the per-sample kernel (global memory) costs more than the launches
+  // of the streaming tier for any number of samples (mesh 1/128: 17.2 / 5.3 ms with 2 samples, 123 / 87 with
+  // 1,024); meshes 1/64 and 1/32 need 2^21 nodes in the call to hide them (mesh 1/64, coarse mesh 1/16: 4.7 / 5.3
+  // ms with 152 samples, 15.1 / 12.3 with 608; mesh 1/32: 3.2 / 4.7 ms with 608, 12.3 / 10.5 with 2,048)
+  return g.nf >= 128 || (g.nf >= 32 && g.B * g.nf * g.nf >= 1L << 21);
 }
 
 // Points per warm-start chain: as long as possible with the chains a multiple of the resident blocks (occ per
@@ -818,9 +819,10 @@ mq_status eval_level_impl(mq_ctx* c, int level, uint32_t k0, uint32_t k1, double
   const mq_level& lv = c->levels[level];
   if (k1 < k0 || k1 > lv.N) return fail(c, MQ_EINVAL, "point range [%u, %u) outside [0, %u)", k0, k1, lv.N);
   MQ_CUDA(c, cudaSetDevice(c->device));
-  const LevelGeom g = geom(c, level);
+  LevelGeom g = geom(c, level);
   const int R = lv.R;
   const int npts = (int)(k1 - k0);
+  g.B = (long)R * npts;
   c->stats = mq_stats{};
   if (npts == 0) return MQ_OK;
   if (c->reuse && level >= 1) {
