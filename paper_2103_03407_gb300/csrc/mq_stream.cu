@@ -17,7 +17,8 @@
 //     step (the last one at the finest level also forms <v, z>).  nu = 1: two kernels per level --
 //     the residual of x1 = om D^-1 b restricted, prolongation + correction + one smoothing step
 //     (+ <v, z>).  The meshes 1/32 .. 1/2 of each sample run inside one CTA in shared memory;
-//   * FP64 iterative refinement around the inner solve and the FP64 Rayleigh quotient.
+//   * iterative refinement around the inner solve and the Rayleigh quotient, in FP64 or (FP32 path) in
+//     double-floats.
 // Partial sums of every reduction are written per (sample, tile) and added in fixed order by
 // the scalar kernels: results do not depend on scheduling.  Converged samples are masked out.
 #include <cuda_bf16.h>
