@@ -116,7 +116,7 @@ struct SS {  // per-sample solver scalars
   int act;        // inner MINRES running
   int pend;       // a w/x update is pending
   int iters, outer, flags;
-  int strict;     // reductions of the inner solves are fixed (given, or after a step without progress)
+  int strict;     // 0: reductions of the inner solves are chosen; k: fixed, and the k-th step without progress is the last
   // FP32 path: coefficients of the inner solution and of the directions w_{j-1}, w_{j-2} over the vectors z of
   // iterations j0 .. j0 + nb - 1 and (last two) the directions stored by the last combination
   float cxs[kBasis + 2], cw1[kBasis + 2], cw2[kBasis + 2];
@@ -356,10 +356,13 @@ __device__ __forceinline__ void outer_step_done(SS<T>& S, double rnew, double xn
   // No progress: stop refining.  Not on the first step: on fine meshes the FP32 rounding of the
   // first inner solution alone leaves an FP64 residual above ||b|| (the operator amplifies its
   // high-frequency part by O(h^-2)); the next step removes it.  A sample whose shift nearly meets the
-  // eigenvalue needs more of each solve than the reductions chosen from the residual ask for: it first goes on with a fixed one.
+  // eigenvalue needs more of each solve than the reductions chosen from the residual ask for: it first goes on with fixed ones
+  // and three more such steps, since the near-null part that a step adds to x brings rounding of its own.
   if (S.outer >= 1 && !(rnew < 0.5 * S.rnorm)) {
-    if (S.strict) S.act_outer = 0;
-    S.strict = 1;
+    if (S.strict == 1)
+      S.act_outer = 0;
+    else
+      S.strict = S.strict ? S.strict - 1 : 4;
   }
   S.rnorm = rnew;
   S.rs = T(1.0 / rnew);
