@@ -922,6 +922,79 @@ __global__ void k_minres_q4(int n, int B, const int* __restrict__ act, const SS<
   tile_partials<1, float>(acc, part, (size_t)b * nt + ch);
 }
 
+// The same operator application on large launches: a thread walks kQRows rows of its four columns with a window of
+// rows of z and of w_y in registers (see the V(1,1) sweeps by rows).  16 samples of
+// mesh 1/1024: 66 -> 51 us in ncu; 128 samples, whole call: 65.1 -> 61.5 ms.  From 2^24 nodes on, as those.
+constexpr int kQRows = 4;
+__host__ __device__ inline int tiles_qrows(int n) {
+  const long t = (long)((n - 1 + kQRows - 1) / kQRows) * (n / kVec);
+  return (int)((t + kThreads - 1) / kThreads);
+}
+__global__ void __launch_bounds__(kThreads, 4) k_minres_q_rows(int n, int B, const int* __restrict__ act,
+                                                               const SS<float>* __restrict__ ss,
+                                                               const float* __restrict__ wx,
+                                                               const float* __restrict__ wy, ZSlot zs,
+                                                               float* __restrict__ qv, double* part,
+                                                               unsigned long long* work) {
+  const int nt = tiles_qrows(n);
+  const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
+  if (b >= B || !act[b]) return;
+  const float sigm = ss[b].sigm, ig = ss[b].ig;
+  const float* __restrict__ z = zs.get();
+  const int ld = sld(n), lgp = ilog2(n) - 2;
+  const size_t off = (size_t)b * ssz(n);
+  // algorithmic bytes: one count per sample
+  if (work && threadIdx.x == 0 && ch == 0) atomicAdd(work, (unsigned long long)(n - 1) * (n - 1) * 4 * sizeof(float));
+  float acc[1] = {0.0f};
+  const int g = ch * kThreads + threadIdx.x;
+  const int j0 = (g >> lgp) * kQRows + 1, c0 = (g & ((1 << lgp) - 1)) * kVec;
+  if (j0 < n) {
+    const bool first = c0 == 0;
+    // columns c0-1 .. c0+4 (index 0..5) of z along row j (rows beyond the mesh are clamped, their values unused)
+    auto zrow = [&](int j, float (&v)[kVec + 2]) {
+      const float* p = z + off + (size_t)min(j, n) * ld + c0;
+      const float4 a = ld4(p);
+      v[0] = first ? 0.0f : p[-1];
+      v[1] = a.x, v[2] = a.y, v[3] = a.z, v[4] = a.w;
+      v[5] = p[kVec];
+    };
+    float zsr[kVec + 2], zc[kVec + 2], zn[kVec + 2];
+    zrow(j0 - 1, zsr);
+    zrow(j0, zc);
+    float4 ys = ld4(wy + off + (size_t)(j0 - 1) * ld + c0);
+#pragma unroll
+    for (int r = 0; r < kQRows; ++r) {
+      const int j = min(j0 + r, n);
+      const size_t p = off + (size_t)j * ld + c0;
+      zrow(j0 + r + 1, zn);
+      const float4 wc = ld4(wx + p), yc = ld4(wy + p);
+      const float wwest = first ? 0.0f : wx[p - 1];
+      float q[kVec], dot = 0.0f;
+#pragma unroll
+      for (int k = 0; k < kVec; ++k) {
+        const float xp = zc[k + 1], xe = zc[k + 2], xw = zc[k], xn = zn[k + 1], xs = zsr[k + 1];
+        const float wwv = k > 0 ? at(wc, k - 1) : wwest;
+        const float st = at(wc, k) * (xp - xe) + wwv * (xp - xw) + at(yc, k) * (xp - xn) + at(ys, k) * (xp - xs);
+        const float ms = 6.0f * xp + (xe + xw) + (xn + xs) + (zn[k + 2] + zsr[k]);
+        const float kz = (st - sigm * ms) * ig;
+        q[k] = (first && k == 0) ? 0.0f : kz;
+        dot += q[k] * xp;
+      }
+      if (j < n) {
+        st4(qv + p, make_float4(q[0], q[1], q[2], q[3]));
+        acc[0] += dot;
+      }
+#pragma unroll
+      for (int k = 0; k < kVec + 2; ++k) {
+        zsr[k] = zc[k];
+        zc[k] = zn[k];
+      }
+      ys = yc;
+    }
+  }
+  tile_partials<1, float>(acc, part, (size_t)b * nt + ch);
+}
+
 // K2, vectorised: v_new = q - c1 v - c2 v_old (into vo)
 __global__ void k_minres_v4(int n, int B, const int* __restrict__ act, const SS<float>* __restrict__ ss,
                             const float* __restrict__ q, const float* __restrict__ v, float* __restrict__ vo) {
@@ -2135,6 +2208,10 @@ __global__ void k_set_int(int B, int* p, int v) {
 int launch_minres_q4(int n, int B, const int* act, const SS<float>* ss, const float* wx, const float* wy, ZSlot zs,
                      float* q, double* part, unsigned long long* work, cudaStream_t st, const float* rx, const float* ry,
                      const float* rd) {
+  if (!rx && (long)B * n * n >= 1L << 24) {
+    k_minres_q_rows<<<B * tiles_qrows(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, zs, q, part, work);
+    return tiles_qrows(n);
+  }
   if (rx)
     k_minres_q4<true><<<B * tiles_vec(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, zs, q, part, work, rx, ry, rd);
   else

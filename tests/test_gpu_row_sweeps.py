@@ -1,6 +1,7 @@
-"""The V(1,1) sweeps by windows of rows (launches with many thread blocks) against the four-node sweeps (few samples) and
+"""The sweeps by windows of rows (launches of at least 2^24 nodes) against the four-node sweeps (few samples) and
 the oracle: the smallest and larger meshes, whose last group of rows is short on every level, one and several
-tiles per sample, only some levels of the cycle by rows (sample counts between the limits), and the reaction term.
+tiles per sample, one and several levels of the cycle by rows (sample counts on both sides of the limits), and the
+reaction term.
 
 The sweeps form the same values by the same expressions, so the iterates of both forms agree but for the
 grouping of the sums <v, z>.  Tolerance 1e-12 relative against both, as for the other streamed values at the
@@ -28,10 +29,10 @@ def B():
     return binding
 
 
-@pytest.mark.parametrize("n,nc,family,pts", [(64, 16, 0, 250), (64, 16, 2, 250), (128, 16, 0, 53), (128, 16, 0, 220),
-                                            (256, 32, 0, 27), (256, 32, 2, 14)])
+@pytest.mark.parametrize("n,nc,family,pts", [(64, 16, 0, 1366), (64, 16, 2, 1366), (128, 16, 0, 342), (128, 16, 0, 1366),
+                                            (256, 32, 0, 86), (256, 32, 2, 86)])
 def test_sweeps_by_rows(B, n, nc, family, pts):
-    lv = Level(n, nc, 16, 4, 1024, 3)
+    lv = Level(n, nc, 16, 4, 2048, 3)
     z = lattice.cbc(lv.N, lv.s)
     delta = shifts(n + pts, [lv])[0]
     some = sorted({0, pts // 2, pts - 1})
