@@ -738,7 +738,7 @@ __device__ __noinline__ int lobpcg32(CoarseWS32& ws, int n, double tol, int maxi
         sh->al = al;
         sh->be = be;
         sh->ok = ok;
-        sh->theta = df_add(sh->theta, two_sum(dl, mu));
+        if (ok) sh->theta = df_add(sh->theta, two_sum(dl, mu));
       });
     }
     if (!sh->ok) break;
@@ -1309,7 +1309,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
   }
   __syncthreads();
   const CoarseVec uH = e32 ? CoarseVec{nullptr, cws32.xh, cws32.xl} : CoarseVec{cws.uprev, nullptr, nullptr};
-  double lam_prev = 0.0;  // coarse eigenvalue of the previous point of the chain
+  double lam_prev = 0.0;  // coarse eigenvalue of the previous point of the chain (not finite: nothing to start from)
   // a fine solve; one on the coarse mesh itself that FP32 corrections could not finish (the shift meets the
   // eigenvalue by accident) runs again in FP64, its workspace in global memory
   auto fine = [&](int n, const double* a, const double* rb, double lamH, int& it, int& outer, int& flags, double& gq) {
@@ -1343,6 +1343,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
       CoarseWS& cw = cws;
       double lamH, gH = 0.0;
       int eit = 0;
+      const bool cold = kk == k0 || !isfinite(lam_prev);
       if (P.u_in) {
         const size_t Vc = gsz(nc);
         for_all(Vc, [&](size_t q) {
@@ -1383,7 +1384,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         if (!build_mg<float>(c32.mg, ac, nc, red, bc, c32.wxl, c32.wyl)) flags |= kFlagBadCoef;
         if (rxn)
           reaction_weights<float, double>(nc, bc, bc + (size_t)nc * nc, c32.rx, c32.ry, c32.rd, c32.rxl, c32.ryl, c32.rdl);
-        if (kk == k0) {
+        if (cold) {
           const float inc = 1.0f / (float)nc;
           for_interior(nc, [&](int p, int i, int j) {
             c32.xh[p] = sinpif(i * inc) * sinpif(j * inc);
@@ -1391,7 +1392,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
           });
         }
         __syncthreads();
-        eit = lobpcg32(c32, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh32, kk == k0 ? 20.0 : lam_prev, lamH, gH);
+        eit = lobpcg32(c32, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh32, cold ? 20.0 : lam_prev, lamH, gH);
         lam_prev = lamH;
         if (eit < 0) flags |= kFlagEigNoConv;
         if (P.u_out) {
@@ -1423,7 +1424,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         if (!build_mg<float>(cw.mg, ac, nc, red, bc)) flags |= kFlagBadCoef;
         weights_from_cells<double, double>(nc, ac, ac + (size_t)nc * nc, cw.wx, cw.wy);
         if (rxn) reaction_weights<double, double>(nc, bc, bc + (size_t)nc * nc, cw.rx, cw.ry, cw.rd);
-        if (kk == k0) {
+        if (cold) {
           const float inc = 1.0f / (float)nc;
           for_interior(nc, [&](int p, int i, int j) { cw.x[p] = (double)(sinpif(i * inc) * sinpif(j * inc)); });
         } else {
@@ -1431,6 +1432,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         }
         __syncthreads();
         eit = lobpcg(cw, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh, lamH, gH);
+        lam_prev = lamH;
         if (eit < 0) flags |= kFlagEigNoConv;
         for_interior(nc, [&](int p, int, int) { cw.uprev[p] = cw.x[p]; });
         if (P.u_out) {
