@@ -287,18 +287,44 @@ __device__ __forceinline__ double react_cells(const double* __restrict__ b, int 
 }
 
 // ---------------------------------------------------------------------------------------------
+// Scale.  FP32 and double-floats hold exponents down to 2^-126 only, and the solvers sum squares: residuals
+// of a sample with coefficients around 2^-60 have squares below that range, its solutions squares above
+// 2^127.  So what is computed in them is the problem times a power of two 2^-k, exactly: K' = 2^-k K,
+// sigma' = 2^-k sigma, x' = 2^k x with the same right-hand side, lambda = 2^k lambda'.  k comes from
+// the largest coefficient (eigensolves) or from the shift (fine solves: the smallest eigenvalue is
+// about 2 pi^2 times the coefficient).  It is a multiple of 32, which leaves ordinary coefficients as they are.
+
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }  // |k| <= 1022
+// k from the upper word of a shift (0 for zero, subnormal and non-finite values)
+__device__ __forceinline__ int scale_exponent(int hi) {
+  const int e = (hi >> 20) & 0x7ff;
+  return e == 0 || e == 0x7ff ? 0 : min(max((e - 1027 + 16) & ~31, -608), 608);  // 2 pi^2 is about 2^4
+}
+__device__ __forceinline__ int scale_of_shift(double sigma) { return scale_exponent(__double2hiint(sigma)); }
+// k from the upper words of the largest a and b (b adds itself to about 2 pi^2 a)
+__device__ __forceinline__ int scale_of_cells(int amax, int bmax) { return scale_exponent(max(amax + (4 << 20), bmax)); }
+
+// ---------------------------------------------------------------------------------------------
 // operator setup.  FP32 arrays are formed on the FP32 units, from FP64 coefficients by double-floats (an
-// FP64 addition or conversion takes sixteen clocks of an SM); FP64 arrays in FP64.
+// FP64 addition or conversion takes sixteen clocks of an SM); FP64 arrays in FP64.  k: FP64
+// coefficients enter times 2^-k.
 template <typename T, typename S>
 struct CellSum {  // (a + b) / 2 and sums of coefficients in T
-  static __device__ __forceinline__ T half(S a, S b) { return T(0.5) * (T(a) + T(b)); }
-  static __device__ __forceinline__ T val(S a) { return T(a); }
+  static __device__ __forceinline__ T half(S a, S b, int) { return T(0.5) * (T(a) + T(b)); }
+  static __device__ __forceinline__ T val(S a, int) { return T(a); }
+};
+template <>
+struct CellSum<double, double> {
+  static __device__ __forceinline__ double half(double a, double b, int k) { return pow2(-1 - k) * (a + b); }
+  static __device__ __forceinline__ double val(double a, int k) { return pow2(-k) * a; }
 };
 template <>
 struct CellSum<float, double> {
-  static __device__ __forceinline__ float half(double a, double b) { return 0.5f * df_add(df_split(a), df_split(b)).h; }
-  static __device__ __forceinline__ float val(double a) {
-    const df d = df_split(a);
+  static __device__ __forceinline__ float half(double a, double b, int k) {
+    return 0.5f * df_add(df_split(a, k), df_split(b, k)).h;
+  }
+  static __device__ __forceinline__ float val(double a, int k) {
+    const df d = df_split(a, k);
     return d.h + d.l;
   }
 };
@@ -307,11 +333,46 @@ __device__ __forceinline__ int cell_invalid(double v, bool zero_ok) {
   const long long b = __double_as_longlong(v);
   return !((zero_ok ? b >= 0 : b > 0) && b <= 0x7ff0000000000000LL);
 }
-__device__ __forceinline__ int cell_invalid(float v, bool zero_ok) { return !(zero_ok ? v >= 0.0f : v > 0.0f); }
+
+// What a block sees in a sample's coefficients: whether every a is positive (Assumption A1) and every b nonnegative, and
+// the upper words of the largest valid ones (0 without b; positive doubles order as their bit patterns, so
+// this runs on the integer units).  look() is one thread's share, finish() the block's barrier and result: between
+// them the operator is built, so that its loads do not wait for the check.
+struct CellCheck {
+  int bad = 0, amax = 0, bmax = 0;
+  __device__ __forceinline__ void look(int n, const double* __restrict__ a, const double* __restrict__ rb) {
+    auto one = [&](double v, bool zero_ok, int& m) {
+      const int no = cell_invalid(v, zero_ok);
+      bad |= no;
+      m = max(m, no ? 0 : __double2hiint(v));
+    };
+    for_all((size_t)2 * n * n, [&](size_t q) { one(a[q], false, amax); });
+    if (rb) for_all((size_t)2 * n * n, [&](size_t q) { one(rb[q], true, bmax); });
+  }
+  // red as in block_sum; the caller's next use of it lies behind another barrier
+  __device__ __forceinline__ bool finish(double* red) {
+    int* part = reinterpret_cast<int*>(red);
+    amax = __reduce_max_sync(0xffffffffu, amax);
+    bmax = __reduce_max_sync(0xffffffffu, bmax);
+    if ((threadIdx.x & 31) == 0) {
+      part[threadIdx.x >> 5] = amax;
+      part[kRedWarps + (threadIdx.x >> 5)] = bmax;
+    }
+    const bool ok = __syncthreads_or(bad) == 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      amax = max(amax, part[w]);
+      bmax = max(bmax, part[kRedWarps + w]);
+    }
+    return ok;
+  }
+};
+// an upper bound of such a largest coefficient
+__device__ __forceinline__ double cell_bound(int hi) { return (1.0 + 0x1p-19) * __hiloint2double(hi, 0); }
 
 // (lx, ly: NULL, or the low parts of the weights -- FP32 weights of FP64 coefficients as double-floats)
 template <typename T, typename S>
-__device__ void weights_from_cells(int n, const S* low, const S* up, T* wx, T* wy, T* lx = nullptr, T* ly = nullptr) {
+__device__ void weights_from_cells(int n, const S* low, const S* up, T* wx, T* wy, T* lx = nullptr, T* ly = nullptr,
+                                   int k = 0) {
   const int ld = n + 1;
   for_all(gsz(n), [&](size_t q) {
     const int i = (int)(q % ld), j = (int)(q / ld);
@@ -319,15 +380,15 @@ __device__ void weights_from_cells(int n, const S* low, const S* up, T* wx, T* w
     if constexpr (sizeof(T) == sizeof(float) && sizeof(S) == sizeof(double)) {
       if (lx) {
         df a = {0.0f, 0.0f}, b = {0.0f, 0.0f};
-        if (e) a = df_add(df_split(low[j * n + i]), df_split(up[(j - 1) * n + i]));
-        if (v) b = df_add(df_split(up[j * n + i]), df_split(low[j * n + i - 1]));
+        if (e) a = df_add(df_split(low[j * n + i], k), df_split(up[(j - 1) * n + i], k));
+        if (v) b = df_add(df_split(up[j * n + i], k), df_split(low[j * n + i - 1], k));
         wx[q] = 0.5f * a.h, lx[q] = 0.5f * a.l;
         wy[q] = 0.5f * b.h, ly[q] = 0.5f * b.l;
         return;
       }
     }
-    wx[q] = e ? CellSum<T, S>::half(low[j * n + i], up[(j - 1) * n + i]) : T(0);
-    wy[q] = v ? CellSum<T, S>::half(up[j * n + i], low[j * n + i - 1]) : T(0);
+    wx[q] = e ? CellSum<T, S>::half(low[j * n + i], up[(j - 1) * n + i], k) : T(0);
+    wy[q] = v ? CellSum<T, S>::half(up[j * n + i], low[j * n + i - 1], k) : T(0);
   });
 }
 
@@ -335,26 +396,26 @@ __device__ void weights_from_cells(int n, const S* low, const S* up, T* wx, T* w
 // rd of the hypotenuse (i,j)-(i+1,j+1) = (b_low(i,j) + b_up(i,j)) / 2
 template <typename T, typename S>
 __device__ void reaction_weights(int n, const S* low, const S* up, T* rx, T* ry, T* rd, T* lx = nullptr,
-                                 T* ly = nullptr, T* ld_ = nullptr) {
-  weights_from_cells<T, S>(n, low, up, rx, ry, lx, ly);
+                                 T* ly = nullptr, T* ld_ = nullptr, int k = 0) {
+  weights_from_cells<T, S>(n, low, up, rx, ry, lx, ly, k);
   const int ld = n + 1;
   for_all(gsz(n), [&](size_t q) {
     const int i = (int)(q % ld), j = (int)(q / ld);
     const bool in = i <= n - 1 && j <= n - 1;
     if constexpr (sizeof(T) == sizeof(float) && sizeof(S) == sizeof(double)) {
       if (ld_) {
-        const df d = in ? df_add(df_split(low[j * n + i]), df_split(up[j * n + i])) : df{0.0f, 0.0f};
+        const df d = in ? df_add(df_split(low[j * n + i], k), df_split(up[j * n + i], k)) : df{0.0f, 0.0f};
         rd[q] = 0.5f * d.h, ld_[q] = 0.5f * d.l;
         return;
       }
     }
-    rd[q] = in ? CellSum<T, S>::half(low[j * n + i], up[j * n + i]) : T(0);
+    rd[q] = in ? CellSum<T, S>::half(low[j * n + i], up[j * n + i], k) : T(0);
   });
 }
 
 // lumped reaction diagonal h^2/6 sum_{T at p} b_T at the interior nodes, 0 on the ring
 template <typename T, typename S>
-__device__ void lumped_reaction(int n, const S* low, const S* up, T* dr) {
+__device__ void lumped_reaction(int n, const S* low, const S* up, T* dr, int k = 0) {
   const int ld = n + 1;
   const T f = T(1) / (T(6) * T(n) * T(n));
   using C = CellSum<T, S>;
@@ -363,24 +424,24 @@ __device__ void lumped_reaction(int n, const S* low, const S* up, T* dr) {
     T v = T(0);
     if (i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1) {
       const int c = j * n + i;
-      v = f * (C::val(low[c]) + C::val(up[c]) + C::val(low[c - 1]) + C::val(up[c - n]) + C::val(low[c - n - 1]) +
-               C::val(up[c - n - 1]));
+      v = f * (C::val(low[c], k) + C::val(up[c], k) + C::val(low[c - 1], k) + C::val(up[c - n], k) +
+               C::val(low[c - n - 1], k) + C::val(up[c - n - 1], k));
     }
     dr[q] = v;
   });
 }
 
 template <typename T, typename S>
-__device__ void coarsen_cells(int n, const S* low, const S* up, T* out) {
+__device__ void coarsen_cells(int n, const S* low, const S* up, T* out, int k = 0) {
   const int m = n / 2;
   using C = CellSum<T, S>;
   for_all((size_t)m * m, [&](size_t q) {
     const int I = (int)(q % m), J = (int)(q / m);
     const int i = 2 * I, j = 2 * J;
-    const T lo = C::val(low[j * n + i]) + C::val(low[j * n + i + 1]) + C::val(low[(j + 1) * n + i + 1]) +
-                 C::val(up[j * n + i + 1]);
-    const T hi = C::val(up[j * n + i]) + C::val(up[(j + 1) * n + i + 1]) + C::val(up[(j + 1) * n + i]) +
-                 C::val(low[(j + 1) * n + i]);
+    const T lo = C::val(low[j * n + i], k) + C::val(low[j * n + i + 1], k) + C::val(low[(j + 1) * n + i + 1], k) +
+                 C::val(up[j * n + i + 1], k);
+    const T hi = C::val(up[j * n + i], k) + C::val(up[(j + 1) * n + i + 1], k) + C::val(up[(j + 1) * n + i], k) +
+                 C::val(low[(j + 1) * n + i], k);
     out[q] = T(0.25) * lo;
     out[m * m + q] = T(0.25) * hi;
   });
@@ -467,20 +528,16 @@ __device__ void coarse_inverse4(const T* wx, const T* wy, T* cinv, const T* dr =
 // Builds every level (weights, inverse diagonals) from the fine centroid coefficients a, and with
 // rb (hierarchy carved with the reaction arrays) the lumped reaction of every level from the
 // centroid values rb of the reaction coefficient (lx, ly: NULL, or the low parts of the finest weights, see
-// weights_from_cells).  Returns true when every a is positive
-// (Assumption A1) and every b nonnegative.
+// weights_from_cells; k: the coefficients enter times 2^-k).  The caller's next barrier closes it.
 template <typename T, typename S = double>
-__device__ bool build_mg(MGDesc<T>& d, const S* __restrict__ a, int n, double* red, const S* __restrict__ rb = nullptr,
-                         T* lx = nullptr, T* ly = nullptr) {
-  int bad = 0;
+__device__ void build_mg(MGDesc<T>& d, const S* __restrict__ a, int n, const S* __restrict__ rb = nullptr,
+                         T* lx = nullptr, T* ly = nullptr, int k = 0) {
   const bool rx = rb != nullptr && d.dr[0] != nullptr;
-  for_all((size_t)2 * n * n, [&](size_t q) { bad |= cell_invalid(a[q], false); });
-  if (rx) for_all((size_t)2 * n * n, [&](size_t q) { bad |= cell_invalid(rb[q], true); });
-  weights_from_cells<T, S>(n, a, a + (size_t)n * n, d.wx[0], d.wy[0], lx, ly);
-  if (d.L > 1) coarsen_cells<T, S>(n, a, a + (size_t)n * n, d.cell[0]);
+  weights_from_cells<T, S>(n, a, a + (size_t)n * n, d.wx[0], d.wy[0], lx, ly, k);
+  if (d.L > 1) coarsen_cells<T, S>(n, a, a + (size_t)n * n, d.cell[0], k);
   if (rx) {
-    lumped_reaction<T, S>(n, rb, rb + (size_t)n * n, d.dr[0]);
-    if (d.L > 1) coarsen_cells<T, S>(n, rb, rb + (size_t)n * n, d.rcell[0]);
+    lumped_reaction<T, S>(n, rb, rb + (size_t)n * n, d.dr[0], k);
+    if (d.L > 1) coarsen_cells<T, S>(n, rb, rb + (size_t)n * n, d.rcell[0], k);
   }
   __syncthreads();
   for (int l = 1; l < d.L; ++l) {
@@ -499,8 +556,6 @@ __device__ bool build_mg(MGDesc<T>& d, const S* __restrict__ a, int n, double* r
   inverse_diagonal<T>(d.n[d.L - 1], d.wx[d.L - 1], d.wy[d.L - 1], d.dinv[d.L - 1], rx ? d.dr[d.L - 1] : nullptr);
   if (d.L >= 2 && threadIdx.x == 0)
     coarse_inverse4<T>(d.wx[d.L - 2], d.wy[d.L - 2], d.cinv, rx ? d.dr[d.L - 2] : nullptr);
-  (void)red;
-  return __syncthreads_or(bad) == 0;
 }
 
 // Symmetric V-cycle for A (A + D_B when the hierarchy holds a lumped reaction, which build_mg must

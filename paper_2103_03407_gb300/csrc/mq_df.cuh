@@ -65,16 +65,16 @@ __device__ __forceinline__ double df_double(df x) { return (double)x.h + (double
 // The leading 48 bits of a double as a double-float, on the integer units (an FP64 conversion costs
 // as much as an FP64 operation): the upper 24 bits of the significand are the high part (truncated),
 // the other 29, rounded to 24, the low part.  Exact exponents for 2^-73 <= |v| < 2^128; smaller
-// values lose the low part, infinities and NaN stay what they are.
-__device__ __forceinline__ df df_split(double v) {
+// values lose the low part, infinities and NaN stay what they are.  k: the pair of 2^-k v (|k| <= 608).
+__device__ __forceinline__ df df_split(double v, int k = 0) {
   const long long u = __double_as_longlong(v);
   const unsigned hi = (unsigned)((unsigned long long)u >> 32), lo = (unsigned)u;
   const int e = (int)((hi >> 20) & 0x7ffu);
   const unsigned sign = hi & 0x80000000u;
-  const int eh = min(max(e - 896, 0), 255);
+  const int eh = min(max(e - 896 - k, 0), 255);
   const unsigned m = (hi << 3 & 0x7fffffu) | (lo >> 29);
   const float h = __uint_as_float(sign | ((unsigned)eh << 23) | m);
-  const int el = eh == 255 ? 0 : max(e - 948, 0);
+  const int el = eh == 255 ? 0 : max(e - 948 - k, 0);
   const float l = __fmul_rn((float)(lo & 0x1fffffffu), __uint_as_float(sign | ((unsigned)el << 23)));
   return {h, l};
 }

@@ -789,6 +789,20 @@ struct CoarseVec {
   __device__ df pair(int q) const { return d ? df_split(d[q]) : df{h[q], l[q]}; }
 };
 
+// The operator of a sample in FP32 with the low parts of its finest weights, coefficients times 2^-k: hierarchy and
+// reaction weights of a coarse (CoarseWS32) or fine (FineWS<float>) workspace
+template <typename WS>
+__device__ __forceinline__ void operator32(WS& ws, int n, const double* a, const double* rb, int k) {
+  build_mg<float>(ws.mg, a, n, rb, ws.wxl, ws.wyl, k);
+  if (rb) reaction_weights<float, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd, ws.rxl, ws.ryl, ws.rdl, k);
+}
+// the same out of line: inlined into twogrid_fine it costs registers that the iterations then spill (first test
+// problem's level 1, 8,192 samples: 7.96 ms inline, 7.84 out of line)
+template <typename WS>
+__device__ __noinline__ void operator32_scaled(WS& ws, int n, const double* a, const double* rb, int k) {
+  operator32(ws, n, a, rb, k);
+}
+
 // MINRES scalars, owned by thread 0 and read by all threads after each reduction.  The
 // recurrences run in the inner precision T (FP32 on the mixed path), the refinement norms in FP64.
 template <typename T>
@@ -803,6 +817,7 @@ struct MinresShared {
   double knorm, xnorm;  // ||A - sigma M|| bound and ||x|| for the FP64 residual floor
   double xax, xmx;      // x.Ax and x.Mx of the last FP64 residual pass (the Rayleigh quotient)
   double xsum;          // sum of the nodal values of x in that pass (h^2 xsum = integral of x)
+  double scale;         // 2^ks: the solve is the problem times 2^-ks
   double tau;           // factor of the right-hand side (1 except in a solve on the coarse mesh itself)
   int done, breakdown;
 };
@@ -854,45 +869,29 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
     zero_vec(ws.rd, n);
   }
   zero_mg(ws.mg);
+  // FP32 kernel: everything below is the problem times 2^-ks (see mq_device.cuh)
+  const int ks = kF32 ? scale_of_shift(sigma) : 0;
+  sigma *= pow2(-ks);
   __syncthreads();
+  CellCheck cells;
+  cells.look(n, a, rb);
   if constexpr (kF32) {
-    if (!build_mg<T>(ws.mg, a, n, red, rb, ws.wxl, ws.wyl)) flags |= kFlagBadCoef;
-    if (rb)
-      reaction_weights<T, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd, ws.rxl, ws.ryl, ws.rdl);
+    operator32_scaled(ws, n, a, rb, ks);
   } else {
-    if (!build_mg<T>(ws.mg, a, n, red, rb)) flags |= kFlagBadCoef;
+    build_mg<T>(ws.mg, a, n, rb);
     if (rb) reaction_weights<T, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd);
   }
-  {
+  if (!cells.finish(red)) flags |= kFlagBadCoef;
+  if (threadIdx.x == 0) {
     // ||A + B - sigma M||_inf <= 8 max a + (max b + sigma) h^2 (row sums of the edge form, of the
-    // reaction and of the mass); positive doubles order as their bit patterns (integer units)
-    long long amax = 0, bmax = 0;
-    for_all((size_t)2 * n * n, [&](size_t q) {
-      amax = max(amax, __double_as_longlong(a[q]));
-      if (rb) bmax = max(bmax, __double_as_longlong(rb[q]));
-    });
-    for (int off = 16; off > 0; off >>= 1) {
-      amax = max(amax, (long long)__shfl_xor_sync(0xffffffffu, amax, off));
-      bmax = max(bmax, (long long)__shfl_xor_sync(0xffffffffu, bmax, off));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      red[threadIdx.x >> 5] = __longlong_as_double(amax);
-      red[32 + (threadIdx.x >> 5)] = __longlong_as_double(bmax);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double m = 0.0, mb = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        m = fmax(m, red[w]);
-        mb = fmax(mb, red[32 + w]);
-      }
-      ms->knorm = 8.0 * m + (mb + sigma) / ((double)n * n);
-      ms->xnorm = 0.0;
-      ms->xax = ms->xmx = 0.0;
-      ms->tau = 1.0;
-    }
-    __syncthreads();
+    // reaction and of the mass)
+    ms->knorm = 8.0 * (pow2(-ks) * cell_bound(cells.amax)) + (pow2(-ks) * cell_bound(cells.bmax) + sigma) / ((double)n * n);
+    ms->scale = pow2(ks);
+    ms->xnorm = 0.0;
+    ms->xax = ms->xmx = 0.0;
+    ms->tau = 1.0;
   }
+  __syncthreads();
   // FP64 kernel: the operator of the residual from the FP64 weights of level 0
   const double* wx64 = (const double*)ws.mg.wx[0];
   const double* wy64 = (const double*)ws.mg.wy[0];
@@ -1258,7 +1257,7 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
     flags |= kFlagLinNoConv;
   // Rayleigh quotient and functional in FP64, from the residual pass over the final iterate
   gq = fabs(ms->xsum) / ((double)n * n * sqrt(ms->xmx));
-  return ms->xax / ms->xmx;
+  return ms->scale * (ms->xax / ms->xmx);
 }
 
 // MAXT: threads per block at most.  Up to 256 threads the FP32 kernel is compiled for three blocks of 256 per SM (80
@@ -1381,9 +1380,12 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         __syncthreads();
         const double* ac = P.a_c + b * ncT;
         const double* bc = rxn ? P.b_c + b * ncT : nullptr;
-        if (!build_mg<float>(c32.mg, ac, nc, red, bc, c32.wxl, c32.wyl)) flags |= kFlagBadCoef;
-        if (rxn)
-          reaction_weights<float, double>(nc, bc, bc + (size_t)nc * nc, c32.rx, c32.ry, c32.rd, c32.rxl, c32.ryl, c32.rdl);
+        CellCheck cells;
+        cells.look(nc, ac, bc);
+        operator32(c32, nc, ac, bc, 0);
+        if (!cells.finish(red)) flags |= kFlagBadCoef;
+        const int ks = scale_of_cells(cells.amax, cells.bmax);
+        if (ks != 0) operator32_scaled(c32, nc, ac, bc, ks);  // (coefficients beyond 2^-16 .. 2^15)
         if (cold) {
           const float inc = 1.0f / (float)nc;
           for_interior(nc, [&](int p, int i, int j) {
@@ -1392,8 +1394,9 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
           });
         }
         __syncthreads();
-        eit = lobpcg32(c32, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh32, cold ? 20.0 : lam_prev, lamH, gH);
-        lam_prev = lamH;
+        eit = lobpcg32(c32, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh32, cold ? 20.0 : pow2(-ks) * lam_prev, lamH,
+                       gH);
+        lam_prev = lamH *= pow2(ks);
         if (eit < 0) flags |= kFlagEigNoConv;
         if (P.u_out) {
           for_interior(nc, [&](int p, int i, int j) {
@@ -1421,9 +1424,14 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         __syncthreads();
         const double* ac = P.a_c + b * ncT;
         const double* bc = rxn ? P.b_c + b * ncT : nullptr;
-        if (!build_mg<float>(cw.mg, ac, nc, red, bc)) flags |= kFlagBadCoef;
-        weights_from_cells<double, double>(nc, ac, ac + (size_t)nc * nc, cw.wx, cw.wy);
-        if (rxn) reaction_weights<double, double>(nc, bc, bc + (size_t)nc * nc, cw.rx, cw.ry, cw.rd);
+        CellCheck cells;
+        cells.look(nc, ac, bc);
+        if (!cells.finish(red)) flags |= kFlagBadCoef;
+        const int ks = scale_of_cells(cells.amax, cells.bmax);  // (its V-cycles and Gram matrices are FP32)
+        build_mg<float>(cw.mg, ac, nc, bc, nullptr, nullptr, ks);
+        weights_from_cells<double, double>(nc, ac, ac + (size_t)nc * nc, cw.wx, cw.wy, nullptr, nullptr, ks);
+        if (rxn)
+          reaction_weights<double, double>(nc, bc, bc + (size_t)nc * nc, cw.rx, cw.ry, cw.rd, nullptr, nullptr, nullptr, ks);
         if (cold) {
           const float inc = 1.0f / (float)nc;
           for_interior(nc, [&](int p, int i, int j) { cw.x[p] = (double)(sinpif(i * inc) * sinpif(j * inc)); });
@@ -1432,7 +1440,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         }
         __syncthreads();
         eit = lobpcg(cw, nc, P.tol_eig, P.max_eig_it, P.nu, omega, red, &esh, lamH, gH);
-        lam_prev = lamH;
+        lam_prev = lamH *= pow2(ks);
         if (eit < 0) flags |= kFlagEigNoConv;
         for_interior(nc, [&](int p, int, int) { cw.uprev[p] = cw.x[p]; });
         if (P.u_out) {

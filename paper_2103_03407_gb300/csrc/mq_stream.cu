@@ -104,14 +104,16 @@ struct SS {  // per-sample solver scalars
   T gam, gam_old, eta, eta0, c, c_old, s, s_old, ig, c1, c2, cx, ia1, a2, a3, delta, rs;
   T tol;          // reduction of the inner solve under way
   T igp;          // 1 / gamma of the previous step: the pending update normalises z_j on the fly
-  T sigm;         // lambda_H h^2 / 12: the mass factor of the shifted operator
+  T sigm;         // sig h^2 / 12: the mass factor of the shifted operator
+  double sig;     // lambda_H, on the FP32 path times 2^-ks: that path solves the problem times 2^-ks (see mq_device.cuh)
+  int ks;
   double rnorm, bnorm, lam_h;
   double xnorm;   // ||x64||
   double xax, xmx;  // x.Ax and x.Mx of the last FP64 residual pass (the Rayleigh quotient)
   double xsum;      // sum of the nodal values of x64 in that pass (h^2 xsum = integral of x)
   float amax;     // largest centroid coefficient (for the bound ||A - sigma M|| <= 8 amax + sigma h^2)
   float bmax;     // largest reaction coefficient (the bound gains bmax h^2)
-  df cs, c12;     // lambda_H h^2 / 12 and lambda_H h^2 as double-floats (FP32 path: the residual's mass factors)
+  df cs, c12;     // sig h^2 / 12 and sig h^2 as double-floats (FP32 path: the residual's mass factors)
   int act_outer;  // refinement still running
   int act;        // inner MINRES running
   int pend;       // a w/x update is pending
@@ -210,9 +212,11 @@ __global__ void k_weights(int n, int B, const S* __restrict__ cells, size_t cstr
   }
 }
 
-// per-triangle coefficients of mesh n/2 as means of the four fine triangles each contains
+// per-triangle coefficients of mesh n/2 as means of the four fine triangles each contains (sigma: the shifts that
+// give the scale where FP64 coefficients enter FP32, else NULL)
 template <typename S, typename T>
-__global__ void k_coarsen(int n, int B, const S* __restrict__ in, size_t istride, T* __restrict__ out) {
+__global__ void k_coarsen(int n, int B, const S* __restrict__ in, size_t istride, T* __restrict__ out,
+                          const double* sigma, int sig_stride) {
   const int m = n / 2;
   const size_t mm = (size_t)m * m;
   const int nt = (int)((mm + kTile - 1) / kTile);
@@ -223,9 +227,10 @@ __global__ void k_coarsen(int n, int B, const S* __restrict__ in, size_t istride
   T* o = out + (size_t)b * 2 * mm;
   // the FP32 path rounds the four values first (the coarse operators only precondition; FP64
   // additions and conversions bound this kernel otherwise)
-  auto val = [](S v) {
+  const int ks = sigma ? scale_of_shift(sigma[(size_t)b * sig_stride]) : 0;
+  auto val = [ks](S v) {
     if constexpr (sizeof(S) == sizeof(double) && sizeof(T) == sizeof(float)) {
-      const df d = df_split(v);
+      const df d = df_split(v, ks);
       return d.h + d.l;
     } else {
       return T(v);
@@ -243,10 +248,13 @@ __global__ void k_coarsen(int n, int B, const S* __restrict__ in, size_t istride
   }
 }
 
+// B arrays of per_sample coefficients (sigma as in k_coarsen)
 template <typename S, typename T>
-__global__ void k_convert(size_t count, const S* __restrict__ in, T* __restrict__ out) {
+__global__ void k_convert(int B, size_t per_sample, const S* __restrict__ in, T* __restrict__ out, const double* sigma,
+                          int sig_stride) {
+  const size_t count = B * per_sample;
   for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < count; q += (size_t)gridDim.x * blockDim.x)
-    out[q] = T(in[q]);
+    out[q] = T(sigma ? pow2(-scale_of_shift(sigma[q / per_sample * sig_stride])) * in[q] : in[q]);
 }
 
 // k 2^-l as a double (0 <= k < 2^l, l <= 30), assembled from its bits on the integer units (the
@@ -335,10 +343,13 @@ __global__ void k_sc_start(int B, int n, const double* sigma, int sig_stride, in
   warp_sum_slots<1>(part, b, nch, t);
   if ((threadIdx.x & 31) != 0) return;
   const double s = t[0];
-  ss[b].sigm = T(sigma[(size_t)b * sig_stride] / (12.0 * n * n));
   SS<T>& S = ss[b];
-  S.cs = df_split(sigma[(size_t)b * sig_stride] / (12.0 * n * n));
-  S.c12 = df_split(sigma[(size_t)b * sig_stride] / ((double)n * n));
+  const double sg = sigma[(size_t)b * sig_stride];
+  S.ks = sizeof(T) == sizeof(float) ? scale_of_shift(sg) : 0;
+  S.sig = pow2(-S.ks) * sg;
+  S.sigm = T(S.sig / (12.0 * n * n));
+  S.cs = df_split(S.sig / (12.0 * n * n));
+  S.c12 = df_split(S.sig / ((double)n * n));
   S.bnorm = S.rnorm = sqrt(s);
   S.rs = T(1.0 / S.rnorm);
   S.act_outer = S.rnorm > 0.0;
@@ -377,8 +388,8 @@ __host__ __device__ inline double residual_target(double tol, double bnorm, doub
 }
 
 template <typename T>
-__device__ inline double knorm_of(const SS<T>& S, int n, double sigma) {
-  return 8.0 * (double)S.amax + ((double)S.bmax + sigma) / ((double)n * n);
+__device__ inline double knorm_of(const SS<T>& S, int n) {
+  return 8.0 * (double)S.amax + ((double)S.bmax + S.sig) / ((double)n * n);
 }
 
 // Reduction asked of an FP32 inner solve, chosen so that no iteration is spent below what the solve can
@@ -399,12 +410,11 @@ __device__ inline double inner_reduction(int n, int outer, double rnorm, double 
 // start of a refinement step: samples above the residual target run an inner solve (target: tol
 // relative to ||b||, but not below a small multiple of the FP64 floor eps (||K|| ||x|| + ||b||))
 template <typename T>
-__global__ void k_sc_outer_begin(int B, int n, const double* sigma, int sig_stride, double tol_lin, double tol_inner,
-                                 SS<T>* ss, int* act, int* count) {
+__global__ void k_sc_outer_begin(int B, int n, double tol_lin, double tol_inner, SS<T>* ss, int* act, int* count) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   SS<T>& S = ss[b];
-  const double kn = knorm_of(S, n, sigma[(size_t)b * sig_stride]);
+  const double kn = knorm_of(S, n);
   const double target = residual_target(tol_lin, S.bnorm, kn, S.xnorm, 16.0);
   const int a = S.act_outer && (S.rnorm > target);
   S.tol = T(tol_inner > 0.0 ? tol_inner : S.strict ? 1e-5 : inner_reduction(n, S.outer, S.rnorm, S.bnorm, target));
@@ -722,7 +732,6 @@ __global__ void __launch_bounds__(kThreads) k_sub_build(int ns, int B, const T* 
                                                         char* __restrict__ subw, size_t wbytes,
                                                         const T* __restrict__ rcells) {
   extern __shared__ __align__(16) char sm[];
-  __shared__ double red[kRedSlots];
   __shared__ MGDesc<T> mg;
   const int b = blockIdx.x;
   if (b >= B) return;
@@ -733,7 +742,7 @@ __global__ void __launch_bounds__(kThreads) k_sub_build(int ns, int B, const T* 
   carve_mg_split<T>(w, v, ns, d, rcells != nullptr);
   if (threadIdx.x == 0) mg = d;
   __syncthreads();
-  build_mg<T, T>(mg, cells + (size_t)b * 2 * ns * ns, ns, red, rcells ? rcells + (size_t)b * 2 * ns * ns : nullptr);
+  build_mg<T, T>(mg, cells + (size_t)b * 2 * ns * ns, ns, rcells ? rcells + (size_t)b * 2 * ns * ns : nullptr);
 }
 
 // meshes 1/ns .. 1/2 of one sample inside one CTA: x = B^{-1} b (operator arrays read from the
@@ -1023,8 +1032,8 @@ __host__ __device__ inline int tiles_setup(int n) {
   return (int)(((long)(n + 1) * (n / kVec + 1) + kThreads - 1) / kThreads);
 }
 
-__device__ __forceinline__ df cell_value(double v) { return df_split(v); }
-__device__ __forceinline__ df cell_value(float v) { return {v, 0.0f}; }
+__device__ __forceinline__ df cell_value(double v, int ks) { return df_split(v, ks); }
+__device__ __forceinline__ df cell_value(float v, int) { return {v, 0.0f}; }
 
 // four coefficients of a cell row at columns c0 .. c0+3 into v[1..4], the one at c0 - 1 into v[0]
 // (zeros when the row or the column is outside); returns nothing beyond the values
@@ -1077,7 +1086,7 @@ __device__ __forceinline__ int cell_bad(float, unsigned long long&) {
 // Edge weights and damped inverse diagonal of mesh n from per-triangle coefficients (lower plane,
 // upper plane), as k_weights<float>: four nodes of one row per thread.  S = double: the finest mesh,
 // with the low parts of the weights in wxl, wyl (and, with the reaction, rxl, ryl, rdl), the
-// coefficient checks and the largest coefficient into ss.  S = float: a coarsened mesh.  wx, wy or
+// coefficient checks, the scale of the shift sigma and the largest coefficient into ss.  S = float: a coarsened mesh.  wx, wy or
 // dinv may be NULL when nothing reads them (the V(1,1) sweeps read the BF16 copies hx, hy, hd).
 // Bound by memory: 16 B in and 30 B out per node of the finest mesh; the FP64 form executed about 14
 // FP64 instructions per node.
@@ -1089,7 +1098,7 @@ struct WeightOut {
 template <typename S, bool RX>
 __global__ void __launch_bounds__(kThreads) k_weights4(int n, int B, const S* __restrict__ cells, size_t cstride,
                                                        const S* __restrict__ rcells, float om, WeightOut W,
-                                                       SS<float>* ss) {
+                                                       SS<float>* ss, const double* sigma, int sig_stride) {
   constexpr bool FINE = sizeof(S) == sizeof(double);
   const int nt = tiles_setup(n);
   const int b = blockIdx.x / nt, ch = blockIdx.x % nt;
@@ -1099,6 +1108,7 @@ __global__ void __launch_bounds__(kThreads) k_weights4(int n, int B, const S* __
   const int j = g / groups, c0 = (g % groups) * kVec;
   unsigned long long top = 0, rtop = 0;
   int bad = 0;
+  const int ks = FINE ? scale_of_shift(sigma[(size_t)b * sig_stride]) : 0;
   if (j <= n) {
     const size_t nn = (size_t)n * n;
     const bool in = c0 < n, up_row = in && j < n, dn_row = in && j >= 1;
@@ -1121,10 +1131,10 @@ __global__ void __launch_bounds__(kThreads) k_weights4(int n, int B, const S* __
       df L0[5], U0[5], L1[5], U1[5];
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
-        L0[k] = cell_value(l0[k]);
-        U0[k] = cell_value(u0[k]);
-        L1[k] = cell_value(l1[k]);
-        U1[k] = cell_value(u1[k]);
+        L0[k] = cell_value(l0[k], ks);
+        U0[k] = cell_value(u0[k], ks);
+        L1[k] = cell_value(l1[k], ks);
+        U1[k] = cell_value(u1[k], ks);
       }
       const bool mid = j >= 1 && j < n;
 #pragma unroll
@@ -1190,7 +1200,7 @@ __global__ void __launch_bounds__(kThreads) k_weights4(int n, int B, const S* __
   if (FINE) {
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&ss[b].flags, kFlagBadCoef);
     auto largest = [&](unsigned long long bits, float* to) {
-      float v = df_split(__longlong_as_double((long long)bits)).h * 1.0001f;
+      float v = df_split(__longlong_as_double((long long)bits), ks).h * 1.0001f;
       if (!(v < INFINITY)) v = 0.0f;
       for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
       if ((threadIdx.x & 31) == 0 && v > 0.0f) atomicMax((int*)to, __float_as_int(v));  // positive floats order as ints
@@ -1491,8 +1501,7 @@ __global__ void __launch_bounds__(kThreads) k_residual4(int n, int B, const int*
 }
 
 // the scalars of a refinement step from the partial sums of k_residual4
-__global__ void k_sc_outer_end4(int B, int n, int nch, const double* part, const double* sigma, int sig_stride,
-                                const int* ran, SS<float>* ss) {
+__global__ void k_sc_outer_end4(int B, int n, int nch, const double* part, const int* ran, SS<float>* ss) {
   const int b = warp_sample();
   if (b >= B || !ran[b]) return;
   double t[5];
@@ -1500,7 +1509,7 @@ __global__ void k_sc_outer_end4(int B, int n, int nch, const double* part, const
   if ((threadIdx.x & 31) != 0) return;
   SS<float>& S = ss[b];
   S.xmx = (t[1] - t[3] / 12.0) / ((double)n * n);
-  S.xax = t[2] + sigma[(size_t)b * sig_stride] * S.xmx;
+  S.xax = t[2] + S.sig * S.xmx;
   S.xsum = t[4];
   outer_step_done(S, sqrt(t[0]), sqrt(t[1]));
 }
@@ -2119,18 +2128,16 @@ __global__ void k_sc_outer_end(int B, int nch, const double* part, const int* ra
 
 // the Rayleigh quotient x.Ax / x.Mx, or with qoi the functional G(x) = h^2 |sum x| / sqrt(x.Mx)
 template <typename T>
-__global__ void k_sc_rq(int B, int n, const double* sigma, int sig_stride, const SS<T>* ss, double tol_lin,
-                        double* lam_out,
-                        int lam_stride, int* it_out, int it_stride, int* outer_out, int outer_stride, int* flags,
+__global__ void k_sc_rq(int B, int n, const SS<T>* ss, double tol_lin, double* lam_out, int lam_stride, int* it_out, int it_stride, int* outer_out, int outer_stride, int* flags,
                         int flag_stride, int qoi) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const SS<T>& S = ss[b];
-  lam_out[(size_t)b * lam_stride] = qoi ? fabs(S.xsum) / ((double)n * n * sqrt(S.xmx)) : S.xax / S.xmx;
+  lam_out[(size_t)b * lam_stride] = qoi ? fabs(S.xsum) / ((double)n * n * sqrt(S.xmx)) : pow2(S.ks) * (S.xax / S.xmx);
   it_out[(size_t)b * it_stride] = S.iters;
   outer_out[(size_t)b * outer_stride] = S.outer;
   int f = S.flags;
-  const double kn = knorm_of(S, n, sigma[(size_t)b * sig_stride]);
+  const double kn = knorm_of(S, n);
   if (!(S.rnorm <= residual_target(fmax(1e-5, 10.0 * tol_lin), S.bnorm, kn, S.xnorm, 256.0))) f |= kFlagLinNoConv;
   flags[(size_t)b * flag_stride] |= f;
 }
@@ -2536,7 +2543,7 @@ cudaError_t outer_pass(const StreamSolve& s, Arena<T>& A, df hm, cudaStream_t st
     else
       k_residual4<false><<<B * nt, kThreads, 0, st>>>(n, B, A.ran, W, A.ss, hm, A.xh, A.xl, A.bh, A.bl, A.v, A.part, s.qoi);
     LAUNCH_CHECK();
-    ++tl_launches, k_sc_outer_end4<<<gw, 256, 0, st>>>(B, n, nt, A.part, s.lamH, s.lam_stride, A.ran, A.ss);
+    ++tl_launches, k_sc_outer_end4<<<gw, 256, 0, st>>>(B, n, nt, A.part, A.ran, A.ss);
   } else {
     const int nt = tiles_interior(n);
     ++tl_launches, k_outer_update<T><<<B * nt, kThreads, 0, st>>>(n, B, A.ss, A.ran, A.xi, A.x64);
@@ -2619,6 +2626,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   ++tl_launches, k_zero<int><<<grid1(Bz * sizeof(SS<T>) / sizeof(int)), 256, 0, st>>>(Bz * sizeof(SS<T>) / sizeof(int), (int*)A.ss);
   LAUNCH_CHECK();
   const size_t astride = (size_t)2 * n * n;
+  const double* const scale = kF32 ? s.lamH : nullptr;
   for (int l = 0; l < (A.Ls > 1 ? A.Ls : 1); ++l) {
     const int nl = n >> l;
     if constexpr (kF32) {
@@ -2634,15 +2642,17 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
         W.wxl = A.wxl, W.wyl = A.wyl;
         W.rx = A.rx, W.ry = A.ry, W.rd = A.rd, W.rxl = A.rxl, W.ryl = A.ryl, W.rdl = A.rdl;
         if (A.rxn)
-          k_weights4<double, true><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, s.a, astride, s.b, om, W, A.ss);
+          k_weights4<double, true><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, s.a, astride, s.b, om, W, A.ss, s.lamH,
+                                                                             s.lam_stride);
         else
-          k_weights4<double, false><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, s.a, astride, nullptr, om, W, A.ss);
+          k_weights4<double, false><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, s.a, astride, nullptr, om, W, A.ss, s.lamH,
+                                                                              s.lam_stride);
       } else if (A.rxn) {
         k_weights4<float, true><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl,
-                                                                          A.rcells[l], om, W, A.ss);
+                                                                          A.rcells[l], om, W, A.ss, nullptr, 0);
       } else {
         k_weights4<float, false><<<B * tiles_setup(nl), kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl,
-                                                                           nullptr, om, W, A.ss);
+                                                                           nullptr, om, W, A.ss, nullptr, 0);
       }
     } else if (l == 0) {
       ++tl_launches, k_weights<T, double><<<B * tiles_padded(nl), kThreads, 0, st>>>(nl, B, s.a, astride, A.wx[0], A.wy[0],
@@ -2656,19 +2666,19 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     const int m = nl / 2;
     const int ntc = (int)(((size_t)m * m + kTile - 1) / kTile);
     if (l == 0) {
-      ++tl_launches, k_coarsen<double, T><<<B * ntc, kThreads, 0, st>>>(nl, B, s.a, astride, A.cells[1]);
-      if (A.rxn) ++tl_launches, k_coarsen<double, T><<<B * ntc, kThreads, 0, st>>>(nl, B, s.b, astride, A.rcells[1]);
+      ++tl_launches, k_coarsen<double, T><<<B * ntc, kThreads, 0, st>>>(nl, B, s.a, astride, A.cells[1], scale, s.lam_stride);
+      if (A.rxn) ++tl_launches, k_coarsen<double, T><<<B * ntc, kThreads, 0, st>>>(nl, B, s.b, astride, A.rcells[1], scale, s.lam_stride);
     } else {
-      ++tl_launches, k_coarsen<T, T><<<B * ntc, kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl, A.cells[l + 1]);
+      ++tl_launches, k_coarsen<T, T><<<B * ntc, kThreads, 0, st>>>(nl, B, A.cells[l], (size_t)2 * nl * nl, A.cells[l + 1], nullptr, 0);
       if (A.rxn)
         ++tl_launches, k_coarsen<T, T><<<B * ntc, kThreads, 0, st>>>(nl, B, A.rcells[l], (size_t)2 * nl * nl,
-                                                                     A.rcells[l + 1]);
+                                                                     A.rcells[l + 1], nullptr, 0);
     }
     LAUNCH_CHECK();
   }
   if (A.Ls == 0) {
-    ++tl_launches, k_convert<double, T><<<grid1(Bz * astride), 256, 0, st>>>(Bz * astride, s.a, A.cells[0]);
-    if (A.rxn) ++tl_launches, k_convert<double, T><<<grid1(Bz * astride), 256, 0, st>>>(Bz * astride, s.b, A.rcells[0]);
+    ++tl_launches, k_convert<double, T><<<grid1(Bz * astride), 256, 0, st>>>(B, astride, s.a, A.cells[0], scale, s.lam_stride);
+    if (A.rxn) ++tl_launches, k_convert<double, T><<<grid1(Bz * astride), 256, 0, st>>>(B, astride, s.b, A.rcells[0], scale, s.lam_stride);
     LAUNCH_CHECK();
   }
   ++tl_launches, k_sub_build<T><<<B, kThreads, sub_smem, st>>>(ns, B, A.cells[A.Ls], A.subw, A.subw_bytes,
@@ -2710,7 +2720,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
     LAUNCH_CHECK();
     if ((e = open_while(st, b0, ho)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(cnt_o, 0, sizeof(int), b0)) != cudaSuccess) return e;
-    ++tl_launches, k_sc_outer_begin<T><<<gs, 256, 0, b0>>>(B, n, s.lamH, s.lam_stride, s.tol_lin, s.tol_inner, A.ss, A.act, cnt_o);
+    ++tl_launches, k_sc_outer_begin<T><<<gs, 256, 0, b0>>>(B, n, s.tol_lin, s.tol_inner, A.ss, A.act, cnt_o);
     LAUNCH_CHECK();
     if ((e = cudaMemcpyAsync(A.ran, A.act, Bz * sizeof(int), cudaMemcpyDeviceToDevice, b0)) != cudaSuccess) return e;
     ++tl_launches, k_inner_init<T><<<B * nt, kThreads, 0, b0>>>(n, B, A.act, A.ss, A.v, kF32 ? nullptr : A.vo, A.w, A.wo, A.xi);
@@ -2772,7 +2782,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   // ---- refinement loop
   for (int o = 0; o < s.max_outer; ++o) {
     cudaMemsetAsync(A.count, 0, sizeof(int), st);
-    ++tl_launches, k_sc_outer_begin<T><<<gs, 256, 0, st>>>(B, n, s.lamH, s.lam_stride, s.tol_lin, s.tol_inner, A.ss, A.act, A.count);
+    ++tl_launches, k_sc_outer_begin<T><<<gs, 256, 0, st>>>(B, n, s.tol_lin, s.tol_inner, A.ss, A.act, A.count);
     LAUNCH_CHECK();
     int active = read_count(A.count, st, e);
     if (e != cudaSuccess) return e;
@@ -2835,7 +2845,7 @@ cudaError_t stream_solve_t(const StreamSolve& s, void* arena, cudaStream_t st, c
   }
   }
   // ---- Rayleigh quotient (from each sample's last residual pass)
-  ++tl_launches, k_sc_rq<T><<<gs, 256, 0, st>>>(B, n, s.lamH, s.lam_stride, A.ss, s.tol_lin, s.lam_out, s.lam_out_stride, s.iters_out,
+  ++tl_launches, k_sc_rq<T><<<gs, 256, 0, st>>>(B, n, A.ss, s.tol_lin, s.lam_out, s.lam_out_stride, s.iters_out,
                                  s.iters_stride, s.outer_out, s.outer_stride, s.flags, s.flags_stride, s.qoi);
   LAUNCH_CHECK();
   return cudaSuccess;
