@@ -603,6 +603,7 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   // The functional G(u_H) of a direct level is first order in the eigenvector error, which the
   // eigen-residual bounds only to ~tol_eig (lambda_H is second order): it takes 1e-11.
   p.tol_eig = c->opt_tol_eig > 0 ? c->opt_tol_eig : (c->qoi == MQ_QOI_FUNCTIONAL ? 1e-11 : (want_u || rxn ? 1e-8 : 1e-6));
+  p.eig32 = given ? g.nc <= mq::kEig32Max : mq::eig32_reaches(g.nc, p.tol_eig);  // (given pairs are only read)
   p.max_eig_it = c->opt_max_eig > 0 ? c->opt_max_eig : 200;
   p.tol_lin = c->tol_lin > 0 ? c->tol_lin : (mixed ? 1e-5 : 1e-6);
   if (mixed) {
@@ -636,7 +637,7 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   const int np_k = given ? 0 : g.np;  // the previous-level solve runs here only without the store
   const int in_kernel_n = std::max(p.mode_f != 2 && !g.direct_f ? g.nf : 0, p.mode_p != 2 && !g.direct_p ? np_k : 0);
   const int threads = g.threads > 0 ? g.threads : threads_for(in_kernel_n, g.nc);
-  const size_t slab = mq::sample_slab_bytes(g.nf, g.nc, np_k, mixed, g.direct_f ? 2 : p.mode_f, g.direct_p ? 2 : p.mode_p,
+  const size_t slab = mq::sample_slab_bytes(g.nf, g.nc, np_k, mixed, p.eig32, g.direct_f ? 2 : p.mode_f, g.direct_p ? 2 : p.mode_p,
                                             p.reaction);
   const int static_smem = mq::sample_static_smem(mixed);
   const size_t smem_cap = (size_t)std::max(0, c->smem_optin - static_smem - 1024);

@@ -31,6 +31,7 @@ struct SampleLaunch {
   int use_smem;
   double tol_eig;
   int max_eig_it;
+  int eig32;               // FP32 kernel: coarse eigensolves by lobpcg32 (see eig32_reaches)
   double tol_lin;          // relative FP64 residual target of the shifted solve
   double tol_inner;        // relative reduction of the preconditioned residual per inner solve
   int max_inner_it;
@@ -153,9 +154,16 @@ enum : int {
   kFlagBreakdown = 8,
 };
 
-size_t sample_slab_bytes(int nf, int nc, int np, int mixed);
 size_t sample_fallback_bytes(int n, int reaction);
-size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int mode_f, int mode_p, int reaction = 0);
+size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int eig32, int mode_f, int mode_p, int reaction = 0);
+// Whether the eigen-residual target tol is within reach of lobpcg32 on mesh 1/nc.  Rounding the iterate to 48 bits
+// alone leaves a residual relative to theta ||Mx|| that grows like n^2 max a / theta: for the sine families
+// targets of 3e-14, 1e-13, 3e-13 and 1e-12 were out of reach of every sample on meshes 1/16, 1/32, 1/64 and
+// 1/128 (1e-13, 3e-13, 1e-12 and 1e-11 were not).  2e-15 n^2 is 16 times the floor of a constant coefficient, room for
+// coefficients up to about 2 a0 with theta as low as a quarter of 2 pi^2 a0.  Other targets, and coefficients
+// that nothing bounds, take the FP64 eigensolver.
+constexpr int kEig32Max = 128;
+inline bool eig32_reaches(int nc, double tol) { return nc <= kEig32Max && tol >= 2e-15 * nc * nc; }
 cudaError_t launch_sample(const SampleLaunch& p, int mixed, int blocks, int threads, size_t smem,
                           cudaStream_t st);
 int sample_occupancy(int mixed, int threads, size_t smem);

@@ -91,14 +91,16 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   if (B == 0) return MQ_OK;
   if (!d_a_coarse || !d_out || !d_stat || !d_outer) return MQ_EINVAL;
   const int mixed = precision == MQ_PREC_MIXED;
-  // the workspace is sized for the solves performed (mode 2: none)
+  // the workspace is sized for the solves performed (mode 2: none); coarse eigensolves in FP64: nothing bounds the
+  // contrast of the caller's coefficients (see eig32_reaches)
+  const int eig32 = 0;
   const int mode_f = d_a_fine ? 0 : 2, mode_p = d_a_prev ? 0 : 2;
-  const size_t slab = mq::sample_slab_bytes(n_fine, n_coarse, n_prev, mixed, mode_f, mode_p);
+  const size_t slab = mq::sample_slab_bytes(n_fine, n_coarse, n_prev, mixed, eig32, mode_f, mode_p);
   // a solve on the coarse mesh itself may fall back to FP64 (see mq_sample.cu)
   const bool near = mixed && ((d_a_fine && n_fine == n_coarse) || (d_a_prev && n_prev == n_coarse));
   const size_t fslab = near ? mq::sample_fallback_bytes(n_coarse, 0) : 0;
   // one block's workspace, with every solve the meshes allow, has to fit in the fixed array (FP64: fine meshes up to 1/256)
-  const size_t full = mq::sample_slab_bytes(n_fine, n_coarse, n_prev, mixed, 0, 0);
+  const size_t full = mq::sample_slab_bytes(n_fine, n_coarse, n_prev, mixed, eig32, 0, 0);
   if (std::max(slab + fslab, full) > kNoAllocScratchBytes || (!mixed && n_fine > 256)) return MQ_EINVAL;
 
   int device = 0;
@@ -138,6 +140,7 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   p.use_smem = 0;
   p.tol_eig = 1e-12;
   p.max_eig_it = 200;
+  p.eig32 = eig32;
   p.tol_lin = tol_linear > 0 ? tol_linear : 1e-10;
   p.tol_inner = mixed ? 1e-5 : 0.1 * p.tol_lin;
   p.max_outer = mixed ? 10 : 4;

@@ -93,9 +93,8 @@ struct CoarseWS32 {
   float *rx, *ry, *rd, *rxl, *ryl, *rdl;  // reaction edge weights and their low parts (NULL without a reaction term)
 };
 
-// Meshes whose coarse problem the FP32 kernel solves with lobpcg32: its residual floor, about 2^-48 4 n / theta
-// relative, stays below every eigen-residual target in use (1e-12 at the least) up to 1/128.
-constexpr int kEig32Max = 128;
+// Meshes up to which the FP32 kernel takes its own form of a solve on the coarse mesh itself (`near` below)
+constexpr int kNear32Max = 128;
 
 // xh, xl come first: they hold the coarse eigenvector through the fine solves
 __host__ __device__ void carve_coarse32(Carver& c, int nc, CoarseWS32& ws, size_t* persist = nullptr,
@@ -175,10 +174,10 @@ __host__ __device__ size_t fine_bytes(int n, bool reaction = false) {
 // exactly as sized here (an unaligned slab start would shift its arrays by up to 15 bytes into
 // the next slab).
 template <typename T>
-__host__ __device__ size_t slab_size(int nf, int nc, int np, int mode_f = 0, int mode_p = 0, bool reaction = false) {
+__host__ __device__ size_t slab_size(int nf, int nc, int np, bool eig32, int mode_f, int mode_p, bool reaction) {
   Carver c(nullptr);
   size_t persist = 0;
-  if (sizeof(T) == sizeof(float) && nc <= kEig32Max) {
+  if (sizeof(T) == sizeof(float) && eig32) {
     CoarseWS32 cw;
     carve_coarse32(c, nc, cw, &persist, reaction);
   } else {
@@ -189,7 +188,7 @@ __host__ __device__ size_t slab_size(int nf, int nc, int np, int mode_f = 0, int
   const size_t coarse = (c.used() + 15) & ~(size_t)15;
   auto need = [&](int n, int mode) -> size_t {
     // (the FP32 kernel's FP64 solve on a large coarse mesh itself has its own workspace)
-    if (mode == 2 || (sizeof(T) == sizeof(float) && n == nc && nc > kEig32Max)) return 0;
+    if (mode == 2 || (sizeof(T) == sizeof(float) && n == nc && nc > kNear32Max)) return 0;
     return fine_bytes<T>(n, reaction);
   };
   size_t m = coarse - persist;
@@ -1281,7 +1280,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
   char* base = P.use_smem ? smem_dyn : P.gscratch + (size_t)blockIdx.x * P.slab_bytes;
   size_t persist_bytes;
   const bool rxn = P.reaction != 0;
-  const bool e32 = sizeof(T) == sizeof(float) && P.nc <= kEig32Max;
+  const bool e32 = sizeof(T) == sizeof(float) && P.eig32;
   if (e32) {
     Carver c(base);
     CoarseWS32 tmp;
@@ -1314,7 +1313,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
   auto fine = [&](int n, const double* a, const double* rb, double lamH, int& it, int& outer, int& flags, double& gq) {
     int fl = 0;
     double v = 0.0;
-    const bool f64 = sizeof(T) == sizeof(float) && n == P.nc && P.nc > kEig32Max;  // beyond the FP32 form's reach
+    const bool f64 = sizeof(T) == sizeof(float) && n == P.nc && P.nc > kNear32Max;  // beyond the FP32 form's reach
     if (!f64) v = twogrid_fine<T>(fws, fine_base, n, a, rb, uH, P.nc, lamH, P, red, &msh, it, outer, fl, gq);
     if constexpr (sizeof(T) == sizeof(float)) {
       if (f64 || (n == P.nc && (fl & (kFlagLinNoConv | kFlagBreakdown)))) {
@@ -1618,13 +1617,9 @@ size_t sample_fallback_bytes(int n, int reaction) {
   return (c.used() + fine_bytes<double>(n, reaction != 0) + 255) & ~(size_t)255;
 }
 
-size_t sample_slab_bytes(int nf, int nc, int np, int mixed) {
-  return mixed ? slab_size<float>(nf, nc, np) : slab_size<double>(nf, nc, np);
-}
-
-size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int mode_f, int mode_p, int reaction) {
-  return mixed ? slab_size<float>(nf, nc, np, mode_f, mode_p, reaction != 0)
-               : slab_size<double>(nf, nc, np, mode_f, mode_p, reaction != 0);
+size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int eig32, int mode_f, int mode_p, int reaction) {
+  return mixed ? slab_size<float>(nf, nc, np, eig32 != 0, mode_f, mode_p, reaction != 0)
+               : slab_size<double>(nf, nc, np, false, mode_f, mode_p, reaction != 0);
 }
 
 namespace {
