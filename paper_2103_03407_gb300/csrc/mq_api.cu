@@ -636,7 +636,8 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   // FP64 inner solves in the per-sample kernel follow the FP64 defaults
   const int np_k = given ? 0 : g.np;  // the previous-level solve runs here only without the store
   const int in_kernel_n = std::max(p.mode_f != 2 && !g.direct_f ? g.nf : 0, p.mode_p != 2 && !g.direct_p ? np_k : 0);
-  const int threads = g.threads > 0 ? g.threads : threads_for(in_kernel_n, g.nc);
+  const int default_threads = threads_for(in_kernel_n, g.nc);
+  const int threads = g.threads > 0 ? g.threads : default_threads;
   const size_t slab = mq::sample_slab_bytes(g.nf, g.nc, np_k, mixed, p.eig32, g.direct_f ? 2 : p.mode_f, g.direct_p ? 2 : p.mode_p,
                                             p.reaction);
   const int static_smem = mq::sample_static_smem(mixed);
@@ -646,7 +647,9 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   if (use_smem) MQ_CUDA(c, mq::set_sample_smem(mixed, (int)smem));
   int occ = mq::sample_occupancy(mixed, threads, smem);
   if (occ < 1) occ = 1;
-  if (chunk <= 0) chunk = chunk_for(c, R, npts, occ);
+  // the chains are those of the default block size, so that results do not depend on the caller's
+  if (chunk <= 0)
+    chunk = chunk_for(c, R, npts, threads == default_threads ? occ : std::max(1, mq::sample_occupancy(mixed, default_threads, smem)));
   p.chunk = chunk;
   const int cpr = (npts + chunk - 1) / chunk;
   const long nchunks = (long)cpr * R;
