@@ -389,8 +389,8 @@ mq_status mq_get_kernel_timing(mq_ctx* ctx, int32_t level, double* percta_ms, do
 mq_status mq_get_launch_count(mq_ctx* ctx, uint64_t* launches);
 
 /* Single explicit parameter vector y[0..s_l-1] on level `level`: the coarse eigenvalue
- * lambda_{H_l,S_l}(y), lambda^l(y) and (l > 0) lambda^{l-1}(y) (Algorithm 1).  Any output may
- * be NULL.  u_H: NULL or host [(n_coarse-1)^2], the coarse eigenvector, ||u_H||_M = 1, sum > 0. */
+ * lambda_{H_l,S_l}(y), lambda^l(y) and (l > 0) lambda^{l-1}(y) (Algorithm 1).  |y_j| <= 1 in
+ * MQ_PREC_MIXED (see mq_coefficients_device).  Any output may be NULL.  u_H: NULL or host [(n_coarse-1)^2], the coarse eigenvector, ||u_H||_M = 1, sum > 0. */
 mq_status mq_eval_point(mq_ctx* ctx, int32_t level, const double* y, double* lam_H,
                         double* lam_h_twogrid, double* lam_hm1_twogrid, double* u_H);
 
@@ -423,7 +423,8 @@ mq_status mq_lattice_points_device(mq_ctx* ctx, int32_t level, uint32_t k0, uint
 
 /* Coefficients at the centroids of mesh 1/n (eq. coeff_s): d_a[b][2n^2] = a0 + sum_{j<s}
  * d_Y[b*ldy + j] psi_{j+1}(c_t), for b < B, with the context's precision mode
- * (FP64: FP64 GEMM; MIXED: tensor-core split GEMM accurate to FP64 rounding of the terms).
+ * (FP64: FP64 GEMM; MIXED: tensor-core split GEMM accurate to FP64 rounding of the terms, for |y| <= 1, twice the
+ * range of the parameters; larger entries lose digits).
  * Family 2: the piecewise a_0 in place of a0. */
 mq_status mq_coefficients_device(mq_ctx* ctx, int32_t n, int32_t s, const double* d_Y,
                                  int32_t B, int32_t ldy, double* d_a);

@@ -378,7 +378,7 @@ mq_status coefficients(mq_ctx* c, int n, int K, const double* d_Y, int B, int ld
   if (c->family == 2 && (st = ensure_base(c, n, which, &base)) != MQ_OK) return st;
   if (!base && which == 0 && use_separable(c, n, K)) return coefficients_separable(c, n, K, d_Y, B, ldy, d_a);
   const double a0 = base ? 0.0 : c->a0;
-  // |a| for |y| <= 2 (the zeroth terms of family 2 are at most pi / sqrt(2) times their values off and on D_f)
+  // a bound of |a| (for |y| <= 2, twice the kernels' domain; the zeroth terms of family 2 are at most pi / sqrt(2) times their values off and on D_f)
   const double z0 = base ? 2.3 * std::max(which ? kSigB[0] : kSigA[0], which ? kSigB[1] : kSigA[1]) : c->a0;
   const double amax = z0 + 2.0 * c->cabs[which];
   if (c->prec == MQ_PREC_MIXED && K > 0) {

@@ -113,8 +113,8 @@ int tc_pad_k(int k);
 // slices of 2^pexp psi (|2^pexp psi| <= 1 required)
 cudaError_t launch_psi_slices(const double* d_psi, int s_rows, int nT, void* d_out, cudaStream_t st, int pexp = 0);
 cudaError_t launch_y_slices(const double* d_Y, int B, int ldy, int k, int kpad, void* d_out, cudaStream_t st);
-// pexp: the scale exponent the psi slices were built with; amax: a bound of |a| (with room for |y| up to
-// 2, four times the lattice points' range), which sets the kernel's fixed-point unit
+// |y| <= 1 (see mq_tc.cu).  pexp: the scale exponent the psi slices were built with; amax: a bound of |a| (with room
+// to spare: for |y| <= 2), which sets the kernel's fixed-point unit
 cudaError_t launch_coef_tc(const void* d_yslices, int B, int kpad, const void* d_pslices, int nT, int kpad_psi,
                            double a0, double* d_a, int* d_err, cudaStream_t st, const double* d_base,
                            int pexp, double amax);

@@ -439,19 +439,27 @@ struct TcOut {
   int cols_fast;  // tile order: 0 row tiles fastest (tiles sharing a column tile run together), 1 columns
 };
 
-// One output's group sums in units of 2^fs, added to w modulo 2^64.  The group sums are integers below
-// 2^24, exact in FP32, |S_g| <= (g + 1) 2^21:
+// Domain: |y| <= 1 (the lattice points lie in [-1/2, 1/2)): the leading digit of y is then at most 256, the
+// largest one exact in BF16, all others at most 128, and a group sum over 16 T terms is bounded by
+//   |S_g| <= (g + 2) 16 T 2^14   (at most 2^24, exact in FP32, for the 128 terms of a chunk).
+// One output's group sums in units of 2^fs, added to w modulo 2^64:
 //   sum_g S_g 2^{8(6-g)-fs} = A 2^{40-fs} + B 2^{24-fs} + S_4 2^{16-fs} + D,
-//   A = S_0 256 + S_1, B = S_2 256 + S_3, D = S_5 2^{8-fs} + floor(S_6 2^-fs),
-// A, B and D below 2^31 (1 <= fs <= 8).
+//   A = S_0 256 + S_1, B = S_2 256 + S_3, D = S_5 2^{8-fs} + floor(S_6 2^-fs) (1 <= fs <= 8);
+// A and D stay below 2^31, B up to 80 terms (a whole chunk: 64 bits).
 __device__ __forceinline__ int group_sum(uint32_t r) { return __float2int_rn(__uint_as_float(r)); }
 // the same for |S_g| <= 2^22 without a conversion instruction (those run at an eighth of the rate): the
 // integer from the significand of 1.5 2^23 + S_g
+constexpr int small_groups(int T) {  // the groups (of the first five) that this holds for
+  int g = 0;
+  while (g < 5 && ((g + 2) * 16 * T) << 14 <= 1 << 22) ++g;
+  return g;
+}
 template <bool SMALL>
 __device__ __forceinline__ int group_sum_if(uint32_t r) {
   return SMALL ? __float_as_int(__uint_as_float(r) + 12582912.0f) - 0x4B400000 : group_sum(r);
 }
-__device__ __forceinline__ long long fold_fixed(int A, int Bv, int s4, int s5, int s6, int fs, long long w) {
+template <typename I>
+__device__ __forceinline__ long long fold_fixed(int A, I Bv, int s4, int s5, int s6, int fs, long long w) {
   long long x = (long long)s4 * (1 << (16 - fs)) + w;
   x = (long long)(s5 * (1 << (8 - fs)) + (s6 >> fs)) * 1 + x;
   x = (long long)Bv * (1 << (24 - fs)) + x;
@@ -487,8 +495,7 @@ struct ResSmem {
   volatile int err;
 };
 
-// SMALL: groups g < SMALL hold sums of at most 2^22, (g + 1) 16 T 2^14 (five groups for T <= 3, three
-// for T <= 5)
+// SMALL: groups g < SMALL hold sums of at most 2^22 (small_groups of the largest T)
 template <int SMALL>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_coef_res(const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmP, int B, int nT, int T,
@@ -812,7 +819,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc_fence_after();
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          int ga[8], gb[8];
+          int ga[8];
+          long long gb[8];
           {
             uint32_t r[4][8];
 #pragma unroll
@@ -822,7 +830,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               ga[i] = group_sum(r[0][i]) * 256 + group_sum(r[1][i]);
-              gb[i] = group_sum(r[2][i]) * 256 + group_sum(r[3][i]);
+              gb[i] = (long long)group_sum(r[2][i]) * 256 + group_sum(r[3][i]);
             }
           }
           uint32_t r[3][8];
@@ -992,12 +1000,12 @@ cudaError_t coef_tc(const void* d_yslices, int B, int kpad, const void* d_pslice
   if (resident) {
     const int nst = std::min(kResStages, (int)((kResSmem - T * kABytes) / (T * kRBytes)));
     const size_t smem = (size_t)T * kABytes + (size_t)nst * T * kRBytes + 1024;
-    const void* kern = T <= 3 ? (const void*)k_coef_res<5> : (const void*)k_coef_res<3>;
-    if ((e = raise_smem_limit(kern, kResSmem + 1024)) != cudaSuccess) return e;
-    if (T <= 3)
-      k_coef_res<5><<<grid, kTcThreads, smem, st>>>(tmY, tmP, B, nT, T, nst, ntn, (int)ntiles, a0, O, d_err, d_base, pexp, fs);
-    else
-      k_coef_res<3><<<grid, kTcThreads, smem, st>>>(tmY, tmP, B, nT, T, nst, ntn, (int)ntiles, a0, O, d_err, d_base, pexp, fs);
+    const auto kern = T <= 2   ? k_coef_res<small_groups(2)>
+                      : T == 3 ? k_coef_res<small_groups(3)>
+                      : T == 4 ? k_coef_res<small_groups(4)>
+                               : k_coef_res<small_groups(5)>;
+    if ((e = raise_smem_limit((const void*)kern, kResSmem + 1024)) != cudaSuccess) return e;
+    kern<<<grid, kTcThreads, smem, st>>>(tmY, tmP, B, nT, T, nst, ntn, (int)ntiles, a0, O, d_err, d_base, pexp, fs);
     return cudaGetLastError();
   }
   const size_t smem = sizeof(TcSmem) + 1024;
