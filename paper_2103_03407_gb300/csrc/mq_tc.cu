@@ -36,7 +36,7 @@
 // rounding the chunk exactly from 128 bits and adding a0 in FP64 took ~300 and eight warps.
 // Measured with the form for short contractions below, 64 samples on mesh 1/1024 with 1,024 terms (134 M
 // outputs, 0.16 ms to write them): 1.8 ms before, 0.5 ms now.
-// Contractions whose a0 is beyond about 2^8 times the largest term keep the 128-bit form.  Every wait is
+// Contractions whose a0 is beyond about 2^8 times the largest term, or below 2^-10 of it, keep the 128-bit form.  Every wait is
 // bounded; a timeout sets an error word, stops the issuing of new work, drains what is in flight
 // and frees the tensor memory.
 #include <cuda.h>
@@ -977,7 +977,8 @@ cudaError_t coef_tc(const void* d_yslices, int B, int kpad, const void* d_pslice
   // the fixed-point unit: the smallest fs >= 1 with |a| < 2^{fs - pexp} (see k_coef_tc)
   int fs = 1;
   while (fs <= 8 && !(std::ldexp(amax, pexp) < std::ldexp(1.0, fs))) ++fs;
-  const bool fixed = fs <= 8;
+  // a zeroth term far below the terms has to be a multiple of that unit too, as it is from 2^{fs - 11 - pexp} on
+  const bool fixed = fs <= 8 && (d_base || a0 >= std::ldexp(1.0, fs - 11 - pexp));
   const int T = kpad / kTK;
   // sample slices of a row tile kept in shared memory: up to kResSteps K steps, in fixed point (the others need
   // the larger stages, respectively the registers, of k_coef_tc).  Measured at K = 64, mesh 1/64, 2,048
