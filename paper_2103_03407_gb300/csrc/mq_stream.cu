@@ -2074,9 +2074,9 @@ __global__ void k_outer_update(int n, int B, const SS<T>* __restrict__ ss, const
 
 // FP64 residual r = b - (A - sigma M) x64 of the FP64 path (the FP32 path: k_residual4); v = T(r).
 // Partials r.r, x.x, x.Ax, x.Mx, sum x: the last pass of a sample gives its Rayleigh quotient and
-// its functional.  The two norms only steer the refinement (stopping tests, the scale of the next
-// correction, which the following pass measures again), so each thread sums them in FP32: GB300
-// issues FP64 at 1/64 of the FP32 rate.  The nodal sum is formed only for the functional (with_sum).
+// its functional.  All in FP64, the two norms that steer the refinement too: in FP32 squares of x beyond 2^64 and of r
+// below 2^-63 left its range, and with them the stopping tests.  The nodal sum is formed only for the
+// functional (with_sum).
 template <typename T>
 __global__ void k_residual(int n, int B, const int* __restrict__ ran, const double* __restrict__ wx64,
                            const double* __restrict__ wy64,
@@ -2093,22 +2093,18 @@ __global__ void k_residual(int n, int B, const int* __restrict__ ran, const doub
   const double* __restrict__ WY = wy64 + off;
   const double* __restrict__ X = x64 + off;
   double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  float rr = 0.0f, xx = 0.0f;
   for_tile(n, ch, [&](int p, int, int) {
     const double xv = X[p];
     const double ax = stiff<double, double>(WX, WY, X, p, ld);
     const double mx = hm * mass7(X, p, ld);
     const double r = b64[off + p] - (ax - sg * mx);
-    const float rf = (float)r, xf = (float)xv;
     v[off + p] = T(r);
-    rr = fmaf(rf, rf, rr);
-    xx = fmaf(xf, xf, xx);
+    acc[0] += r * r;
+    acc[1] += xv * xv;
     acc[2] += xv * ax;
     acc[3] += xv * mx;
     if (with_sum) acc[4] += xv;
   });
-  acc[0] = (double)rr;
-  acc[1] = (double)xx;
   tile_partials<5, double>(acc, part, (size_t)b * nt + ch);
 }
 
