@@ -181,9 +181,10 @@ mq_status mq_set_precision(mq_ctx* ctx, mq_precision prec, double tol_linear);
 
 /* Inner solver options (values <= 0 keep the defaults): tol_inner is the reduction of the
  * preconditioned MINRES residual per refinement step (default in MQ_PREC_MIXED: chosen for each
- * step from the residual for eigenvalues of the sine families in the streaming tier, otherwise 1e-4
- * for fine meshes up to 1/128 and 1e-5 beyond; tol_linear/10 in MQ_PREC_FP64), max_inner the MINRES iteration cap per step (500), max_outer the cap on FP64
- * refinement steps (10 mixed, 4 FP64). */
+ * step from the residual for eigenvalues of the sine families in the streaming tier with max_outer of
+ * at least 10, otherwise 1e-4 for fine meshes up to 1/128 and 1e-5 beyond; tol_linear/10 in MQ_PREC_FP64),
+ * max_inner the MINRES iteration cap per step (500), max_outer the cap on refinement steps (10
+ * mixed, 4 FP64). */
 mq_status mq_set_solver_options(mq_ctx* ctx, double tol_inner, int32_t max_inner, int32_t max_outer);
 
 /* Coarse eigensolver options (values <= 0 keep the defaults): tol_eig is the target of the
