@@ -778,7 +778,13 @@ __device__ __noinline__ int lobpcg32(CoarseWS32& ws, int n, double tol, int maxi
   return conv ? it : -1;
 }
 
-constexpr int kNearInner = 24;  // MINRES iterations per correction of a solve on the coarse mesh itself
+// MINRES iterations per correction of a solve on the coarse mesh itself.  Ten to thirteen reduce a residual by the 1e-4 asked for;
+// where the shift nearly meets the eigenvalue they leave what r has along the near-null direction, and iterations
+// beyond run into FP32's idea of that eigenvalue: the correction grows without bound (450 ||u_H||, residual 1e2
+// to 1e4 ||b||).  With 24 one sample in 150 needed the FP64 solve behind it, and calls of few samples waited
+// for it: 128 solves on mesh 1/64 7.2 ms, on 1/128 31.7 ms.  With 12 none of 5,000 did: 2.5 and 12.7 ms (FP64 throughout: 4.6 and
+// 20.0); 8,192 samples of the first test problem's level 1 7.85 -> 6.83 ms; with 10, 14, 16 and 18: 6.81, 6.94, 7.32, 7.78.
+constexpr int kNearInner = 12;
 
 // The coarse eigenvector as the fine solves read it: FP64 values, or double-float pairs.
 struct CoarseVec {
