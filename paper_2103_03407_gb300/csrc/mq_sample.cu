@@ -808,6 +808,16 @@ __device__ __noinline__ void operator32_scaled(WS& ws, int n, const double* a, c
   operator32(ws, n, a, rb, k);
 }
 
+// the operator of the FP64 eigensolver: FP32 hierarchy, FP64 weights
+__device__ __forceinline__ void operator64(CoarseWS& ws, int n, const double* a, const double* rb, int k) {
+  build_mg<float>(ws.mg, a, n, rb, nullptr, nullptr, k);
+  weights_from_cells<double, double>(n, a, a + (size_t)n * n, ws.wx, ws.wy, nullptr, nullptr, k);
+  if (rb) reaction_weights<double, double>(n, rb, rb + (size_t)n * n, ws.rx, ws.ry, ws.rd, nullptr, nullptr, nullptr, k);
+}
+__device__ __noinline__ void operator64_scaled(CoarseWS& ws, int n, const double* a, const double* rb, int k) {
+  operator64(ws, n, a, rb, k);
+}
+
 // MINRES scalars, owned by thread 0 and read by all threads after each reduction.  The
 // recurrences run in the inner precision T (FP32 on the mixed path), the refinement norms in FP64.
 template <typename T>
@@ -1431,12 +1441,10 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
         const double* bc = rxn ? P.b_c + b * ncT : nullptr;
         CellCheck cells;
         cells.look(nc, ac, bc);
+        operator64(cw, nc, ac, bc, 0);
         if (!cells.finish(red)) flags |= kFlagBadCoef;
         const int ks = scale_of_cells(cells.amax, cells.bmax);  // (its V-cycles and Gram matrices are FP32)
-        build_mg<float>(cw.mg, ac, nc, bc, nullptr, nullptr, ks);
-        weights_from_cells<double, double>(nc, ac, ac + (size_t)nc * nc, cw.wx, cw.wy, nullptr, nullptr, ks);
-        if (rxn)
-          reaction_weights<double, double>(nc, bc, bc + (size_t)nc * nc, cw.rx, cw.ry, cw.rd, nullptr, nullptr, nullptr, ks);
+        if (ks != 0) operator64_scaled(cw, nc, ac, bc, ks);
         if (cold) {
           const float inc = 1.0f / (float)nc;
           for_interior(nc, [&](int p, int i, int j) { cw.x[p] = (double)(sinpif(i * inc) * sinpif(j * inc)); });
