@@ -164,9 +164,10 @@ size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int eig32, int mode_
 // that nothing bounds, take the FP64 eigensolver.
 constexpr int kEig32Max = 128;
 inline bool eig32_reaches(int nc, double tol) { return nc <= kEig32Max && tol >= 2e-15 * nc * nc; }
+// wide: the FP32 kernel without its bound on registers
 cudaError_t launch_sample(const SampleLaunch& p, int mixed, int blocks, int threads, size_t smem,
-                          cudaStream_t st);
-int sample_occupancy(int mixed, int threads, size_t smem);
+                          cudaStream_t st, int wide = 0);
+int sample_occupancy(int mixed, int threads, size_t smem, int wide = 0);
 int sample_static_smem(int mixed);
 cudaError_t set_sample_smem(int mixed, int bytes);
 // Raises a kernel's dynamic shared memory limit to at least `bytes` on the current device and

@@ -111,7 +111,11 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return MQ_ECUDA;
 
   const int threads = n_fine <= 16 ? 128 : 256;
-  int occ = mq::sample_occupancy(mixed, threads, 0);
+  // the kernel without the bound of three blocks per SM: its FP64 eigensolver and global workspaces wait on memory, and
+  // registers spilled for the bound cost more than the third block hides (mixed, mesh 1/32 over 1/16, 2,048 samples 7.5 against
+  // 6.7 ms, 1/64 over 1/32, 512 samples 15.7 against 13.9)
+  constexpr int wide = 1;
+  int occ = mq::sample_occupancy(mixed, threads, 0, wide);
   if (occ < 1) occ = 1;
   const long fit = (long)(kNoAllocScratchBytes / (slab + fslab));
   const long blocks = std::max(1L, std::min<long>({(long)B, (long)sms * occ, fit}));
@@ -147,6 +151,6 @@ extern "C" mq_status mq_twogrid_samples_noalloc(int32_t n_fine, int32_t n_coarse
   p.max_inner_it = 500;
   p.nu = 2;
   p.omega = 0.8;
-  const cudaError_t e = mq::launch_sample(p, mixed, (int)blocks, threads, 0, (cudaStream_t)cuda_stream);
+  const cudaError_t e = mq::launch_sample(p, mixed, (int)blocks, threads, 0, (cudaStream_t)cuda_stream, wide);
   return e == cudaSuccess ? MQ_OK : MQ_ECUDA;
 }

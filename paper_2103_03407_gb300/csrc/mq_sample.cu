@@ -1638,20 +1638,20 @@ size_t sample_slab_bytes(int nf, int nc, int np, int mixed, int eig32, int mode_
 
 namespace {
 using SampleFn = void (*)(SampleLaunch);
-SampleFn sample_fn(int mixed, int threads) {
-  return mixed ? (threads <= 256 ? sample_kernel<float, 256> : sample_kernel<float, 512>) : sample_kernel<double, 512>;
+SampleFn sample_fn(int mixed, int threads, int wide) {
+  return mixed ? (threads <= 256 && !wide ? sample_kernel<float, 256> : sample_kernel<float, 512>) : sample_kernel<double, 512>;
 }
 }  // namespace
 
-int sample_occupancy(int mixed, int threads, size_t smem) {
+int sample_occupancy(int mixed, int threads, size_t smem, int wide) {
   int nb = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sample_fn(mixed, threads), threads, smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sample_fn(mixed, threads, wide), threads, smem);
   return e == cudaSuccess ? nb : 0;
 }
 
 int sample_static_smem(int mixed) {
   cudaFuncAttributes fa;
-  const cudaError_t e = cudaFuncGetAttributes(&fa, sample_fn(mixed, 512));
+  const cudaError_t e = cudaFuncGetAttributes(&fa, sample_fn(mixed, 512, 1));
   return e == cudaSuccess ? (int)fa.sharedSizeBytes : 8192;
 }
 
@@ -1670,8 +1670,8 @@ cudaError_t raise_smem_limit(const void* func, int bytes) {
 }
 
 cudaError_t set_sample_smem(int mixed, int bytes) {
-  const cudaError_t e = raise_smem_limit((const void*)sample_fn(mixed, 256), bytes);
-  return e == cudaSuccess ? raise_smem_limit((const void*)sample_fn(mixed, 512), bytes) : e;
+  const cudaError_t e = raise_smem_limit((const void*)sample_fn(mixed, 256, 0), bytes);
+  return e == cudaSuccess ? raise_smem_limit((const void*)sample_fn(mixed, 512, 1), bytes) : e;
 }
 
 cudaError_t launch_apply_operator(int n, int B, const double* d_a, int which, double sigma, const double* d_x,
@@ -1688,8 +1688,9 @@ cudaError_t launch_shift_sums(const double* d_out, const int* d_stat, int R, int
   return cudaGetLastError();
 }
 
-cudaError_t launch_sample(const SampleLaunch& p, int mixed, int blocks, int threads, size_t smem, cudaStream_t st) {
-  sample_fn(mixed, threads)<<<blocks, threads, smem, st>>>(p);
+cudaError_t launch_sample(const SampleLaunch& p, int mixed, int blocks, int threads, size_t smem, cudaStream_t st,
+                          int wide) {
+  sample_fn(mixed, threads, wide)<<<blocks, threads, smem, st>>>(p);
   return cudaGetLastError();
 }
 
