@@ -493,8 +493,8 @@ def stream_bytes(wl, level, st, prec, samples):
 # ncu DRAM traffic of the per-sample kernel's launch on a level (one launch of the benchmark's size:
 # level 1 of the six-level workload, 4,096 samples; summarised under profiles/), valid only for the
 # kernel source it was measured on
-SAMPLE_KERNEL_TRAFFIC = {"source_sha256": "4e49346cf2040e4ba93d6889a0bf4b5ebe68fc90eb32010d7a5f9c282243139a",
-                         "level": 1, "precision": "mixed", "bytes_per_launch": 141.633792e6 + 96.069888e6}
+SAMPLE_KERNEL_TRAFFIC = {"source_sha256": "9527b13be56fc0c2d0d8374f0095f2358898dbb7e2ea1a5129372541d8db9107",
+                         "level": 1, "precision": "mixed", "bytes_per_launch": 142.348288e6 + 96.288768e6}
 
 
 # ncu DRAM traffic of the operator sweep k_minres_q per algorithmic byte: one launch (4 arrays per node) on mesh

@@ -61,9 +61,16 @@ typedef enum {
 } mq_qoi;
 
 typedef enum {
-  MQ_PREC_FP64 = 0,  /* every step in FP64 */
-  MQ_PREC_MIXED = 1  /* FP32 multigrid-preconditioned MINRES inside FP64 iterative refinement;
-                        coefficients, residuals, Rayleigh quotients, coarse eigenpairs in FP64 */
+  MQ_PREC_FP64 = 0,  /* every step in FP64 (V-cycles and Rayleigh-Ritz steps of the coarse eigensolver, which only
+                        steer it, in FP32) */
+  MQ_PREC_MIXED = 1  /* coefficients exact to FP64 rounding; FP32 multigrid-preconditioned MINRES inside
+                        iterative refinement.  What the refinement keeps (edge weights, right-hand side,
+                        solution, residual, the sums of Rayleigh quotients and functionals) and, for
+                        eigen-residual targets of 2e-15 n^2 and more on coarse meshes up to 1/128, the coarse
+                        eigenvector and its residual are pairs of FP32, 48 bits; the search directions of
+                        that eigensolver are FP32.  Other coarse eigenpairs in FP64 as above.  Eigenvalues
+                        differ from those of MQ_PREC_FP64 by a few 1e-15 relative from rounding, beside
+                        the solver targets */
 } mq_precision;
 
 /* One MLQMC level (Algorithm 2).  n_fine = 1/h_l and n_coarse = 1/H_l are powers of two with
@@ -176,7 +183,7 @@ mq_status mq_set_reuse(mq_ctx* ctx, int32_t on);
  * Rayleigh quotient lambda^h moves to first order in the solve error with a constant damped by
  * the two-grid error (about 3e-7 on meshes 1/16..1/128), so the defaults keep lambda^h within
  * ~3e-13 of the exact two-grid value.  Samples whose final residual is above max(1e-5,
- * 10 tol_linear) (or a small multiple of the FP64 rounding floor) are flagged. */
+ * 10 tol_linear) (or a small multiple of the rounding floor) are flagged. */
 mq_status mq_set_precision(mq_ctx* ctx, mq_precision prec, double tol_linear);
 
 /* Inner solver options (values <= 0 keep the defaults): tol_inner is the reduction of the
@@ -192,6 +199,7 @@ mq_status mq_set_solver_options(mq_ctx* ctx, double tol_inner, int32_t max_inner
  * iteration cap (200).  The Rayleigh quotient theta = lambda_H is accurate to about the square of
  * tol_eig, the eigenvector (and so G(u_H)) to about tol_eig: the relative eigenvalue error is at
  * most tol_eig^2 kappa(M) theta / (lambda_2 - theta), kappa(M) <= 4 for the P1 mass matrix.
+ * In MQ_PREC_MIXED targets below 2e-15 n_coarse^2, and coarse meshes beyond 1/128, take the FP64 eigensolver.
  * Defaults: 1e-6 for level evaluations of eigenvalues with coefficient families 0 and 1
  * (lambda_H within ~3e-12 relative at worst, 5e-14 measured on the six-level workload; the
  * two-grid values depend on u_H only through one shifted inverse-iteration step and stay at FP64
@@ -209,7 +217,7 @@ mq_status mq_set_smoothing(mq_ctx* ctx, int32_t nu);
 /* Execution tier of the fine solves: fine meshes 1/n with n >= stream_min_n run in
  * the batched streaming tier (one kernel per sweep over all samples of a pass, lockstep across
  * samples); coarser ones run inside the per-sample kernel (one CTA per sample, workspace in
- * shared memory when it fits).  Both tiers compute the same values to rounding.  Default (or
+ * shared memory when it fits).  Both tiers compute the same values to the solver tolerances.  Default (or
  * stream_min_n = 0): 32 in MQ_PREC_MIXED; in MQ_PREC_FP64 128, or 32 in calls of at least 2^21 fine nodes. */
 mq_status mq_set_tier(mq_ctx* ctx, int32_t stream_min_n);
 
@@ -253,7 +261,10 @@ mq_status mq_autotune_level(mq_ctx* ctx, int32_t level, uint32_t points, const c
  *               lambda^{-1} = 0 on level 0.
  *   shift_sums: NULL or host [R]; sum over k of the differences is ADDED to each entry.
  * The context also accumulates the sums for mq_estimate.  Returns MQ_ENOCONV (results written)
- * when any sample hit an iteration cap. */
+ * when any sample hit an iteration cap.
+ * A sample's last bits may depend on how many samples share the call (or a pass of it, which the free memory
+ * limits): the warm-start chains (solver tolerances), the sums of the streaming tier in launches of 2^24
+ * nodes and more (rounding) and the default tier of MQ_PREC_FP64 (solver tolerances) follow their number. */
 mq_status mq_eval_level(mq_ctx* ctx, int32_t level, uint32_t k0, uint32_t k1, double* per_sample,
                         double* shift_sums);
 
@@ -287,7 +298,7 @@ mq_status mq_eval_levels_device(mq_ctx* ctx, int32_t nlevels, const int32_t* lev
  * conditional WHILE nodes whose conditions the kernels set on the device (no host reads), and the
  * per-shift sums and sample flags accumulate on the device.  mq_graph_launch replays the graph
  * with one cudaGraphLaunch, waits for it and adds its sums to the context (mq_estimate), as the
- * level-by-level calls would; the per-sample results equal theirs bit for bit.  k0s: NULL to
+ * level-by-level calls would; the per-sample results equal those of calls of the same ranges bit for bit.  k0s: NULL to
  * replay the captured ranges, or new start points for ranges of the captured lengths (the offset
  * reaches the kernels through device memory).  The per-level timers are not updated by the graph.
  * Any setter, and any call that has to enlarge a buffer the graph uses, drops the graph
@@ -438,7 +449,7 @@ mq_status mq_reaction_coefficients_device(mq_ctx* ctx, int32_t n, int32_t s, con
 /* Operator apply on mesh 1/n for B coefficient fields d_a[b][2n^2] (FP64):
  * which = 0: y = A x, 1: y = M x, 2: y = (A - sigma M) x; with d_a holding reaction coefficients b,
  * which = 3: y = B x, the reaction matrix in the edge-weight form the inner solves use, and 4: the
- * same from the centroid values (the form of the FP64 residual).  d_x, d_y: [B][(n-1)^2]. */
+ * same from the centroid values.  d_x, d_y: [B][(n-1)^2]. */
 mq_status mq_apply_operator_device(mq_ctx* ctx, int32_t n, int32_t B, const double* d_a,
                                    int32_t which, double sigma, const double* d_x, double* d_y);
 
@@ -471,7 +482,8 @@ mq_status mq_apply_operator_device(mq_ctx* ctx, int32_t n, int32_t B, const doub
  * tol_linear / 10 (FP64), at most 500 inner iterations and 10 (mixed) or 4 (FP64) refinement
  * steps, V(2,2) damped Jacobi (omega 0.8).  A solve on the coarse mesh itself (n_fine or n_prev
  * equal to n_coarse) is nearly singular: in mixed precision it is solved for the change of the
- * eigenvector, and again in FP64 where that does not converge.  These
+ * eigenvector, and again in FP64 where that does not converge.  Coarse eigensolves are in FP64 in either
+ * precision (nothing bounds the contrast of the coefficients).  These
  * targets are tighter than mq_eval_level's defaults, so on larger coarse meshes a sample can hit
  * the eigensolver cap (flag 1) where mq_eval_level converges.
  *

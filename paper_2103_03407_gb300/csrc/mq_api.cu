@@ -595,7 +595,7 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
   // Rayleigh quotient lambda^h of the shifted-solve iterate is stationary only at an eigenvector;
   // the two-grid iterate is an O(H^4) perturbation of one, so lambda^h moves to first order in the
   // solve error with a small constant: on the 4-level workload (meshes 1/16..1/128) the largest
-  // relative change of lambda^h is about 3e-7 times the relative residual.  An FP64 residual of
+  // relative change of lambda^h is about 3e-7 times the relative residual.  A residual of
   // 1e-6 keeps lambda^h within ~3e-13 of the exact two-grid value.  The mixed path refines
   // twice whatever the targets (the FP32 rounding of the first correction, which is
   // amplified by the near-singular shift, leaves a residual of ~1e-4): inner reductions of 1e-4
@@ -633,7 +633,6 @@ mq_status run_samples(mq_ctx* c, const LevelGeom& g, int R, int npts, int chunk,
     if ((st = grow(c, c->upad, B * Vc * sizeof(double))) != MQ_OK) return st;
     if (!given) p.u_pad = (double*)c->upad.p;
   }
-  // FP64 inner solves in the per-sample kernel follow the FP64 defaults
   const int np_k = given ? 0 : g.np;  // the previous-level solve runs here only without the store
   const int in_kernel_n = std::max(p.mode_f != 2 && !g.direct_f ? g.nf : 0, p.mode_p != 2 && !g.direct_p ? np_k : 0);
   const int default_threads = threads_for(in_kernel_n, g.nc);

@@ -244,21 +244,6 @@ __device__ __forceinline__ T mass7(const T* x, int p, int ld) {
   return T(6) * x[p] + (x[p + 1] + x[p - 1]) + (x[p + ld] + x[p - ld]) + (x[p + ld + 1] + x[p - ld - 1]);
 }
 
-// FP64 stiffness at interior node (i, j) of mesh n with the edge weights formed from the
-// centroid coefficients a (lower triangles first, then upper).
-__device__ __forceinline__ double stiff_cells(const double* __restrict__ a, int n, const double* x, int p, int ld,
-                                              int i, int j) {
-  const double* lo = a;
-  const double* up = a + (size_t)n * n;
-  const int c = j * n + i;
-  const double lij = lo[c], li1j = lo[c - 1], li1j1 = lo[c - n - 1];
-  const double uij = up[c], uij1 = up[c - n], ui1j1 = up[c - n - 1];
-  const double we = 0.5 * (lij + uij1), ww = 0.5 * (li1j + ui1j1);
-  const double wn = 0.5 * (uij + li1j), ws = 0.5 * (uij1 + li1j1);
-  const double xp = x[p];
-  return we * (xp - x[p + 1]) + ww * (xp - x[p - 1]) + wn * (xp - x[p + ld]) + ws * (xp - x[p - ld]);
-}
-
 // reaction seven-point sum without the h^2/12 factor, from the edge weights rx (edge to E), ry (to
 // N) and rd (to NE) of the padded nodes
 template <typename T, typename X>

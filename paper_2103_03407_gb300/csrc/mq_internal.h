@@ -32,7 +32,7 @@ struct SampleLaunch {
   double tol_eig;
   int max_eig_it;
   int eig32;               // FP32 kernel: coarse eigensolves by lobpcg32 (see eig32_reaches)
-  double tol_lin;          // relative FP64 residual target of the shifted solve
+  double tol_lin;          // relative residual target of the shifted solve
   double tol_inner;        // relative reduction of the preconditioned residual per inner solve
   int max_inner_it;
   int max_outer;

@@ -8,7 +8,8 @@
 //   2. for the fine mesh of the level (and, on l > 0, the fine mesh of level l-1, from the same
 //      coarse pair -- Algorithm 2), forms b = M_h P u_H (P: P1 interpolation), solves
 //      (A_h - lambda_H M_h) w = b (eq. 2grid_source) by MINRES preconditioned with a symmetric
-//      multigrid V-cycle on A_h, inside FP64 iterative refinement, and returns the Rayleigh
+//      multigrid V-cycle on A_h, inside iterative refinement (solution, right-hand side and residual in
+//      FP64, in the FP32 kernel as double-floats: pairs of FP32, 48 bits), and returns the Rayleigh
 //      quotient w^T A_h w / w^T M_h w (Algorithm 1 steps 3-4, eq. RQ_update);
 //   3. writes lambda_H, lambda^l, lambda^{l-1} and the difference (or, for the functional
 //      quantity of interest, lambda_H and G of the two eigenfunction approximations and their
@@ -819,7 +820,7 @@ __device__ __noinline__ void operator64_scaled(CoarseWS& ws, int n, const double
 }
 
 // MINRES scalars, owned by thread 0 and read by all threads after each reduction.  The
-// recurrences run in the inner precision T (FP32 on the mixed path), the refinement norms in FP64.
+// recurrences run in the inner precision T (FP32 on the mixed path); the refinement's scalars are FP64.
 template <typename T>
 struct MinresShared {
   T gam, gam_old, eta, eta0, c, c_old, s, s_old;
@@ -829,8 +830,8 @@ struct MinresShared {
   T delta;
   T rs;           // 1 / ||r|| of the refinement residual
   double rnorm, bnorm;
-  double knorm, xnorm;  // ||A - sigma M|| bound and ||x|| for the FP64 residual floor
-  double xax, xmx;      // x.Ax and x.Mx of the last FP64 residual pass (the Rayleigh quotient)
+  double knorm, xnorm;  // ||A - sigma M|| bound and ||x|| for the residual's rounding floor
+  double xax, xmx;      // x.Ax and x.Mx of the last residual pass (the Rayleigh quotient)
   double xsum;          // sum of the nodal values of x in that pass (h^2 xsum = integral of x)
   double scale;         // 2^ks: the solve is the problem times 2^-ks
   double tau;           // factor of the right-hand side (1 except in a solve on the coarse mesh itself)
@@ -838,7 +839,8 @@ struct MinresShared {
 };
 
 // Residual target of the refinement: tol relative to ||b||, but never below a small multiple of
-// the FP64 rounding floor eps (||K|| ||x|| + ||b||) of the residual itself (on fine meshes the
+// the rounding floor eps (||K|| ||x|| + ||b||) of an FP64 residual (double-floats stop short of it by the lack of
+// progress; on fine meshes the
 // near-singular shifted system puts that floor above 1e-7 ||b||).
 __host__ __device__ inline double residual_target(double tol, double bnorm, double knorm, double xnorm, double f) {
   const double floor_ = f * 2.220446049250313e-16 * (knorm * xnorm + bnorm);
@@ -1267,10 +1269,10 @@ __device__ __noinline__ double twogrid_fine(FineWS<T>& ws, char* fine_base, int 
       break;
     }
   }
-  // flagged only well above the target (or the FP64 floor): the refinement may stop a little short
+  // flagged only well above the target (or the rounding floor): the refinement may stop a little short
   if (!(ms->rnorm <= residual_target(fmax(1e-5, 10.0 * P.tol_lin), fabs(ms->tau) * ms->bnorm, ms->knorm, ms->xnorm, 256.0)))
     flags |= kFlagLinNoConv;
-  // Rayleigh quotient and functional in FP64, from the residual pass over the final iterate
+  // Rayleigh quotient and functional from the sums of the residual pass over the final iterate (FP64, or 48 bits)
   gq = fabs(ms->xsum) / ((double)n * n * sqrt(ms->xmx));
   return ms->scale * (ms->xax / ms->xmx);
 }
@@ -1506,7 +1508,7 @@ __global__ void __launch_bounds__(MAXT, sizeof(T) == sizeof(float) && MAXT == 25
 // Operator application for parity checks of the stencils: one CTA per coefficient field; the
 // scratch holds four padded grids per field.  Uses the same weight builders and stencils as the
 // solver.  which: 0 stiffness, 1 mass, 2 stiffness - sigma mass; 3 the reaction matrix of the
-// field (edge-weight form), 4 the same from the centroid values (the FP64 residual's form).
+// field (edge-weight form), 4 the same from the centroid values.
 __global__ void apply_kernel(int n, const double* __restrict__ a, int which, double sigma,
                              const double* __restrict__ x, double* __restrict__ y, double* scratch) {
   const size_t V = gsz(n);

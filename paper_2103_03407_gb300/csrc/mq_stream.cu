@@ -109,7 +109,7 @@ struct SS {  // per-sample solver scalars
   int ks;
   double rnorm, bnorm, lam_h;
   double xnorm;   // ||x64||
-  double xax, xmx;  // x.Ax and x.Mx of the last FP64 residual pass (the Rayleigh quotient)
+  double xax, xmx;  // x.Ax and x.Mx of the last residual pass (the Rayleigh quotient)
   double xsum;      // sum of the nodal values of x64 in that pass (h^2 xsum = integral of x)
   float amax;     // largest centroid coefficient (for the bound ||A - sigma M|| <= 8 amax + sigma h^2)
   float bmax;     // largest reaction coefficient (the bound gains bmax h^2)
@@ -365,7 +365,7 @@ template <typename T>
 __device__ __forceinline__ void outer_step_done(SS<T>& S, double rnew, double xn) {
   S.xnorm = xn;
   // No progress: stop refining.  Not on the first step: on fine meshes the FP32 rounding of the
-  // first inner solution alone leaves an FP64 residual above ||b|| (the operator amplifies its
+  // first inner solution alone leaves a residual above ||b|| (the operator amplifies its
   // high-frequency part by O(h^-2)); the next step removes it.  A sample whose shift nearly meets the
   // eigenvalue needs more of each solve than the reductions chosen from the residual ask for: it first goes on with fixed ones
   // and three more such steps, since the near-null part that a step adds to x brings rounding of its own.
@@ -2211,7 +2211,7 @@ __global__ void k_set_int(int B, int* p, int v) {
 int launch_minres_q4(int n, int B, const int* act, const SS<float>* ss, const float* wx, const float* wy, ZSlot zs,
                      float* q, double* part, unsigned long long* work, cudaStream_t st, const float* rx, const float* ry,
                      const float* rd) {
-  if (!rx && (long)B * n * n >= 1L << 24) {
+  if (!rx && up_by_rows(n, B)) {
     k_minres_q_rows<<<B * tiles_qrows(n), kThreads, 0, st>>>(n, B, act, ss, wx, wy, zs, q, part, work);
     return tiles_qrows(n);
   }
@@ -2371,12 +2371,8 @@ cudaError_t vcycle_stream(Arena<T>& A, const T* b0, T* x0, const int* act, T om,
           continue;
         }
       }
-      if (A.hx[l])
-        ++tl_launches, k_restrict1<T, __nv_bfloat16><<<B * tiles_interior(nl / 2), kThreads, 0, st>>>(
-            nl, B, act, A.hx[l], A.hy[l], A.hd[l], b, bc, ldo);
-      else
-        ++tl_launches, k_restrict1<T><<<B * tiles_interior(nl / 2), kThreads, 0, st>>>(nl, B, act, A.wx[l], A.wy[l],
-                                                                                     A.dinv[l], b, bc, ldo);
+      ++tl_launches, k_restrict1<T><<<B * tiles_interior(nl / 2), kThreads, 0, st>>>(nl, B, act, A.wx[l], A.wy[l],
+                                                                                   A.dinv[l], b, bc, ldo);
       LAUNCH_CHECK();
     }
     const int ns = n >> A.Ls;
